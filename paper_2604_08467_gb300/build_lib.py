@@ -22,7 +22,7 @@ HOST_FLAGS = ["-O2", "-fPIC", "-std=c++17", "-ffp-contract=off", "-Wall", "-Wno-
 CU_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler",
             "-fPIC,-ffp-contract=off", "-I" + INCLUDE] + ARCH
 
-CPP_SOURCES = ["planner.cpp"]
+CPP_SOURCES = ["planner.cpp", "small_runs.cpp"]
 CU_SOURCES = ["runtime.cu", "kernels_contract.cu", "kernels_sample.cu", "kernels_gemm.cu", "stats.cu", "noalloc.cu",
               "kernels_expval.cu", "kernels_merge.cu", "kernels_harvest.cu", "tune.cu",
               "kernels_cache.cu"]

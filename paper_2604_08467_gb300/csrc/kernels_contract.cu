@@ -402,65 +402,109 @@ __global__ void k_finalize_sum(const double* __restrict__ part, int64_t tiles, i
 
 // A run of consecutive small trajectory-class steps (the gate-level start of a
 // block's path: outputs of at most 2^kSmallOutBits elements from operands of
-// at most 2^kSmallOpBits) in one launch: one CTA per trajectory of the chunk
-// walks the run in order, each step's descriptor staged in shared memory and
-// its outputs written to the arena, with a CTA barrier between steps (the
-// next step reads them back from L1/L2).  A CTA touches only its own
-// trajectory's instances, and the planner admits a step into a run only if no
-// other CTA's instances can share its output's addresses (small_step,
-// fuse_prev), so the CTA barrier is the only ordering the run needs.  Every
-// output is the same complex multiply-add chain over the summed bits as in
-// k_contract_direct.
-constexpr int kSmallThreads = 128;
+// at most 2^kSmallOpBits) in one launch, one CTA per trajectory.  The run is
+// bound by latency, not by its arithmetic (0.2-0.5 M multiply-adds per
+// trajectory), so it is walked level by level of its dataflow
+// (small_runs.cpp) with one barrier per level instead of step by step: 19
+// barriers for the 731 steps of the first 30-qubit block.  The operand and
+// output addresses of all its steps are resolved into shared memory first
+// (one dependent chain of table reads for the whole run), and a thread takes
+// output elements of any step of the level, whose operand offsets were laid
+// out by the host.  A CTA touches only its own trajectory's instances, and the
+// planner admits a step into a run only if no other CTA's instances can share
+// its output's addresses (small_step, fuse_prev).  Every output is the same
+// complex multiply-add chain over the summed bits as in k_contract_direct.
+// Measured against the walk with two barriers and a 2.7 KB descriptor per
+// step: 689 steps of the last 30-qubit block, 131 trajectories 1.67 -> 0.09 ms;
+// 731 steps of the first, 4096 trajectories 8.2 -> 2.6 ms.
+struct SmallArgs {
+    const SmallStep* steps;
+    const SmallEnt* ent;
+    const int32_t* lvl;
+    const uint32_t* ktab;
+    int32_t n_steps, n_lvl;
+};
+struct SmallRes {
+    const float2 *A, *B;
+    float2* out;
+    uint32_t loop;
+    int32_t ktab;
+};
 
-__global__ void __launch_bounds__(kSmallThreads) k_small_steps(const StepDesc* __restrict__ steps, int n_steps,
-                                                               const __grid_constant__ ChunkCtx c) {
-    __shared__ __align__(16) StepDesc s;
-    const int64_t inst = blockIdx.x;
-    for (int k = 0; k < n_steps; k++) {
-        {
-            const int4* src = reinterpret_cast<const int4*>(steps + k);
-            int4* dst = reinterpret_cast<int4*>(&s);
-            for (int i = threadIdx.x; i < (int)(sizeof(StepDesc) / sizeof(int4)); i += blockDim.x) dst[i] = src[i];
+__device__ __forceinline__ const float2* small_operand(const SmallOp& d, int64_t tl, const ChunkCtx& c) {
+    if (d.src < 0) {
+        int64_t var = 0;
+        if (d.col >= 0) var = c.var_ids[(int64_t)c.chunk_traj[tl] * c.n_var_cols + d.col];
+        return c.vtab + d.base + var * d.size;
+    }
+    int64_t oi = 0;
+    if (d.inst == CLS_TRAJ)
+        oi = (d.cache > 0 && c.cache_rep) ? (int64_t)c.cache_rep[(int64_t)(d.cache - 1) * c.cache_n + tl] : tl;
+    return c.arena[d.src] + d.base * c.arena_inst[d.src] + oi * d.size;
+}
+
+__device__ __forceinline__ void small_term(float2& acc, const float2 x, const float2 y, float sa, float sb) {
+    const float xi = sa * x.y, yi = sb * y.y;
+    acc.x = fmaf(x.x, y.x, acc.x);
+    acc.x = fmaf(-xi, yi, acc.x);
+    acc.y = fmaf(x.x, yi, acc.y);
+    acc.y = fmaf(xi, y.x, acc.y);
+}
+
+__global__ void __launch_bounds__(1024) k_small_steps(const SmallArgs a, const __grid_constant__ ChunkCtx c) {
+    extern __shared__ __align__(16) uint8_t small_smem[];
+    SmallRes* res = reinterpret_cast<SmallRes*>(small_smem);
+    const int64_t tl = blockIdx.x;
+    for (int t = threadIdx.x; t < 2 * a.n_steps; t += blockDim.x) {
+        const SmallStep& s = a.steps[t >> 1];
+        const float2* p = small_operand(s.op[t & 1], tl, c);
+        SmallRes& r = res[t >> 1];
+        if (t & 1) {
+            r.B = p;
+            r.loop = s.loop;
+            r.ktab = s.ktab;
+        } else {
+            r.A = p;
+            r.out = c.arena[s.out_arena] + s.out_off * c.arena_inst[s.out_arena] + tl * s.out_size;
         }
-        __syncthreads();   // descriptor staged; the previous step's outputs are visible
-        const float2* A = operand_ptr(s.op[0], CLS_TRAJ, inst, c);
-        const float2* B = operand_ptr(s.op[1], CLS_TRAJ, inst, c);
-        float2* out = c.arena[s.out_arena] + s.out_off * c.arena_inst[s.out_arena] + inst * s.out_size;
-        const float sa = s.op[0].conj ? -1.f : 1.f, sb = s.op[1].conj ? -1.f : 1.f;
-        const int nk = 1 << s.n_sum;
-        for (int64_t o = threadIdx.x; o < s.out_size; o += blockDim.x) {
-            int64_t oa = 0, ob = 0;
-            for (int p = 0; p < s.n_out; p++)
-                if ((o >> p) & 1) {
-                    oa += s.out_stride[0][p];
-                    ob += s.out_stride[1][p];
-                }
+    }
+    int e1 = a.lvl[0];
+    int i = e1 + (int)threadIdx.x;
+    for (int l = 0; l < a.n_lvl; l++) {
+        e1 = a.lvl[l + 1];
+        SmallEnt e = i < e1 ? a.ent[i] : SmallEnt{0, 0, 0};
+        __syncthreads();   // addresses resolved; the previous level's outputs are visible
+        while (i < e1) {
+            const int nx = i + (int)blockDim.x;
+            const SmallEnt en = nx < e1 ? a.ent[nx] : SmallEnt{0, 0, 0};
+            const SmallRes r = res[e.step];
+            const float2 *A = r.A + (e.offs & 0xffffu), *B = r.B + (e.offs >> 16);
+            const float sa = (r.loop & kSmallConjA) ? -1.f : 1.f, sb = (r.loop & kSmallConjB) ? -1.f : 1.f;
+            const int nk = (int)(r.loop & 0xffffu);
             float2 acc = make_float2(0.f, 0.f);
-            for (int kk = 0; kk < nk; kk++) {
-                int64_t ka = oa, kb = ob;
-                for (int q = 0; q < s.n_sum; q++)
-                    if ((kk >> q) & 1) {
-                        ka += s.sum_stride[0][q];
-                        kb += s.sum_stride[1][q];
-                    }
-                const float2 x = A[ka], y = B[kb];
-                const float xi = sa * x.y, yi = sb * y.y;
-                acc.x = fmaf(x.x, y.x, acc.x);
-                acc.x = fmaf(-xi, yi, acc.x);
-                acc.y = fmaf(x.x, yi, acc.y);
-                acc.y = fmaf(xi, y.x, acc.y);
+            if (r.loop & kSmallDense) {
+#pragma unroll 4
+                for (int k = 0; k < nk; k++) small_term(acc, A[k], B[k], sa, sb);
+            } else {
+                const uint32_t* kt = a.ktab + r.ktab;
+#pragma unroll 4
+                for (int k = 0; k < nk; k++) {
+                    const uint32_t ko = kt[k];
+                    small_term(acc, A[ko & 0xffffu], B[ko >> 16], sa, sb);
+                }
             }
-            out[o] = acc;
+            r.out[e.o] = acc;
+            i = nx;
+            e = en;
         }
-        __syncthreads();   // outputs written before the descriptor is replaced
+        i = e1 + (int)threadIdx.x;
     }
 }
 
 }  // namespace
 
-void launch_small_steps(const StepDesc* d_steps, const StepDesc* h_steps, int n_steps, const ChunkCtx& ctx,
-                        int64_t n_traj, cudaStream_t s) {
+void launch_small_steps(const SmallRuns& sr, std::pair<int32_t, int32_t> parts, const StepDesc* h_steps, int n_steps,
+                        const ChunkCtx& ctx, int64_t n_traj, cudaStream_t s) {
     if (n_steps <= 0 || n_traj <= 0) return;
     double bytes = 0.0, flops = 0.0;
     for (int k = 0; k < n_steps; k++) {
@@ -469,7 +513,16 @@ void launch_small_steps(const StepDesc* d_steps, const StepDesc* h_steps, int n_
         flops += 8.0 * (double)n_traj * (double)h.out_size * (double)(1ll << h.n_sum);
     }
     StatScope sc(K_CONTRACT_SMALL, s, bytes, flops);
-    k_small_steps<<<(unsigned)n_traj, kSmallThreads, 0, s>>>(d_steps, n_steps, ctx);
+    // up to one trajectory per SM: the levels' elements over as many threads as a
+    // CTA has (latency); more trajectories: smaller CTAs, several per SM, so that
+    // one's barriers and address chains overlap another's arithmetic
+    const int threads = n_traj <= 152 ? 1024 : (n_traj <= 304 ? 512 : 256);
+    for (int p = parts.first; p < parts.second; p++) {
+        const SmallPart& pt = sr.parts[p];
+        const SmallArgs a{sr.d_steps + pt.step0, sr.d_ent, sr.d_lvl + pt.lvl0, sr.d_ktab, pt.n_steps, pt.n_lvl};
+        if (p > parts.first) count_launches(K_CONTRACT_SMALL);
+        k_small_steps<<<(unsigned)n_traj, threads, sizeof(SmallRes) * pt.n_steps, s>>>(a, ctx);
+    }
 }
 
 void launch_contract_step(const StepDesc* d_step, const StepDesc& h, const ChunkCtx& ctx, int64_t n_inst,

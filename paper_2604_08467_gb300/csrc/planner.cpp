@@ -1415,6 +1415,8 @@ ptn_status build_expval_plan(ptn_plan* plan) {
         delete bp;
         return e;
     }
+    build_small_runs(bp->steps, plan->opts.fuse_max, bp->small);
+    build_small_runs(bp->bwd, plan->opts.fuse_max, bp->small_bwd);
     plan->expval = bp;
     return PTN_OK;
 }
@@ -1853,6 +1855,7 @@ ptn_status build_plan(const ptn_circuit* c, const ptn_noise* nz, const int32_t* 
             if (!e) clear_error();
         }
         if (e) return e;
+        build_small_runs(bp.steps, plan->opts.fuse_max, bp.small);
         plan->blocks.push_back(std::move(bp));
         start += b;
     }

@@ -4,7 +4,9 @@
 
 #include <stdint.h>
 
+#include <map>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/ptn.h"
@@ -100,6 +102,48 @@ inline bool small_step(const StepDesc& h) {
            h.op[0].inst_size <= (1ll << kSmallOpBits) && h.op[1].inst_size <= (1ll << kSmallOpBits);
 }
 
+// Fused runs as k_small_steps executes them (small_runs.cpp): compact steps,
+// the output elements of every level, and summed-offset tables.
+struct SmallOp {
+    int64_t base;            // leaf: element of variant 0 in the variant table; buffer: arena offset per instance
+    int32_t size;            // elements per variant / instance
+    int32_t src;             // -1: merged-gate leaf; else the buffer's arena
+    int32_t inst;            // buffer: storage class (CLS_CONST: one instance)
+    int32_t col;             // leaf: variant column, -1 = single variant
+    int32_t cache;           // as OperandDesc.cache
+    int32_t pad;
+};
+struct SmallStep {
+    SmallOp op[2];
+    int64_t out_off;
+    int32_t out_size, out_arena;
+    uint32_t loop;           // terms (1 .. 256) and the kSmall* flags
+    int32_t ktab;            // first summed-offset entry (not kSmallDense)
+    int32_t pad[2];
+};
+constexpr uint32_t kSmallConjA = 1u << 16, kSmallConjB = 1u << 17, kSmallDense = 1u << 18;   // dense: offsets 0, 1, 2, ...
+struct SmallEnt {
+    uint32_t offs;           // element's offset in operand 0 (low half) and 1 (high half)
+    uint16_t step, o;        // step within the part, output element
+};
+struct SmallPart {           // at most kSmallPartSteps steps of a run: one launch
+    int32_t step0, n_steps, lvl0, n_lvl;
+};
+constexpr int kSmallPartSteps = 1024;
+struct SmallRuns {
+    std::map<int32_t, std::pair<int32_t, int32_t>> run_at;   // first step of a run -> its parts [first, second)
+    std::vector<SmallPart> parts;
+    std::vector<SmallStep> steps;
+    std::vector<SmallEnt> ent;
+    std::vector<int32_t> lvl;    // per part n_lvl + 1 entry positions
+    std::vector<uint32_t> ktab;
+    // device copies
+    SmallStep* d_steps = nullptr;
+    SmallEnt* d_ent = nullptr;
+    int32_t* d_lvl = nullptr;
+    uint32_t* d_ktab = nullptr;
+};
+
 struct LeafInfo {
     int32_t gate;            // source gate, -1 for a |0> state
     int32_t part;            // 0 whole gate / |0>, 1 factor on q0, 2 factor on q1
@@ -162,6 +206,7 @@ struct BlockPlan {
     int32_t n_cache = 0, cache_words = 0;
     std::vector<uint32_t> cache_bits;
     uint32_t* d_cache_bits = nullptr;
+    SmallRuns small, small_bwd;          // fused runs of `steps` and (gradient plans) of `bwd`
     // device copy
     StepDesc* d_steps = nullptr;
     // expectation/gradient plans only: the reversed path and its targets
@@ -214,6 +259,8 @@ ptn_status build_plan(const ptn_circuit* c, const ptn_noise* nz, const int32_t* 
 std::string describe_plan(const ptn_plan* plan, int detail);
 void classify_step(StepDesc& st, int64_t pack_floats[2][3], bool allow_tc);   // planner.cpp
 ptn_status build_expval_plan(ptn_plan* plan);                                   // planner.cpp
+int small_run_len(const std::vector<StepDesc>& steps, size_t k, int fuse_max);  // small_runs.cpp: steps of the run starting at k
+void build_small_runs(const std::vector<StepDesc>& steps, int fuse_max, SmallRuns& sr);
 // merged tensor of a parametrised leaf at angle theta (and its derivative),
 // written as complex64 into out[n_var * size] (out_d likewise)
 void param_leaf_tables(const LeafInfo& L, double theta, float* out, float* out_d);

@@ -201,6 +201,35 @@ namespace {
 
 PlanWorkspace* workspace(const ptn_plan* plan);
 
+// Device copies of a step list's fused runs (plan lifetime).
+ptn_status upload_small_runs(SmallRuns& sr) {
+    if (sr.parts.empty() || sr.d_steps) return PTN_OK;
+    auto up = [](const auto& v, auto** d) -> ptn_status {
+        const size_t by = v.size() * sizeof(v[0]);
+        if (!*d) PTN_CUDA(cudaMalloc(d, std::max(by, (size_t)16)));
+        if (by) PTN_CUDA(cudaMemcpy(*d, v.data(), by, cudaMemcpyHostToDevice));
+        return PTN_OK;
+    };
+    ptn_status e;
+    if ((e = up(sr.ent, &sr.d_ent)) || (e = up(sr.lvl, &sr.d_lvl)) || (e = up(sr.ktab, &sr.d_ktab))) return e;
+    return up(sr.steps, &sr.d_steps);
+}
+void free_small_runs(SmallRuns& sr) {
+    cudaFree(sr.d_steps);
+    cudaFree(sr.d_ent);
+    cudaFree(sr.d_lvl);
+    cudaFree(sr.d_ktab);
+}
+// Launches the fused run starting at step k, if one does; the number of steps it covers, else 0.
+int launch_small_run(const SmallRuns& sr, const std::vector<StepDesc>& steps, size_t k, int fuse_max,
+                     const ChunkCtx& ctx, int64_t n_traj, cudaStream_t s) {
+    const auto it = sr.run_at.find((int32_t)k);
+    if (it == sr.run_at.end()) return 0;
+    const int len = small_run_len(steps, k, fuse_max);
+    launch_small_steps(sr, it->second, &steps[k], len, ctx, n_traj, s);
+    return len;
+}
+
 ptn_status ensure_device(const ptn_plan* cplan) {
     ptn_plan* plan = const_cast<ptn_plan*>(cplan);
     int dev = -1;
@@ -227,6 +256,7 @@ ptn_status ensure_device(const ptn_plan* cplan) {
         size_t by = bp.steps.size() * sizeof(StepDesc);
         PTN_CUDA(cudaMalloc(&bp.d_steps, std::max(by, (size_t)16)));
         if (by) PTN_CUDA(cudaMemcpy(bp.d_steps, bp.steps.data(), by, cudaMemcpyHostToDevice));
+        if (ptn_status es = upload_small_runs(bp.small)) return es;
         if (!bp.cache_bits.empty()) {
             const size_t cb = bp.cache_bits.size() * sizeof(uint32_t);
             PTN_CUDA(cudaMalloc(&bp.d_cache_bits, cb));
@@ -525,14 +555,9 @@ ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const
             const StepDesc& h = bp.steps[st];
             if (h.virt) continue;   // formed inside its consumer's operand pack
             StepTag tag(j, (int)st);
-            if (small_step(h)) {   // a run of small trajectory-class steps: one fused launch
-                size_t en = st + 1;
-                while (en < bp.steps.size() && en - st < (size_t)plan->opts.fuse_max && bp.steps[en].fuse_prev) en++;
-                if (en - st >= 2) {
-                    launch_small_steps(bp.d_steps + st, &bp.steps[st], (int)(en - st), ctx, c.n_traj, ls);
-                    st = en - 1;
-                    continue;
-                }
+            if (const int len = launch_small_run(bp.small, bp.steps, st, plan->opts.fuse_max, ctx, c.n_traj, ls)) {
+                st += len - 1;
+                continue;
             }
             int64_t ni = h.out_cls == CLS_CONST ? 1 : (h.out_cls == CLS_TRAJ ? c.n_traj : c.n_net);
             if (ccnt && h.cache > 0) ni = ccnt[h.cache - 1];
@@ -657,8 +682,13 @@ void ptn_plan_destroy(ptn_plan* plan) {
         for (auto& b : plan->blocks) {
             cudaFree(b.d_steps);
             cudaFree(b.d_cache_bits);
+            free_small_runs(b.small);
         }
         cudaFree(plan->d_roots);
+    }
+    if (plan->expval) {
+        free_small_runs(plan->expval->small);
+        free_small_runs(plan->expval->small_bwd);
     }
     delete plan->expval;
     delete plan;
@@ -1009,9 +1039,10 @@ ptn_status ptn_contract_batch(const ptn_plan* plan, const ptn_traj* traj, int32_
 namespace {
 // Device copies of the whole-circuit ket plan (forward steps, reversed steps,
 // root, parametrised leaves), made once per plan.
-ptn_status upload_expval_plan(const BlockPlan& bp, PlanWorkspace* ws) {
+ptn_status upload_expval_plan(BlockPlan& bp, PlanWorkspace* ws) {
     if (ws->ev_steps.p) return PTN_OK;
     ptn_status e;
+    if ((e = upload_small_runs(bp.small)) || (e = upload_small_runs(bp.small_bwd))) return e;
     if ((e = ws->ev_steps.grow(sizeof(StepDesc) * std::max<size_t>(bp.steps.size(), 1))) ||
         (e = ws->ev_bwd.grow(sizeof(StepDesc) * std::max<size_t>(bp.bwd.size(), 1))) ||
         (e = ws->ev_root.grow(sizeof(RootRef))) ||
@@ -1053,7 +1084,7 @@ ptn_status ptn_trajectory_amplitudes(const ptn_plan* cplan, const ptn_traj* traj
     if (n_traj == 0) return PTN_OK;
     cudaStream_t s = (cudaStream_t)stream;
     PlanWorkspace* ws = workspace(plan);
-    const BlockPlan& bp = *plan->expval;
+    BlockPlan& bp = *plan->expval;
     if ((e = upload_expval_plan(bp, ws))) return e;
     const int64_t E = traj->n_unique;
     if ((e = ws->ev_iota.grow(sizeof(int32_t) * E))) return e;
@@ -1095,14 +1126,9 @@ ptn_status ptn_trajectory_amplitudes(const ptn_plan* cplan, const ptn_traj* traj
         for (size_t k = 0; k < bp.steps.size(); k++) {
             const StepDesc& h = bp.steps[k];
             StepTag tag(-2, (int)k);
-            if (small_step(h)) {   // a run of small trajectory-class steps: one fused launch
-                size_t en = k + 1;
-                while (en < bp.steps.size() && en - k < (size_t)plan->opts.fuse_max && bp.steps[en].fuse_prev) en++;
-                if (en - k >= 2) {
-                    launch_small_steps(ws->ev_steps.as<StepDesc>() + k, &bp.steps[k], (int)(en - k), ctx, nt, s);
-                    k = en - 1;
-                    continue;
-                }
+            if (const int len = launch_small_run(bp.small, bp.steps, k, plan->opts.fuse_max, ctx, nt, s)) {
+                k += len - 1;
+                continue;
             }
             const int64_t ni = h.out_cls == CLS_CONST ? 1 : nt;
             if (h.kind != STEP_DIRECT) {
@@ -1150,7 +1176,7 @@ ptn_status ptn_expval_grad(const ptn_plan* cplan, const ptn_traj* traj, const pt
     if ((e = ensure_device(plan))) return e;
     cudaStream_t s = (cudaStream_t)stream;
     PlanWorkspace* ws = workspace(plan);
-    const BlockPlan& bp = *plan->expval;
+    BlockPlan& bp = *plan->expval;
     const int n = plan->n_qubits;
     const int64_t E = traj->n_unique;
     const int np = std::max(n_theta, 1);
@@ -1215,18 +1241,14 @@ ptn_status ptn_expval_grad(const ptn_plan* cplan, const ptn_traj* traj, const pt
         ctx.arena_inst[CLS_CONST] = 1;
         ctx.arena_inst[CLS_TRAJ] = ctx.arena_inst[ARENA_ADJ] = ctx.arena_inst[ARENA_LGRAD] = nt;
         ctx.arena_inst[CLS_NET] = 0;
-        auto run = [&](const std::vector<StepDesc>& steps, const StepDesc* d_steps, int tag_block) -> ptn_status {
+        auto run = [&](const std::vector<StepDesc>& steps, const StepDesc* d_steps, const SmallRuns& runs,
+                       int tag_block) -> ptn_status {
             for (size_t k = 0; k < steps.size(); k++) {
                 const StepDesc& h = steps[k];
                 StepTag tag(tag_block, (int)k);
-                if (small_step(h)) {   // a run of small trajectory-class steps: one fused launch
-                    size_t en = k + 1;
-                    while (en < steps.size() && en - k < (size_t)plan->opts.fuse_max && steps[en].fuse_prev) en++;
-                    if (en - k >= 2) {
-                        launch_small_steps(d_steps + k, &steps[k], (int)(en - k), ctx, nt, s);
-                        k = en - 1;
-                        continue;
-                    }
+                if (const int len = launch_small_run(runs, steps, k, plan->opts.fuse_max, ctx, nt, s)) {
+                    k += len - 1;
+                    continue;
                 }
                 const int64_t ni = h.out_cls == CLS_CONST ? 1 : nt;
                 if (h.kind != STEP_DIRECT) {
@@ -1239,10 +1261,10 @@ ptn_status ptn_expval_grad(const ptn_plan* cplan, const ptn_traj* traj, const pt
             }
             return PTN_OK;
         };
-        if ((e = run(bp.steps, ws->ev_steps.as<StepDesc>(), -2))) return e;
+        if ((e = run(bp.steps, ws->ev_steps.as<StepDesc>(), bp.small, -2))) return e;
         launch_observable(ws->ev_root.as<RootRef>(), ctx, n, ws->ev_terms.as<ObsTerm>(), (int)terms.size(),
                           bp.root_adj_off, t0, ws->ev_F.as<double>(), s);
-        if ((e = run(bp.bwd, ws->ev_bwd.as<StepDesc>(), -3))) return e;
+        if ((e = run(bp.bwd, ws->ev_bwd.as<StepDesc>(), bp.small_bwd, -3))) return e;
         launch_leaf_grad(ctx, ws->ev_pl.as<ParamLeaf>(), (int)bp.pleaves.size(), ws->ev_dvt.as<float2>(), t0, nt, np,
                          ws->ev_partial.as<double>(), s);
     }
