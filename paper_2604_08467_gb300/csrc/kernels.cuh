@@ -102,6 +102,8 @@ struct ChunkCtx {
     const int32_t* cache_rep = nullptr;
     const int32_t* cache_list = nullptr;
     int64_t cache_n = 0;
+    // first network of every local trajectory ([arena_inst[CLS_TRAJ] + 1]), or null
+    const int32_t* grp_net0 = nullptr;
 };
 
 // Instance of a TRAJ-class buffer that local trajectory tl reads.

@@ -337,6 +337,580 @@ static void launch_micro(const StepDesc* d_step, const ChunkCtx& ctx, int64_t n_
     k_contract_micro<RA, RB><<<(unsigned)blocks, kDirThreads, 0, s>>>(d_step, ctx, n_inst, mb);
 }
 
+// SIMT contraction with both operands' summed axis contiguous (every step whose
+// operands were laid out for it): the rows a CTA needs are staged in shared
+// memory 16 terms at a time.  The kernels above let each thread walk its own
+// rows, and neighbouring lanes' rows lie a whole row apart: at 64 terms (512
+// bytes) the lines of all resident threads exceed L1 and every 8-byte read
+// fetches a sector again (the middle 30-qubit block's network step read at 131
+// GB/s).  Here a row chunk is copied once by consecutive 16-byte cp.async and
+// read back two terms at a time; rows are pitched by one extra 16-byte slot, so
+// the eight lanes of a 128-bit shared read hit different banks.  Three stages,
+// one barrier per chunk: the copies of the chunk after next are in flight while
+// a chunk is contracted.  A CTA takes units (instance, sub-tile of the output)
+// with the stride of the grid; the operand addresses of a unit are formed by
+// one thread per operand an iteration before its first copy is issued.
+// Every output is the multiply-add chain of k_contract_direct: terms in
+// increasing order within 256, blocks of 256 in Gray-code order.  Measured
+// against the micro-tiles: 1024 terms, 4096 trajectories 5.47 -> 1.81 ms (5.3
+// TB/s); 64 terms, 1024 outputs, 10,240 networks 0.65 -> 0.18 ms.
+constexpr int kRowsMax = 10;          // row bits per operand, sub-tile bits, thread-tile bits
+constexpr int kRowsChunk = 16;        // terms per stage
+constexpr int kRowsStages = 3;
+constexpr int kRowsSmem = 110 * 1024; // stages of one CTA (two per SM)
+constexpr int kRowsMinSum = 3;        // shortest summed axis (bits)
+constexpr int kGroupLog = 3;          // log2 networks contracted together by k_contract_group
+constexpr int64_t kGroupMin = 6;      // least networks per unit on average
+struct RowsArgs {
+    int32_t rb[2];                     // log2 rows staged per operand
+    int32_t r_stride[2][kRowsMax];     // operand stride of each row bit
+    int32_t n_sub, n_lane, n_sum, kc_log;
+    int32_t sub_stride[2][kMaxOut];    // sub-tile bits: operand strides, output strides
+    int64_t sub_out[kMaxOut];
+    int32_t lane_row[2][kRowsMax];     // thread index bits: row weights, output strides
+    int32_t lane_out[kRowsMax];
+    int32_t tile_row_a[2], tile_row_b[2], tile_out_a[2], tile_out_b[2];   // micro-tile bits
+};
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// two consecutive terms of one output
+__device__ __forceinline__ void rows_terms(float2& acc, const float4& a, const float4& b) {
+    acc.x = fmaf(a.x, b.x, acc.x);
+    acc.x = fmaf(-a.y, b.y, acc.x);
+    acc.y = fmaf(a.x, b.y, acc.y);
+    acc.y = fmaf(a.y, b.x, acc.y);
+    acc.x = fmaf(a.z, b.z, acc.x);
+    acc.x = fmaf(-a.w, b.w, acc.x);
+    acc.y = fmaf(a.z, b.w, acc.y);
+    acc.y = fmaf(a.w, b.z, acc.y);
+}
+
+template <int RA, int RB>
+__global__ void __launch_bounds__(256) k_contract_rows(const StepDesc* __restrict__ s, const __grid_constant__ ChunkCtx c,
+                                                       const int64_t n_inst, const __grid_constant__ RowsArgs r) {
+    extern __shared__ __align__(16) uint8_t rows_smem[];
+    constexpr int NA = 1 << RA, NB = 1 << RB;
+    const int KC = 1 << r.kc_log, pitch = KC + 2;
+    const int rows_a = 1 << r.rb[0], rows = rows_a + (1 << r.rb[1]);
+    float2* stage0 = reinterpret_cast<float2*>(rows_smem);
+    const int stage_elems = rows * pitch;
+    int32_t* row_off = reinterpret_cast<int32_t*>(stage0 + kRowsStages * stage_elems);
+    __shared__ const float2* ptr[4][2];    // operand addresses of the units in flight
+    __shared__ int64_t out_tl[4];
+    for (int i = threadIdx.x; i < rows; i += blockDim.x) {
+        const int o = i >= rows_a, v = i - (o ? rows_a : 0);
+        int32_t off = 0;
+        for (int b = 0; b < r.rb[o]; b++)
+            if ((v >> b) & 1) off += r.r_stride[o][b];
+        row_off[i] = off;
+    }
+    const int64_t n_units = n_inst << r.n_sub;
+    const int chunks_log = r.n_sum - r.kc_log, n_chunk = 1 << chunks_log;
+    const int64_t my_units = n_units > blockIdx.x ? (n_units - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+    const int64_t n_items = my_units << chunks_log;
+    auto set_unit = [&](int64_t u) {       // one thread per operand: addresses of this CTA's u-th unit
+        const int o = threadIdx.x >> 5;
+        const int64_t unit = blockIdx.x + u * gridDim.x, inst = unit >> r.n_sub;
+        const int64_t tl = step_inst(s->cache, inst, c);
+        int64_t off = 0;
+        for (int b = 0; b < r.n_sub; b++)
+            if ((unit >> b) & 1) off += r.sub_stride[o][b];
+        ptr[u & 3][o] = operand_ptr(s->op[o], s->out_cls, tl, c) + off;
+        if (o == 0) out_tl[u & 3] = tl;
+    };
+    const bool setter = threadIdx.x == 0 || threadIdx.x == 32;
+    // copies of item it (its unit's chunk) into stage it % 3
+    const int piece_log = r.kc_log - 1;    // 16-byte pieces per row chunk
+    auto issue = [&](int64_t it) {
+        if (it < n_items) {
+            const int64_t u = it >> chunks_log;
+            const int ch = (int)(it & (n_chunk - 1));
+            int k0 = ch << r.kc_log;
+            if (r.n_sum > 8) {             // blocks of 256 terms in Gray-code order
+                const int hi = k0 >> 8;
+                k0 = ((hi ^ (hi >> 1)) << 8) | (k0 & 255);
+            }
+            const float2* pa = ptr[u & 3][0] + k0;
+            const float2* pb = ptr[u & 3][1] + k0;
+            const uint32_t st = static_cast<uint32_t>(__cvta_generic_to_shared(stage0 + (int)(it % kRowsStages) * stage_elems));
+            const int n = rows << piece_log;
+            for (int i = threadIdx.x; i < n; i += blockDim.x) {
+                const int row = i >> piece_log, pc = i & ((1 << piece_log) - 1);
+                cp_async16(st + (uint32_t)(row * pitch + 2 * pc) * 8u, (row < rows_a ? pa : pb) + row_off[row] + 2 * pc);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (setter)
+        for (int64_t u = 0; u < 3 && u < my_units; u++) set_unit(u);
+    // this thread's rows and output offset
+    const bool act = (int)threadIdx.x < (1 << r.n_lane);
+    int ra = 0, rb = 0;
+    int64_t o0 = 0;
+    for (int b = 0; b < r.n_lane; b++)
+        if ((threadIdx.x >> b) & 1) {
+            ra += r.lane_row[0][b];
+            rb += r.lane_row[1][b];
+            o0 += r.lane_out[b];
+        }
+    int da[NA], db[NB];
+#pragma unroll
+    for (int i = 0; i < NA; i++) {
+        da[i] = 0;
+#pragma unroll
+        for (int j = 0; j < RA; j++)
+            if ((i >> j) & 1) da[i] += r.tile_row_a[j];
+        da[i] = (ra + da[i]) * pitch;
+    }
+#pragma unroll
+    for (int i = 0; i < NB; i++) {
+        db[i] = 0;
+#pragma unroll
+        for (int j = 0; j < RB; j++)
+            if ((i >> j) & 1) db[i] += r.tile_row_b[j];
+        db[i] = (rows_a + rb + db[i]) * pitch;
+    }
+    const float sa = s->op[0].conj ? -1.f : 1.f, sb = s->op[1].conj ? -1.f : 1.f;
+    float2* outbase = c.arena[s->out_arena] + s->out_off * c.arena_inst[s->out_arena];
+    const int64_t out_size = s->out_size;
+    __syncthreads();
+    issue(0);
+    issue(1);
+    float2 acc[NA][NB];
+    for (int64_t it = 0; it < n_items; it++) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();                   // chunk `it` has landed; stage (it + 2) % 3 is free
+        issue(it + 2);
+        if (setter && ((it + 3) & (n_chunk - 1)) == 0 && it + 3 < n_items && ((it + 3) >> chunks_log) >= 3)
+            set_unit((it + 3) >> chunks_log);
+        const int64_t u = it >> chunks_log;
+        const int ch = (int)(it & (n_chunk - 1));
+        if (!act) continue;
+        if (ch == 0) {
+#pragma unroll
+            for (int i = 0; i < NA; i++)
+#pragma unroll
+                for (int j = 0; j < NB; j++) acc[i][j] = make_float2(0.f, 0.f);
+        }
+        const float2* st = stage0 + (int)(it % kRowsStages) * stage_elems;
+#pragma unroll 2
+        for (int k = 0; k < KC; k += 2) {
+            float4 av[NA], bv[NB];
+#pragma unroll
+            for (int i = 0; i < NA; i++) {
+                av[i] = *reinterpret_cast<const float4*>(st + da[i] + k);
+                av[i].y *= sa;
+                av[i].w *= sa;
+            }
+#pragma unroll
+            for (int j = 0; j < NB; j++) {
+                bv[j] = *reinterpret_cast<const float4*>(st + db[j] + k);
+                bv[j].y *= sb;
+                bv[j].w *= sb;
+            }
+#pragma unroll
+            for (int i = 0; i < NA; i++)
+#pragma unroll
+                for (int j = 0; j < NB; j++) rows_terms(acc[i][j], av[i], bv[j]);
+        }
+        if (ch == n_chunk - 1) {
+            const int64_t unit = blockIdx.x + u * gridDim.x;
+            int64_t o = out_tl[u & 3] * out_size + o0;
+            for (int b = 0; b < r.n_sub; b++)
+                if ((unit >> b) & 1) o += r.sub_out[b];
+#pragma unroll
+            for (int i = 0; i < NA; i++)
+#pragma unroll
+                for (int j = 0; j < NB; j++) {
+                    int64_t t = o;
+#pragma unroll
+                    for (int q = 0; q < RA; q++)
+                        if ((i >> q) & 1) t += r.tile_out_a[q];
+#pragma unroll
+                    for (int q = 0; q < RB; q++)
+                        if ((j >> q) & 1) t += r.tile_out_b[q];
+                    outbase[t] = acc[i][j];
+                }
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// Networks of one trajectory whose prefixes agree on the bits an operand is
+// sliced by read the same rows of it.  k_contract_group takes units
+// (trajectory, slice value, sub-tile): it stages the shared operand's rows
+// once, lists the unit's networks, and contracts them 2^g at a time, the other
+// operand's rows double-buffered.  The middle 30-qubit block's network step (a
+// 64-term vector against 512 shared rows per network) read its rows once per
+// network, 7.3 GB through L2 for 28,000 networks: 2.98 ms by the micro-tiles,
+// 2.43 ms by k_contract_rows, 0.31 ms here (93.7 -> 9.1 ms in the 10^6-shot job).
+// Batches of 8 have to be mostly full: with 5 networks per unit 0.053 ms by
+// k_contract_rows became 0.130, with 6.6 it went from 0.115 to 0.053.
+constexpr int kGroupWin = 512;         // networks scanned at a time
+constexpr int kGroupSmem = 72 * 1024;  // stages of one CTA (three per SM)
+struct GroupArgs {
+    RowsArgs r;                        // thread, micro-tile and sub-tile bits; the private operand's row
+                                       // index has the network's place in the batch above its own rows
+    int32_t shared_op, g_log, ns;      // shared operand; log2 networks per batch; its slice bits
+    int32_t seg_log;                   // a trajectory's networks are split into 2^seg_log ranges
+    int64_t n_groups;
+};
+
+template <int RA, int RB>
+__global__ void __launch_bounds__(256) k_contract_group(const StepDesc* __restrict__ s, const __grid_constant__ ChunkCtx c,
+                                                        const __grid_constant__ GroupArgs ga) {
+    extern __shared__ __align__(16) uint8_t rows_smem[];
+    constexpr int NA = 1 << RA, NB = 1 << RB;
+    const RowsArgs& r = ga.r;
+    const int P = ga.shared_op, Q = 1 - P, K = 1 << r.n_sum, pitch = K + 2, G = 1 << ga.g_log;
+    const int rows_p = 1 << r.rb[P], rows_q = 1 << r.rb[Q];
+    float2* st_p = reinterpret_cast<float2*>(rows_smem);
+    float2* st_q0 = st_p + rows_p * pitch;
+    const int q_elems = (rows_q << ga.g_log) * pitch;
+    const float2** qptr = reinterpret_cast<const float2**>(st_q0 + 2 * q_elems);   // [kGroupWin]
+    int32_t* list = reinterpret_cast<int32_t*>(qptr + kGroupWin);                  // [kGroupWin]
+    int32_t* row_off = list + kGroupWin;                                           // [rows_p + rows_q]
+    __shared__ int cnt;
+    __shared__ const float2* pptr;
+    for (int i = threadIdx.x; i < rows_p + rows_q; i += blockDim.x) {
+        const int o = i < rows_p ? P : Q, v = i < rows_p ? i : i - rows_p;
+        int32_t off = 0;
+        for (int b = 0; b < r.rb[o]; b++)
+            if ((v >> b) & 1) off += r.r_stride[o][b];
+        row_off[i] = off;
+    }
+    const bool act = (int)threadIdx.x < (1 << r.n_lane);
+    int row0[2] = {0, 0};
+    int64_t o0 = 0;
+    for (int b = 0; b < r.n_lane; b++)
+        if ((threadIdx.x >> b) & 1) {
+            row0[0] += r.lane_row[0][b];
+            row0[1] += r.lane_row[1][b];
+            o0 += r.lane_out[b];
+        }
+    int da[NA], db[NB];
+#pragma unroll
+    for (int i = 0; i < NA; i++) {
+        da[i] = row0[0];
+#pragma unroll
+        for (int j = 0; j < RA; j++)
+            if ((i >> j) & 1) da[i] += r.tile_row_a[j];
+    }
+#pragma unroll
+    for (int i = 0; i < NB; i++) {
+        db[i] = row0[1];
+#pragma unroll
+        for (int j = 0; j < RB; j++)
+            if ((i >> j) & 1) db[i] += r.tile_row_b[j];
+    }
+    const OperandDesc& dp = s->op[P];
+    const float sa = s->op[0].conj ? -1.f : 1.f, sb = s->op[1].conj ? -1.f : 1.f;
+    float2* outbase = c.arena[s->out_arena] + s->out_off * c.arena_inst[s->out_arena];
+    const int64_t out_size = s->out_size;
+    const int64_t n_units = ga.n_groups << (r.n_sub + ga.ns + ga.seg_log);
+    const int piece_log = r.n_sum - 1;
+    for (int64_t unit = blockIdx.x; unit < n_units; unit += gridDim.x) {
+        const int sub = (int)(unit & ((1 << r.n_sub) - 1));
+        const int var = (int)((unit >> r.n_sub) & ((1 << ga.ns) - 1));
+        const int seg = (int)((unit >> (r.n_sub + ga.ns)) & ((1 << ga.seg_log) - 1));
+        const int64_t grp = unit >> (r.n_sub + ga.ns + ga.seg_log);
+        const int g0 = c.grp_net0[grp], gn = c.grp_net0[grp + 1] - g0;
+        const int n0 = g0 + (int)(((int64_t)gn * seg) >> ga.seg_log), n1 = g0 + (int)(((int64_t)gn * (seg + 1)) >> ga.seg_log);
+        int64_t sub_off[2] = {0, 0}, sub_out = o0;
+        for (int b = 0; b < r.n_sub; b++)
+            if ((sub >> b) & 1) {
+                sub_off[0] += r.sub_stride[0][b];
+                sub_off[1] += r.sub_stride[1][b];
+                sub_out += r.sub_out[b];
+            }
+        bool have_p = false;
+        for (int w0 = n0; w0 < n1; w0 += kGroupWin) {
+            __syncthreads();   // the previous window's list is no longer read
+            if (threadIdx.x == 0) cnt = 0;
+            __syncthreads();
+            const int w1 = min(w0 + kGroupWin, n1);
+            for (int net = w0 + (int)threadIdx.x; net < w1; net += blockDim.x) {
+                const uint64_t* pre = c.net_prefix + (int64_t)net * c.n_words;
+                int key = 0;
+                for (int b = 0; b < ga.ns; b++) key |= (int)bits_get(pre, dp.slice_qubit[b]) << b;
+                if (key == var) {
+                    const int i = atomicAdd(&cnt, 1);
+                    list[i] = net;
+                    qptr[i] = operand_ptr(s->op[Q], CLS_NET, net, c) + (Q ? sub_off[1] : sub_off[0]);
+                    if (i == 0) pptr = operand_ptr(dp, CLS_NET, net, c) + (P ? sub_off[1] : sub_off[0]);
+                }
+            }
+            __syncthreads();
+            const int m = cnt;
+            if (m == 0) continue;
+            if (!have_p) {
+                const uint32_t st = static_cast<uint32_t>(__cvta_generic_to_shared(st_p));
+                for (int i = threadIdx.x; i < rows_p << piece_log; i += blockDim.x) {
+                    const int row = i >> piece_log, pc = i & ((1 << piece_log) - 1);
+                    cp_async16(st + (uint32_t)(row * pitch + 2 * pc) * 8u, pptr + row_off[row] + 2 * pc);
+                }
+                have_p = true;
+            }
+            auto issue = [&](int batch) {
+                const int left = min(G, m - (batch << ga.g_log));
+                if (left > 0) {
+                    const uint32_t st = static_cast<uint32_t>(__cvta_generic_to_shared(st_q0 + (batch & 1) * q_elems));
+                    const int n = (left * rows_q) << piece_log;
+                    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+                        const int row = i >> piece_log, pc = i & ((1 << piece_log) - 1);
+                        const int net = row >> r.rb[Q], rq = row & (rows_q - 1);
+                        cp_async16(st + (uint32_t)(row * pitch + 2 * pc) * 8u,
+                                   qptr[(batch << ga.g_log) + net] + row_off[rows_p + rq] + 2 * pc);
+                    }
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            };
+            const int n_batch = (m + G - 1) >> ga.g_log;
+            issue(0);
+            for (int batch = 0; batch < n_batch; batch++) {
+                issue(batch + 1);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+                __syncthreads();
+                if (act) {
+                    const float2* sq = st_q0 + (batch & 1) * q_elems;
+                    const float2 *base_a = P == 0 ? st_p : sq, *base_b = P == 0 ? sq : st_p;
+                    float2 acc[NA][NB];
+#pragma unroll
+                    for (int i = 0; i < NA; i++)
+#pragma unroll
+                        for (int j = 0; j < NB; j++) acc[i][j] = make_float2(0.f, 0.f);
+#pragma unroll 2
+                    for (int k = 0; k < K; k += 2) {
+                        float4 av[NA], bv[NB];
+#pragma unroll
+                        for (int i = 0; i < NA; i++) {
+                            av[i] = *reinterpret_cast<const float4*>(base_a + da[i] * pitch + k);
+                            av[i].y *= sa;
+                            av[i].w *= sa;
+                        }
+#pragma unroll
+                        for (int j = 0; j < NB; j++) {
+                            bv[j] = *reinterpret_cast<const float4*>(base_b + db[j] * pitch + k);
+                            bv[j].y *= sb;
+                            bv[j].w *= sb;
+                        }
+#pragma unroll
+                        for (int i = 0; i < NA; i++)
+#pragma unroll
+                            for (int j = 0; j < NB; j++) rows_terms(acc[i][j], av[i], bv[j]);
+                    }
+#pragma unroll
+                    for (int i = 0; i < NA; i++)
+#pragma unroll
+                        for (int j = 0; j < NB; j++) {
+                            const int net = (batch << ga.g_log) + ((Q ? db[j] : da[i]) >> r.rb[Q]);
+                            if (net >= m) continue;
+                            int64_t t = list[net] * out_size + sub_out;
+#pragma unroll
+                            for (int q = 0; q < RA; q++)
+                                if ((i >> q) & 1) t += r.tile_out_a[q];
+#pragma unroll
+                            for (int q = 0; q < RB; q++)
+                                if ((j >> q) & 1) t += r.tile_out_b[q];
+                            outbase[t] = acc[i][j];
+                        }
+                }
+                __syncthreads();   // this batch's stage may be refilled
+            }
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// Split of a step for k_contract_rows (shared < 0) or, with operand `shared`
+// kept for a group of 2^g_log networks, k_contract_group; false where it does
+// not apply: a summed axis that is not contiguous in both operands, 16-byte
+// misaligned rows, or more bits than the tables hold.
+bool rows_split(const StepDesc& h, const ChunkCtx& ctx, int shared, int g_log, RowsArgs& r, int& ra, int& rb, int& smem) {
+    memset(&r, 0, sizeof r);
+    if (h.n_sum < kRowsMinSum || h.n_out < 1 || h.out_size >= (1ll << 31)) return false;
+    // 64-byte rows with few outputs to share them: 0.051 ms by the micro-tiles
+    // against 0.070 here (256 outputs per network, 28,000 networks); with 2048
+    // outputs 0.156 against 0.111 ms
+    if (h.n_sum == 3 && h.n_out < 9) return false;
+    for (int o = 0; o < 2; o++) {
+        const OperandDesc& d = h.op[o];
+        for (int q = 0; q < h.n_sum; q++)
+            if (h.sum_stride[o][q] != (int64_t)1 << q) return false;
+        const int64_t base = d.mode == OP_LEAF ? d.leaf_base : d.arena_off * ctx.arena_inst[d.arena];
+        if ((base | d.inst_size) & 1 || d.inst_size >= (1ll << 31)) return false;
+        for (int p = 0; p < h.n_out; p++)
+            if (h.out_stride[o][p] & 1) return false;
+        for (int p = 0; p < d.n_slice; p++)
+            if (d.slice_stride[p] & 1) return false;
+    }
+    // bits by who varies along them: 1 operand 0, 2 operand 1, 3 both; the places
+    // of a group's networks are extra bits n_out .. of the private operand alone
+    const int n_bits = h.n_out + (shared < 0 ? 0 : g_log), priv = 1 - shared;
+    int kind[kMaxOut + 8], rbits[2] = {0, 0};
+    bool sub[kMaxOut + 8] = {}, tile[kMaxOut + 8] = {};
+    for (int p = 0; p < h.n_out; p++) {
+        kind[p] = (h.out_stride[0][p] ? 1 : 0) | (h.out_stride[1][p] ? 2 : 0);
+        for (int o = 0; o < 2; o++) rbits[o] += (kind[p] >> o) & 1;
+    }
+    for (int p = h.n_out; p < n_bits; p++) kind[p] = 1 + priv;
+    r.n_sum = h.n_sum;
+    r.kc_log = shared >= 0 ? h.n_sum : (h.n_sum < 4 ? h.n_sum : 4);
+    const int pitch = (1 << r.kc_log) + 2;
+    auto bytes = [&] {
+        const int rows = (1 << rbits[0]) + (1 << rbits[1]);
+        if (shared < 0) return kRowsStages * rows * pitch * 8 + rows * 4;
+        return ((1 << rbits[shared]) + (2 << (rbits[priv] + g_log))) * pitch * 8 + kGroupWin * 12 + rows * 4;
+    };
+    auto free_bits = [&](int k) {
+        int n = 0;
+        for (int p = 0; p < n_bits; p++) n += kind[p] == k && !sub[p];
+        return n;
+    };
+    // sub-tiles: highest bits of the operand with more rows, until the stages of
+    // two (three) CTAs fit an SM and a 4 x 4 micro-tile leaves at most 256 threads
+    const int cap = shared < 0 ? kRowsSmem : kGroupSmem;
+    for (;;) {
+        int left = 0;
+        for (int p = 0; p < n_bits; p++) left += !sub[p];
+        const int t = std::min(2, free_bits(1)) + std::min(2, free_bits(2));
+        if (rbits[0] <= kRowsMax && rbits[1] <= kRowsMax && bytes() <= cap && left - t <= 8) break;
+        int pick = -1;
+        const int big = rbits[0] >= rbits[1] ? 1 : 2;
+        for (int want : {big, 3, 3 - big}) {
+            for (int p = h.n_out - 1; p >= 0 && pick < 0; p--)
+                if (!sub[p] && kind[p] == want) pick = p;
+            if (pick >= 0) break;
+        }
+        if (pick < 0) return false;
+        sub[pick] = true;
+        for (int o = 0; o < 2; o++) rbits[o] -= (kind[pick] >> o) & 1;
+        r.sub_stride[0][r.n_sub] = (int32_t)h.out_stride[0][pick];
+        r.sub_stride[1][r.n_sub] = (int32_t)h.out_stride[1][pick];
+        r.sub_out[r.n_sub++] = (int64_t)1 << pick;
+    }
+    // micro-tile: the highest one-operand bits (a group's networks first), the
+    // operand with fewer tile bits first, while more than 128 threads remain
+    int left = n_bits - r.n_sub;
+    int tb[2] = {0, 0}, tbit[2][2] = {{-1, -1}, {-1, -1}};
+    while (left > 7) {
+        int pick = -1;
+        for (int o : {tb[0] <= tb[1] ? 0 : 1, tb[0] <= tb[1] ? 1 : 0}) {
+            if (tb[o] >= 2) continue;
+            for (int p = n_bits - 1; p >= 0 && pick < 0; p--)
+                if (!sub[p] && !tile[p] && kind[p] == o + 1) pick = p;
+            if (pick >= 0) {
+                tbit[o][tb[o]++] = pick;
+                break;
+            }
+        }
+        if (pick < 0) break;
+        tile[pick] = true;
+        left--;
+    }
+    if (left > 8) return false;
+    ra = tb[0];
+    rb = tb[1];
+    int w[2] = {0, 0};
+    for (int p = 0; p < n_bits; p++) {
+        if (sub[p]) continue;
+        int32_t weight[2] = {0, 0};
+        for (int o = 0; o < 2; o++)
+            if ((kind[p] >> o) & 1) {
+                weight[o] = 1 << w[o];
+                if (p < h.n_out) r.r_stride[o][w[o]] = (int32_t)h.out_stride[o][p];
+                w[o]++;
+            }
+        const int32_t out = p < h.n_out ? 1 << p : 0;
+        if (tile[p]) {
+            const int o = kind[p] - 1, j = tbit[o][0] == p ? 0 : 1;
+            (o ? r.tile_row_b : r.tile_row_a)[j] = weight[o];
+            (o ? r.tile_out_b : r.tile_out_a)[j] = out;
+        } else {
+            r.lane_row[0][r.n_lane] = weight[0];
+            r.lane_row[1][r.n_lane] = weight[1];
+            r.lane_out[r.n_lane++] = out;
+        }
+    }
+    r.rb[0] = rbits[0];
+    r.rb[1] = rbits[1];
+    smem = bytes();
+    return true;
+}
+
+template <int RA, int RB>
+void launch_rows_t(const StepDesc* d_step, const ChunkCtx& ctx, int64_t n_inst, const GroupArgs& g, int smem,
+                   cudaStream_t s) {
+    static const bool attr_set = [] {
+        cudaFuncSetAttribute(k_contract_rows<RA, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowsSmem);
+        cudaFuncSetAttribute(k_contract_group<RA, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGroupSmem);
+        return true;
+    }();
+    (void)attr_set;
+    const int threads = std::max(64, 1 << g.r.n_lane);
+    const int64_t cap = 152ll * std::max(1, std::min(2048 / threads / 2, 220 * 1024 / (smem + 1024)));
+    if (g.n_groups) {
+        const int64_t units = g.n_groups << (g.r.n_sub + g.ns + g.seg_log);
+        k_contract_group<RA, RB><<<(unsigned)std::min(units, cap), threads, smem, s>>>(d_step, ctx, g);
+    } else {
+        const int64_t units = n_inst << g.r.n_sub;
+        k_contract_rows<RA, RB><<<(unsigned)std::min(units, cap), threads, smem, s>>>(d_step, ctx, n_inst, g.r);
+    }
+}
+
+// Runs a step by k_contract_group or k_contract_rows where one of them applies.
+bool launch_rows(const StepDesc* d_step, const StepDesc& h, const ChunkCtx& ctx, int64_t n_inst, cudaStream_t s) {
+    GroupArgs g;
+    memset(&g, 0, sizeof g);
+    int ra, rb, smem;
+    // shared operand: a trajectory- or circuit-level buffer, the one with more
+    // elements per network; grouped where a unit finds at least kGroupMin
+    // networks on average
+    bool ok = false;
+    if (h.out_cls == CLS_NET && ctx.grp_net0 && h.n_sum <= 8) {
+        int p = -1;
+        int64_t best = 0;
+        for (int o = 0; o < 2; o++) {
+            const OperandDesc& d = h.op[o];
+            const int64_t elems = d.inst_size >> d.n_slice;
+            if (d.mode == OP_BUF && d.cls != CLS_NET && d.n_slice <= 12 && elems > best) {
+                best = elems;
+                p = o;
+            }
+        }
+        const int64_t groups = ctx.arena_inst[CLS_TRAJ];
+        if (p >= 0 && n_inst >= kGroupMin * (groups << h.op[p].n_slice) &&
+            rows_split(h, ctx, p, kGroupLog, g.r, ra, rb, smem)) {
+            g.shared_op = p;
+            g.g_log = kGroupLog;
+            g.ns = h.op[p].n_slice;
+            g.n_groups = groups;
+            // ranges of a trajectory's networks: enough units for every CTA slot,
+            // each still with kGroupMin networks
+            while ((groups << (g.r.n_sub + g.ns + g.seg_log)) < 152 * 6 &&
+                   n_inst >= 2 * kGroupMin * (groups << (g.ns + g.seg_log)))
+                g.seg_log++;
+            ok = true;
+        }
+    }
+    if (!ok && !rows_split(h, ctx, -1, 0, g.r, ra, rb, smem)) return false;
+    switch (ra * 3 + rb) {
+        case 0: launch_rows_t<0, 0>(d_step, ctx, n_inst, g, smem, s); break;
+        case 1: launch_rows_t<0, 1>(d_step, ctx, n_inst, g, smem, s); break;
+        case 2: launch_rows_t<0, 2>(d_step, ctx, n_inst, g, smem, s); break;
+        case 3: launch_rows_t<1, 0>(d_step, ctx, n_inst, g, smem, s); break;
+        case 4: launch_rows_t<1, 1>(d_step, ctx, n_inst, g, smem, s); break;
+        case 5: launch_rows_t<1, 2>(d_step, ctx, n_inst, g, smem, s); break;
+        case 6: launch_rows_t<2, 0>(d_step, ctx, n_inst, g, smem, s); break;
+        case 7: launch_rows_t<2, 1>(d_step, ctx, n_inst, g, smem, s); break;
+        default: launch_rows_t<2, 2>(d_step, ctx, n_inst, g, smem, s); break;
+    }
+    return true;
+}
+
 // marg[n][x] = Re(root_n[x]) (the double-layer diagonal), Z[n] = sum_x in FP64.
 // One block per (network, tile of kFinTile consecutive block outcomes x); a
 // thread takes kFinPer consecutive x and steps its root offset from x to x + 1
@@ -548,6 +1122,7 @@ void launch_contract_step(const StepDesc* d_step, const StepDesc& h, const Chunk
     }
     const double flops = 8.0 * (double)total * (double)(1ll << h.n_sum);
     StatScope sc(K_CONTRACT_DIRECT, s, bytes, flops);
+    if (!h.tile && launch_rows(d_step, h, ctx, n_inst, s)) return;
     // micro-tile bits: the highest output bits along which only one operand varies
     MicroBits mb;
     memset(&mb, 0, sizeof mb);

@@ -546,6 +546,7 @@ ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const
         ctx.arena_inst[CLS_CONST] = 1;
         ctx.arena_inst[CLS_TRAJ] = c.n_traj;
         ctx.arena_inst[CLS_NET] = c.n_net;
+        ctx.grp_net0 = gt.d_net0;
         if (ccnt) {
             ctx.cache_rep = ws->c_rep.as<int32_t>();
             ctx.cache_list = ws->c_list.as<int32_t>();
