@@ -32,6 +32,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstring>
 
@@ -107,6 +108,7 @@ struct PackArgs {
     // each factor having at most 2^31 elements per instance); xconj: conjugate the product
     int32_t prod, xconj;
     OperandDesc op1;
+    int32_t run_log;         // k_pack_rows: log2 consecutive units of a warp
 };
 
 struct GemmArgs {
@@ -416,6 +418,276 @@ __global__ void __launch_bounds__(256) k_pack(const __grid_constant__ PackArgs a
                     im = csign * v.y;
                 }
                 pack_store<F>(a, d0, rowlen, kc, re, im);
+            }
+        }
+    }
+}
+
+// Four real components (two consecutive complex slots) of a packed row: the
+// hi and lo stores of a role.
+template <int F>
+struct Quad;
+template <>
+struct Quad<FMT_TF32> {
+    static __device__ __forceinline__ void store(float* d, float a, float b, float c, float e) {
+        *reinterpret_cast<float4*>(d) = make_float4(a, b, c, e);
+    }
+};
+template <>
+struct Quad<FMT_BF16> {
+    static __device__ __forceinline__ void store(__nv_bfloat16* d, __nv_bfloat16 a, __nv_bfloat16 b, __nv_bfloat16 c,
+                                                 __nv_bfloat16 e) {
+        __nv_bfloat162 v[2] = {__halves2bfloat162(a, b), __halves2bfloat162(c, e)};
+        *reinterpret_cast<uint2*>(d) = *reinterpret_cast<uint2*>(v);
+    }
+};
+template <>
+struct Quad<FMT_FP16> {
+    static __device__ __forceinline__ void store(__half* d, __half a, __half b, __half c, __half e) {
+        __half2 v[2] = {__halves2half2(a, b), __halves2half2(c, e)};
+        *reinterpret_cast<uint2*>(d) = *reinterpret_cast<uint2*>(v);
+    }
+};
+// Slots kc, kc + 1 = (re0, im0), (re1, im1) of the row at d0 (the pair of rows, realified).
+template <int F, int ROLE>
+__device__ __forceinline__ void pack_store2(typename Fmt<F>::T* d0, int64_t Kh, int kc, float re0, float im0, float re1,
+                                            float im1) {
+    using T = typename Fmt<F>::T;
+    T rh0, rl0, ih0, il0, rh1, rl1, ih1, il1;
+    split<F>(re0, rh0, rl0);
+    split<F>(im0, ih0, il0);
+    split<F>(re1, rh1, rl1);
+    split<F>(im1, ih1, il1);
+    T* d = d0 + 2 * kc;
+    if (ROLE == 0) {
+        Quad<F>::store(d, rh0, ih0, rh1, ih1);
+        Quad<F>::store(d + Kh, rl0, il0, rl1, il1);
+    } else {
+        T nh0, nl0, nh1, nl1;
+        split<F>(-im0, nh0, nl0);
+        split<F>(-im1, nh1, nl1);
+        Quad<F>::store(d, rh0, nh0, rh1, nh1);
+        Quad<F>::store(d + Kh, rl0, nl0, rl1, nl1);
+        Quad<F>::store(d + 2 * Kh, ih0, rh0, ih1, rh1);
+        Quad<F>::store(d + 3 * Kh, il0, rl0, il1, rl1);
+    }
+}
+// Scale of a segment whose largest |component| over the lanes of a row (g of
+// them) is mx, and its exponent.
+template <int G>
+__device__ __forceinline__ float seg_scale(float mx, int g, int& e) {
+#pragma unroll
+    for (int o = G >> 1; o > 0; o >>= 1)
+        if (o < g) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    e = row_exponent(mx);
+    return ldexpf(1.f, -e);
+}
+
+// Packing of an operand whose summed axis is contiguous and 16-byte aligned
+// (all but a few steps): k_pack above forms an offset and reads 8 bytes per
+// slot, keeps 16 registers of slots whatever the row's length, and walks rows
+// grid-strided, so short rows spend most of their time on addresses (2.6 TB/s
+// at 128 slots per row).  Here a lane takes two consecutive slots per 16-byte
+// read, a warp a run of consecutive units (row, segment of at most 512
+// slots) so that the instance's address is formed once per run, and NV * UN
+// reads per lane are in flight.  Row offsets come from a three-level table of
+// 7 bits each.  Same values, scales and layout as k_pack.  It is bound by
+// HBM: 4096 trajectories of the middle 30-qubit block, 128 slots per row (74.5 GB)
+// 29.0 -> 12.3 ms (6.1 TB/s), 256 slots (23.2 GB) 4.82 -> 3.44 ms.
+template <int F, int ROLE, int NV>
+__global__ void __launch_bounds__(256) k_pack_rows(const __grid_constant__ PackArgs a, const __grid_constant__ ChunkCtx c) {
+    using T = typename Fmt<F>::T;
+    constexpr int UN = NV >= 4 ? 1 : 4 / NV;            // units in flight per lane group
+    __shared__ int64_t rtab[3 * 128];
+    for (int i = threadIdx.x; i < 3 * 128; i += blockDim.x) {
+        int64_t off = 0;
+        for (int t = 0; t < 7; t++) {
+            const int b = (i >> 7) * 7 + t;
+            if (b < a.n_rb && ((i >> t) & 1)) off += a.r_stride[b];
+        }
+        rtab[i] = off;
+    }
+    __syncthreads();
+    T* dst = static_cast<T*>(a.dst);
+    const int lane = threadIdx.x & 31;
+    const int seg_log = a.n_kb < 9 ? a.n_kb : 9;        // slots of a unit
+    const int nseg_log = a.n_kb - seg_log;
+    const int g_log = seg_log < 6 ? seg_log - 1 : 5;    // lanes per unit
+    const int g = 1 << g_log, l0 = lane & (g - 1), per_log = 5 - g_log;
+    const int kcp = a.Kh / 2, pad = kcp - (1 << a.n_kb);   // padding slots (rows of one unit only)
+    const int64_t n_units = (a.n_pinst << (a.n_hb + a.n_rb)) << nseg_log;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const float csign = a.op.conj ? -1.f : 1.f;
+    int64_t cur_z = -1;
+    const float2* base = nullptr;
+    const int run = 1 << a.run_log;
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; (w << a.run_log) < n_units; w += warps) {
+        for (int i0 = 0; i0 < run; i0 += UN << per_log) {
+            float4 v[UN][NV];
+            int64_t unit[UN];
+#pragma unroll
+            for (int j = 0; j < UN; j++) {
+                unit[j] = (w << a.run_log) + i0 + (j << per_log) + (lane >> g_log);
+                const bool act = unit[j] < n_units;
+                if (!act) unit[j] = -1;
+                const int64_t jr = (act ? unit[j] : n_units - 1) >> nseg_log;
+                const int64_t row = jr & (((int64_t)1 << a.n_rb) - 1), z = jr >> a.n_rb;
+                if (z != cur_z) {
+                    cur_z = z;
+                    const int64_t h = z & (((int64_t)1 << a.n_hb) - 1);
+                    const int64_t pi = a.inst_map ? (int64_t)a.inst_map[z >> a.n_hb] : z >> a.n_hb;
+                    base = pack_operand_ptr(a.op, a.pcls, pi, c);
+                    for (int t = 0; t < a.n_hb; t++)
+                        if ((h >> t) & 1) base += a.h_stride[t];
+                }
+                int64_t off = rtab[row & 127] + rtab[128 + ((row >> 7) & 127)] + rtab[256 + ((row >> 14) & 127)];
+                for (int t = 21; t < a.n_rb; t++)
+                    if ((row >> t) & 1) off += a.r_stride[t];
+                const float2* src = base + off + ((act ? unit[j] & ((1 << nseg_log) - 1) : 0) << seg_log) + 2 * l0;
+#pragma unroll
+                for (int q = 0; q < NV; q++)
+                    v[j][q] = *reinterpret_cast<const float4*>(src + 2 * (q << g_log));
+            }
+#pragma unroll
+            for (int j = 0; j < UN; j++) {
+                float sc = 1.f;
+                if constexpr (F == FMT_FP16) {
+                    float mx = 0.f;
+#pragma unroll
+                    for (int q = 0; q < NV; q++)
+                        mx = fmaxf(mx, fmaxf(fmaxf(fabsf(v[j][q].x), fabsf(v[j][q].y)),
+                                             fmaxf(fabsf(v[j][q].z), fabsf(v[j][q].w))));
+                    int e;
+                    sc = seg_scale<32>(mx, g, e);
+                    if (l0 == 0 && unit[j] >= 0) a.row_exp[unit[j]] = (int8_t)e;
+                }
+                if (unit[j] >= 0) {
+                    const float si = csign * sc;
+                    T* d0 = dst + (unit[j] >> nseg_log) * (ROLE ? 4 : 2) * (int64_t)a.Kh;
+                    const int k0 = (int)(unit[j] & ((1 << nseg_log) - 1)) << seg_log;
+#pragma unroll
+                    for (int q = 0; q < NV; q++)
+                        pack_store2<F, ROLE>(d0, a.Kh, k0 + 2 * (l0 + (q << g_log)), v[j][q].x * sc, v[j][q].y * si,
+                                             v[j][q].z * sc, v[j][q].w * si);
+                    for (int k = 2 * l0; k < pad; k += 2 << g_log)
+                        pack_store2<F, ROLE>(d0, a.Kh, (1 << a.n_kb) + k, 0.f, 0.f, 0.f, 0.f);
+                }
+            }
+        }
+    }
+}
+
+// Packing of an outer-product operand: the factors' elements that one packed
+// instance's rows read (2^n_rb rows by the summed bits each factor varies
+// along) are staged in shared memory in the order of the summed axis, so that
+// forming a slot is two conflict-free shared reads instead of two scattered
+// global ones with table offsets.  One CTA per packed instance at a time, a
+// warp per (row, segment).  Same values as k_pack.  Bound by the HBM writes of
+// the packed rows: the middle 30-qubit block's product rows (8 x 4096 slots per
+// network) with the trajectory operand they meet, 274 GB, 96.2 -> 43.7 ms (6.3
+// TB/s).
+constexpr int kProdStage = 1024;      // elements of one factor per packed instance
+constexpr int kProdHi = 256;          // combinations of the summed bits above the lowest six
+template <int F, int ROLE>
+__global__ void __launch_bounds__(256) k_pack_prod(const __grid_constant__ PackArgs a, const __grid_constant__ ChunkCtx c) {
+    using T = typename Fmt<F>::T;
+    __shared__ float2 st[2][kProdStage];
+    __shared__ int16_t hidx[2][kProdHi];
+    __shared__ int64_t sbase[2];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // compact index of a factor: its summed bits in order (n_kf of them), rows above
+    int n_kf[2] = {0, 0}, lidx[2][2] = {{0, 0}, {0, 0}};   // lane's two slots: index of the low six bits
+    for (int t = 0; t < a.n_kb; t++) {
+        const int64_t sf[2] = {a.k_stride[t] & kLo32, a.k_stride[t] >> 32};
+#pragma unroll
+        for (int f = 0; f < 2; f++) {
+            if (!sf[f]) continue;
+            if (t < 6) {
+                lidx[f][0] |= ((2 * lane) >> t & 1) << n_kf[f];
+                lidx[f][1] |= ((2 * lane + 1) >> t & 1) << n_kf[f];
+            }
+            n_kf[f]++;
+        }
+    }
+    const int n_hi = 1 << (a.n_kb - 6);
+    for (int i = threadIdx.x; i < 2 * n_hi; i += blockDim.x) {
+        const int f = i >= n_hi, v = i & (n_hi - 1);
+        int x = 0, n = 0;
+        for (int t = 0; t < a.n_kb; t++) {
+            if (!(f ? a.k_stride[t] >> 32 : a.k_stride[t] & kLo32)) continue;
+            if (t >= 6) x |= (v >> (t - 6) & 1) << n;
+            n++;
+        }
+        hidx[f][v] = (int16_t)x;
+    }
+    T* dst = static_cast<T*>(a.dst);
+    const int seg_log = a.n_kb < 9 ? a.n_kb : 9, nseg_log = a.n_kb - seg_log, nv = 1 << (seg_log - 6);
+    const float csign = a.xconj ? -1.f : 1.f;
+    const float s0 = a.op.conj ? -1.f : 1.f, s1 = a.op1.conj ? -1.f : 1.f;
+    const int64_t nz = a.n_pinst << a.n_hb;
+    for (int64_t z = blockIdx.x; z < nz; z += gridDim.x) {
+        __syncthreads();   // the previous instance's factors are no longer read
+        if (lane == 0 && warp < 2) {
+            const int64_t h = z & (((int64_t)1 << a.n_hb) - 1);
+            const int64_t pi = a.inst_map ? (int64_t)a.inst_map[z >> a.n_hb] : z >> a.n_hb;
+            int64_t off = 0;
+            for (int t = 0; t < a.n_hb; t++)
+                if ((h >> t) & 1) off += a.h_stride[t];
+            sbase[warp] = reinterpret_cast<int64_t>(warp ? pack_operand_ptr(a.op1, a.pcls, pi, c) + (off >> 32)
+                                                         : pack_operand_ptr(a.op, a.pcls, pi, c) + (off & kLo32));
+        }
+        __syncthreads();
+#pragma unroll
+        for (int f = 0; f < 2; f++) {
+            const float2* b = reinterpret_cast<const float2*>(sbase[f]);
+            for (int i = threadIdx.x; i < 1 << (n_kf[f] + a.n_rb); i += blockDim.x) {
+                int64_t off = 0;
+                int n = 0;
+                for (int t = 0; t < a.n_kb; t++) {
+                    const int64_t sf = f ? a.k_stride[t] >> 32 : a.k_stride[t] & kLo32;
+                    if (sf && ((i >> n++) & 1)) off += sf;
+                }
+                for (int t = 0; t < a.n_rb; t++)
+                    if ((i >> (n_kf[f] + t)) & 1) off += f ? a.r_stride[t] >> 32 : a.r_stride[t] & kLo32;
+                float2 x = b[off];
+                x.y *= f ? s1 : s0;
+                st[f][i] = x;
+            }
+        }
+        __syncthreads();
+        for (int u = warp; u < 1 << (a.n_rb + nseg_log); u += 8) {
+            const int row = u >> nseg_log, sg = u & ((1 << nseg_log) - 1);
+            const float2 *f0 = st[0] + (row << n_kf[0]), *f1 = st[1] + (row << n_kf[1]);
+            float4 v[8];
+            float mx = 0.f;
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                if (q >= nv) break;
+                const int h0 = hidx[0][(sg << (seg_log - 6)) + q], h1 = hidx[1][(sg << (seg_log - 6)) + q];
+                float r[4];
+#pragma unroll
+                for (int e = 0; e < 2; e++) {
+                    const float2 x = f0[lidx[0][e] + h0], y = f1[lidx[1][e] + h1];
+                    r[2 * e] = fmaf(-x.y, y.y, fmaf(x.x, y.x, 0.f));
+                    r[2 * e + 1] = fmaf(x.y, y.x, fmaf(x.x, y.y, 0.f));
+                }
+                v[q] = make_float4(r[0], r[1], r[2], r[3]);
+                mx = fmaxf(mx, fmaxf(fmaxf(fabsf(r[0]), fabsf(r[1])), fmaxf(fabsf(r[2]), fabsf(r[3]))));
+            }
+            const int64_t jr = (z << a.n_rb) + row;
+            float sc = 1.f;
+            if constexpr (F == FMT_FP16) {
+                int e;
+                sc = seg_scale<32>(mx, 32, e);
+                if (lane == 0) a.row_exp[(jr << nseg_log) + sg] = (int8_t)e;
+            }
+            const float si = csign * sc;
+            T* d0 = dst + jr * (ROLE ? 4 : 2) * (int64_t)a.Kh;
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                if (q >= nv) break;
+                pack_store2<F, ROLE>(d0, a.Kh, (sg << seg_log) + 64 * q + 2 * lane, v[q].x * sc, v[q].y * si, v[q].z * sc,
+                                     v[q].w * si);
             }
         }
     }
@@ -973,6 +1245,55 @@ unsigned grid_of(int64_t n) {
     return (unsigned)(b > 152 * 16 ? 152 * 16 : (b < 1 ? 1 : b));
 }
 
+// Whether an operand's summed axis is contiguous and its rows start on 16-byte
+// boundaries (k_pack_rows).
+bool pack_dense(const PackArgs& p, const ChunkCtx& c) {
+    const OperandDesc& d = p.op;
+    if (p.prod || p.n_kb < 3) return false;
+    for (int t = 0; t < p.n_kb; t++)
+        if (p.k_stride[t] != (int64_t)1 << t) return false;
+    const int64_t base = d.mode == OP_LEAF ? d.leaf_base : d.arena_off * c.arena_inst[d.arena];
+    int64_t odd = base | d.inst_size;
+    for (int t = 0; t < p.n_rb; t++) odd |= p.r_stride[t];
+    for (int t = 0; t < p.n_hb; t++) odd |= p.h_stride[t];
+    for (int t = 0; t < d.n_slice; t++) odd |= d.slice_stride[t];
+    return !(odd & 1);
+}
+// Whether the factors' elements of one packed instance fit k_pack_prod's stages.
+bool pack_prod_fits(const PackArgs& p) {
+    if (!p.prod || p.n_kb < 6 || (1 << (p.n_kb - 6)) > kProdHi || p.n_rb > 10) return false;
+    int n[2] = {p.n_rb, p.n_rb};
+    for (int t = 0; t < p.n_kb; t++) {
+        n[0] += (p.k_stride[t] & kLo32) != 0;
+        n[1] += (p.k_stride[t] >> 32) != 0;
+    }
+    return (1 << n[0]) <= kProdStage && (1 << n[1]) <= kProdStage;
+}
+template <int F, int ROLE>
+void launch_pack_rows(PackArgs p, const ChunkCtx& ctx, int64_t n_units, cudaStream_t s) {
+    // a warp takes up to 32 consecutive units, fewer (at least what it handles at
+    // once) where that would leave some of eight CTAs per SM without work
+    const int per_log = p.n_kb < 6 ? 6 - p.n_kb : 0, un_log = p.n_kb <= 6 ? 2 : (p.n_kb == 7 ? 1 : 0);
+    p.run_log = 5;
+    while (p.run_log > per_log + un_log && (n_units >> p.run_log) < 152 * 8 * 8) p.run_log--;
+    const int64_t per_block = (int64_t)8 << p.run_log;
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((n_units + per_block - 1) / per_block, 152 * 8));
+    switch (p.n_kb) {
+        default: k_pack_rows<F, ROLE, 8><<<(unsigned)blocks, 256, 0, s>>>(p, ctx); break;
+        case 8: k_pack_rows<F, ROLE, 4><<<(unsigned)blocks, 256, 0, s>>>(p, ctx); break;
+        case 7: k_pack_rows<F, ROLE, 2><<<(unsigned)blocks, 256, 0, s>>>(p, ctx); break;
+        case 6: case 5: case 4: case 3: k_pack_rows<F, ROLE, 1><<<(unsigned)blocks, 256, 0, s>>>(p, ctx); break;
+    }
+}
+template <int F, int ROLE>
+void launch_pack(const PackArgs& p, const ChunkCtx& ctx, int64_t slots, cudaStream_t s) {
+    const int64_t rows = p.n_pinst << (p.n_hb + p.n_rb);
+    if (pack_dense(p, ctx)) launch_pack_rows<F, ROLE>(p, ctx, rows << (p.n_kb > 9 ? p.n_kb - 9 : 0), s);
+    else if (pack_prod_fits(p))
+        k_pack_prod<F, ROLE><<<(unsigned)std::min<int64_t>(p.n_pinst << p.n_hb, 152 * 8), 256, 0, s>>>(p, ctx);
+    else k_pack<F><<<grid_of(slots), 256, 0, s>>>(p, ctx);   // (grid_of sizes by complex slots; the kernel strides over rows)
+}
+
 template <int F>
 ptn_status run_gemm(const StepDesc& st, const ChunkCtx& ctx, int64_t n_inst, void* pack_a, void* pack_b,
                     int* err, const GroupTable& grp, cudaStream_t s, const StepDesc* prod_src) {
@@ -1112,11 +1433,8 @@ ptn_status run_gemm(const StepDesc& st, const ChunkCtx& ctx, int64_t n_inst, voi
         };
         StatScope sc(K_PACK, s, rd(pa, tot_a) + rd(pb, tot_b) + 4.0 * kEB * (double)tot_a + 8.0 * kEB * (double)tot_b,
                      0.0);
-        // (grid_of sizes by complex slots; the kernels stride over rows)
-        for (PackArgs* pk : {&pa, &pb}) {
-            const int64_t tot = pk == &pa ? tot_a : tot_b;
-            k_pack<F><<<grid_of(tot), 256, 0, s>>>(*pk, ctx);
-        }
+        launch_pack<F, 0>(pa, ctx, tot_a, s);
+        launch_pack<F, 1>(pb, ctx, tot_b, s);
         count_launches(K_PACK);   // two pack kernels under one scope
     }
     CUtensorMap mA, mB;
