@@ -50,10 +50,11 @@ constexpr int kStages = 3;        // pipeline depth (4 tiles of 16 KB per stage)
 constexpr int kTileA = kBM * kRowBytes;
 constexpr int kTileB = kBN * kRowBytes;
 constexpr int kStageBytes = 2 * kTileA + 2 * kTileB;
-// epilogue staging for column-contiguous outputs: per epilogue warp a 32-row x
-// 16-column complex fragment (rows padded to 17 slots) and its 32 row offsets
-constexpr int kStgPitch = 17;
-constexpr int kStgBytes = 4 * (32 * kStgPitch * 8 + 32 * 8);
+// epilogue staging: per epilogue warp a fragment of 32 rows x 8 complex columns,
+// rows padded to 9 slots (the 8-byte writes of a column and most reads hit
+// different banks)
+constexpr int kStgPitch = 9;
+constexpr int kStgBytes = 8 * 32 * kStgPitch * 8;
 constexpr int kTabBytes = 8192;   // barriers, TMEM slot, per-warp column offsets and FP16 column scales
 constexpr int kGemmSmem = 1024 + kStages * kStageBytes + kTabBytes + kStgBytes;   // align slack + stages + tables + staging
 constexpr int kMaxPackBits = 40;
@@ -116,7 +117,14 @@ struct GemmArgs {
     int32_t n_h;
     int32_t a_pcls, b_pcls, out_cls;
     int32_t n_mb, n_nb, n_hb;
-    int32_t col_out;             // the lowest output bit is a column (N) bit: stores go column-contiguous
+    // Staged stores: the 8 bits of a fragment (5 row bits, 3 column bits) by
+    // increasing output stride; a lane stores pairs along bit 0, bits 1-5 run
+    // over the lanes, bits 6-7 over its four stores.
+    int32_t staged;              // 0: the lowest five output bits are row bits, lanes store their own rows
+    int32_t frag_vec;            // bit 0 has stride 1 and every address is even: 16-byte stores
+    int32_t frag_sm[8], frag_row[8];   // place in the staged fragment, row within the 32
+    int64_t frag_out[8];
+    int64_t row_hi[2];           // output strides of rows 32 and 64 of a tile
     int64_t tiles_m, tiles_n, n_inst, n_tiles;
     const int32_t* net_tl;
     // stacked mode: the rows of all networks of one trajectory form one GEMM
@@ -893,8 +901,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
     volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
     int64_t* noff_all = reinterpret_cast<int64_t*>(tslot + 4);   // 8 epilogue warps x kBN / 2 column offsets
     float* ucol_all = reinterpret_cast<float*>(noff_all + 8 * (kBN / 2));   // FP16: column scales 2^eb
-    float2* stg_all = reinterpret_cast<float2*>(smem + kStages * kStageBytes + kTabBytes);   // column-contiguous staging
-    int64_t* rbase_all = reinterpret_cast<int64_t*>(stg_all + 4 * 32 * kStgPitch);
+    float2* stg_all = reinterpret_cast<float2*>(smem + kStages * kStageBytes + kTabBytes);   // staged fragments
     // Work items are (tile, K segment) pairs.  A tile's k-blocks run in
     // segments of at most kSegKb; the tensor core's accumulation truncates, so
     // long chains drift: every segment is accumulated on its own and the
@@ -916,7 +923,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
         }
         for (int k = 0; k < 2; k++) {
             mbar_init(&acc_full[k], 1);
-            mbar_init(&acc_empty[k], g.col_out ? 4 : 8);   // one arrival per working epilogue warp
+            mbar_init(&acc_empty[k], 8);   // one arrival per epilogue warp
         }
         mbar_init(drain, 1);
         *abort = 0;
@@ -1016,21 +1023,35 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
         // epilogue warps 2..9: TMEM lane quadrant q = warp % 4 holds tile rows
         // 32q..32q+31; two warps per quadrant drain half of the tile's columns
         // each (one warp per SM sub-partition leaves its load and store
-        // latencies exposed).  Column-contiguous outputs, which go through the
-        // staging buffers, use warps 2..5 only, each over all columns.
+        // latencies exposed).  Where the lowest five output bits are row bits a
+        // lane stores its own row's columns and the warp writes 256 consecutive
+        // bytes.  Every other layout goes through a staged fragment whose
+        // elements the lanes take in the order of the output (sorting the
+        // fragment's row and column bits by stride): a layout of 2^20 outputs
+        // by 128 terms with seven low column bits wrote at 1.4 TB/s with four
+        // warps staging 16 columns.  4096 trajectories of the middle 30-qubit
+        // block: that step 23.9 -> 16.1 ms, one with four hyper bits (55 GB)
+        // 12.7 -> 9.1 ms (6.0 TB/s); all GEMMs of the 10^6-shot job 149 -> 132 ms.
         const int ew = warp - 2, q = warp & 3;
-        const int n_epi = g.col_out ? 4 : 8;
-        const int c_lo = g.col_out ? 0 : (ew >> 2) * (kBN / 2), c_hi = g.col_out ? kBN : c_lo + kBN / 2;
+        const int c_lo = (ew >> 2) * (kBN / 2), c_hi = c_lo + kBN / 2;
         int64_t* noff = noff_all + ew * (kBN / 2);
         float* ucol = ucol_all + ew * (kBN / 2);
-        float2* stg = stg_all + (ew & 3) * 32 * kStgPitch;
-        int64_t* rbase = rbase_all + (ew & 3) * 32;
+        float2* stg = stg_all + ew * 32 * kStgPitch;
+        int sm_l = 0, row_l = 0;
+        int64_t out_l = (q & 1 ? g.row_hi[0] : 0) + (q & 2 ? g.row_hi[1] : 0);
+        for (int b = 0; b < 5; b++)
+            if ((lane >> b) & 1) {
+                sm_l += g.frag_sm[b + 1];
+                row_l += g.frag_row[b + 1];
+                out_l += g.frag_out[b + 1];
+            }
         int64_t lt = 0;
-        bool live = ew < n_epi;
+        bool live = true;
         for (int64_t tile = blockIdx.x; tile < n_tiles && live; tile += gridDim.x) {
             if (__shfl_sync(0xffffffffu, *abort, 0)) break;   // warp-uniform stop
             const TileInfo t = decode_tile(g, tile);
-            for (int c = c_lo / 2 + lane; c < c_hi / 2; c += 32) {   // output offsets of this warp's columns
+            // output offsets of this warp's columns (staged: of its fragments' first columns)
+            for (int c = c_lo / 2 + lane; c < c_hi / 2; c += 32) {
                 const int64_t n = (int64_t)(t.n0 / 2) + c;
                 int64_t off = 0;
                 for (int i = 0; i < g.n_nb; i++)
@@ -1038,10 +1059,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                 noff[c] = off;
             }
             const int64_t row = (int64_t)t.m0 + q * 32 + lane;
-            int64_t m = row, out_inst = g.out_map ? (int64_t)g.out_map[t.inst] : t.inst;
+            const int64_t row0 = g.staged ? (int64_t)t.m0 : row;   // staged: the tile's first row
+            int64_t m = row0, out_inst = g.out_map ? (int64_t)g.out_map[t.inst] : t.inst;
             if (g.stacked) {
-                out_inst = row >> g.m_bits;
-                m = row & (((int64_t)1 << g.m_bits) - 1);
+                out_inst = row0 >> g.m_bits;
+                m = row0 & (((int64_t)1 << g.m_bits) - 1);
             }
             int64_t moff = 0;
             for (int i = 0; i < g.n_mb; i++)
@@ -1049,8 +1071,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
             for (int i = 0; i < g.n_hb; i++)
                 if ((t.h >> i) & 1) moff += g.h_stride[i];
             const bool row_ok = row < t.row_end;
-            float2* out = g.out + (row_ok ? out_inst : 0) * g.out_size + moff;
-            if (g.col_out) rbase[lane] = row_ok ? out_inst * g.out_size + moff : -1;
+            const int row_lim = (int)(t.row_end - t.m0 < 128 ? t.row_end - t.m0 : 128) - q * 32;   // valid rows of this quadrant
+            float2* out = g.out + (row_ok || g.staged ? out_inst : 0) * g.out_size + moff + (g.staged ? out_l : 0);
             __syncwarp();
             for (int sg = 0; sg < n_seg; sg++, lt++) {
                 const int set = (int)(lt % n_sets);
@@ -1089,29 +1111,32 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                 // one chunk of 32 columns of this thread's row: v[2j], v[2j+1] = complex
                 // column (c0 / 2 + j), written through the output strides
                 auto store_chunk = [&](int c0, const float* v) {
-                    if (g.col_out) {
-                        // column-contiguous output: the warp's 32 x 16 fragment goes
-                        // through shared memory, then 16 lanes store 16 consecutive
-                        // columns of one row (two rows per store instruction)
+                    if (g.staged) {
 #pragma unroll
-                        for (int j = 0; j < 16; j++) stg[lane * kStgPitch + j] = make_float2(v[2 * j], v[2 * j + 1]);
-                        __syncwarp();
-                        const int cc = lane & 15;
-                        const bool col_ok = t.n0 + c0 + 2 * cc < g.N2;
-                        const int64_t no = noff[(c0 >> 1) + cc];
-#pragma unroll 4
-                        for (int i = 0; i < 16; i++) {
-                            const int rr = 2 * i + (lane >> 4);
-                            const int64_t rb = rbase[rr];
-                            if (rb >= 0 && col_ok) g.out[rb + no] = stg[rr * kStgPitch + cc];
+                        for (int f = 0; f < 2; f++) {
+#pragma unroll
+                            for (int j = 0; j < 8; j++)
+                                stg[lane * kStgPitch + j] = make_float2(v[16 * f + 2 * j], v[16 * f + 2 * j + 1]);
+                            __syncwarp();
+                            float2* o = out + noff[(c0 >> 1) + 8 * f];
+#pragma unroll
+                            for (int i = 0; i < 4; i++) {
+                                const int sm = sm_l + (i & 1 ? g.frag_sm[6] : 0) + (i & 2 ? g.frag_sm[7] : 0);
+                                const int rr = row_l + (i & 1 ? g.frag_row[6] : 0) + (i & 2 ? g.frag_row[7] : 0);
+                                float2* d = o + ((i & 1 ? g.frag_out[6] : 0) + (i & 2 ? g.frag_out[7] : 0));
+                                const float2 x = stg[sm], y = stg[sm + g.frag_sm[0]];
+                                if (g.frag_vec && rr + g.frag_row[0] < row_lim) {
+                                    *reinterpret_cast<float4*>(d) = make_float4(x.x, x.y, y.x, y.y);
+                                } else {
+                                    if (rr < row_lim) d[0] = x;
+                                    if (rr + g.frag_row[0] < row_lim) d[g.frag_out[0]] = y;
+                                }
+                            }
+                            __syncwarp();
                         }
-                        __syncwarp();
                     } else if (row_ok) {
 #pragma unroll
-                        for (int j = 0; j < 16; j++) {
-                            const int col = t.n0 + c0 + 2 * j;
-                            if (col < g.N2) out[noff[(c0 >> 1) + j]] = make_float2(v[2 * j], v[2 * j + 1]);
-                        }
+                        for (int j = 0; j < 16; j++) out[noff[(c0 >> 1) + j]] = make_float2(v[2 * j], v[2 * j + 1]);
                     }
                 };
                 if (n_seg == 1) {
@@ -1397,13 +1422,38 @@ ptn_status run_gemm(const StepDesc& st, const ChunkCtx& ctx, int64_t n_inst, voi
     ga.n_mb = nm;
     ga.n_nb = nn;
     ga.n_hb = nh;
-    ga.col_out = (nn > 0 && ga.n_stride[0] == 1) ? 1 : 0;
     ga.tiles_m = (M + kBM - 1) / kBM;
     ga.tiles_n = (2 * N + kBN - 1) / kBN;
     ga.n_inst = n_inst;
     ga.net_tl = ctx.net_tl;
     ga.out = ctx.arena[st.out_arena] + st.out_off * ctx.arena_inst[st.out_arena];
     ga.out_size = st.out_size;
+    {
+        // rows' output strides: a stacked tile's rows above m_bits are networks
+        auto row_stride = [&](int i) {
+            return i < nm ? ga.m_stride[i] : (stacked ? st.out_size << (i - nm) : (int64_t)0);
+        };
+        bool direct = true;
+        for (int i = 0; i < 5; i++) direct = direct && row_stride(i) == (int64_t)1 << i;
+        ga.staged = direct ? 0 : 1;
+        struct Bit {
+            int64_t out;
+            int32_t sm, row;
+        } bit[8];
+        for (int i = 0; i < 5; i++) bit[i] = {row_stride(i), kStgPitch << i, 1 << i};
+        for (int i = 0; i < 3; i++) bit[5 + i] = {ga.n_stride[i], 1 << i, 0};
+        std::sort(bit, bit + 8, [](const Bit& x, const Bit& y) { return x.out < y.out; });
+        for (int i = 0; i < 8; i++) {
+            ga.frag_out[i] = bit[i].out;
+            ga.frag_sm[i] = bit[i].sm;
+            ga.frag_row[i] = bit[i].row;
+        }
+        ga.row_hi[0] = row_stride(5);
+        ga.row_hi[1] = row_stride(6);
+        // every bit above stride 1 is even; so must the instances' bases be
+        ga.frag_vec = bit[0].out == 1 && !((st.out_off * ctx.arena_inst[st.out_arena] | st.out_size) & 1);
+        if (N < kBN / 2) return set_error(PTN_ERR_INVALID_ARG, "internal: tensor-core step narrower than a tile");
+    }
     ga.out_map = cmap;
     ga.err = err;
     ga.wait_ns = g_wait_ns.load(std::memory_order_relaxed);

@@ -1,6 +1,6 @@
 """Operand packing by rows (k_pack_rows) and of outer products (k_pack_prod)
 over the lengths of the summed axis, in every format: amplitudes of circuits
-whose tensor-core steps sum 2^3 .. 2^9 terms, against the statevector.
+whose tensor-core steps sum 2^3 .. 2^12 terms, against the statevector.
 Tolerances: 1e-5 where operands hold 22 bits or more, 2^-16 relative per
 BF16 hi/lo operand pair and product, i.e. 1e-4 over a path, for BF16."""
 import numpy as np
