@@ -11,6 +11,8 @@
 //    smallest x with floor(a T / 2^64) < C[x], a = x0 << 32 | x1, T = C[last].
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "kernels.cuh"
 #include "stats.h"
 
@@ -343,8 +345,8 @@ __global__ void __launch_bounds__(256) k_sample_parents(const float* __restrict_
     if (threadIdx.x == 0) ndist[n] = wpos;
 }
 
-// Blocks of up to 2^10 bins: one warp per parent, kSampWarps parents per CTA,
-// no CTA-wide barrier.  The row is read in coalesced rounds of 32 bins (lane l
+// Blocks of up to 2^10 bins: one warp per parent at a time, kSampWarps warps per
+// CTA, no CTA-wide barrier, parents with more than min_count shots.  The row is read in coalesced rounds of 32 bins (lane l
 // holds bin 32 i + l of round i, kept in registers): the row maximum is a
 // shuffle reduction; the exact-integer CDF is built round by round with a
 // shuffle scan plus the running total in 64-bit integers (the values the FP64
@@ -354,6 +356,7 @@ __global__ void __launch_bounds__(256) k_sample_parents(const float* __restrict_
 // arithmetic and results as k_sample_parents.
 constexpr int kSampWarps = 4;
 constexpr int kSampWarpMaxBits = 10;
+constexpr int kFewShots = 16;   // parents of at most this many shots draw in registers (k_sample_few)
 
 __device__ __forceinline__ uint64_t warp_incl_scan_u64(uint64_t v, int lane) {
     for (int o = 1; o < 32; o <<= 1) {
@@ -364,8 +367,8 @@ __device__ __forceinline__ uint64_t warp_incl_scan_u64(uint64_t v, int lane) {
 }
 
 
-__global__ void __launch_bounds__(kSampWarps * 32) k_sample_parents_warp(
-    const float* __restrict__ marg, int b, int64_t n_parent, const int32_t* __restrict__ traj,
+__device__ __forceinline__ void sample_parent_warp(
+    const float* __restrict__ marg, int b, int64_t n, const int32_t* __restrict__ traj,
     const int64_t* __restrict__ count, const int64_t* __restrict__ rank0, const int64_t* __restrict__ tmp_off,
     int64_t tmp_cap, uint2 key, uint32_t tagw, int32_t* __restrict__ tmp_x, int64_t* __restrict__ tmp_c,
     int64_t* __restrict__ ndist) {
@@ -376,13 +379,7 @@ __global__ void __launch_bounds__(kSampWarps * 32) k_sample_parents_warp(
     uint64_t* C = reinterpret_cast<uint64_t*>(smem) + (int64_t)wib * nb;
     unsigned* hist = reinterpret_cast<unsigned*>(reinterpret_cast<uint64_t*>(smem) + (int64_t)kSampWarps * nb) +
                      (int64_t)wib * nb;
-    const int64_t n = (int64_t)blockIdx.x * kSampWarps + wib;
-    if (n >= n_parent) return;                 // the whole warp leaves together
     const int64_t c = count[n];
-    if (c <= 0) {
-        if (lane == 0) ndist[n] = 0;
-        return;
-    }
     const float* p = marg + n * (int64_t)nb;
     const int rounds = (nb + 31) >> 5;
     float v[kMaxRounds];
@@ -443,6 +440,137 @@ __global__ void __launch_bounds__(kSampWarps * 32) k_sample_parents_warp(
         pos += __popc(mask);
     }
     if (lane == 0) ndist[n] = pos - tmp_off[n];
+}
+
+__global__ void __launch_bounds__(kSampWarps * 32) k_sample_parents_warp(
+    const float* __restrict__ marg, int b, int64_t n_parent, const int32_t* __restrict__ traj,
+    const int64_t* __restrict__ count, const int64_t* __restrict__ rank0, const int64_t* __restrict__ tmp_off,
+    int64_t tmp_cap, uint2 key, uint32_t tagw, int32_t* __restrict__ tmp_x, int64_t* __restrict__ tmp_c,
+    int64_t* __restrict__ ndist, int64_t min_count, int grp) {
+    // the parents are taken grp <= 32 at a time (lane l looks at parent n0 + l),
+    // the chosen ones one after another by the whole warp
+    const int64_t warps = (int64_t)gridDim.x * kSampWarps;
+    const int lane = threadIdx.x & 31;
+    for (int64_t n0 = grp * ((int64_t)blockIdx.x * kSampWarps + (threadIdx.x >> 5)); n0 < n_parent; n0 += grp * warps) {
+        const bool mine = lane < grp && n0 + lane < n_parent;
+        const int64_t c = mine ? count[n0 + lane] : 0;
+        if (min_count < 0 && mine && c <= 0) ndist[n0 + lane] = 0;
+        for (unsigned todo = __ballot_sync(0xffffffffu, c > 0 && c > min_count); todo; todo &= todo - 1) {
+            sample_parent_warp(marg, b, n0 + __ffs(todo) - 1, traj, count, rank0, tmp_off, tmp_cap, key, tagw, tmp_x,
+                               tmp_c, ndist);
+            __syncwarp();   // the warp's CDF and histogram are free again
+        }
+    }
+}
+// Parents of 1 to kFewShots shots (nearly all of them past a job's first block)
+// of blocks of 128 NI bins, NI <= 8: one warp per parent, no shared memory.  The
+// full CDF of k_sample_parents_warp (a 64-bit warp scan per 32 bins, 48 KB of
+// shared memory per CTA) is not needed for a few draws: the lanes hold four
+// consecutive bins per 512-byte read, only the NI totals of 128 bins are
+// formed (one butterfly that adds and distributes them at once), and each draw
+// scans the lanes' sums of its own 128 bins.  p * 2^sigma is exact in FP32
+// (two power-of-two factors; smaller values round to zero either way), so the
+// 64-bit conversion, which rounds half to even, gives quant_pow2's integer;
+// rows with an infinite entry use quant_pow2 itself.  Bound by issue and HBM:
+// 150,000 rows of 2^10 bins with 2.5 shots on average 1.56 -> 0.37 ms (1.7
+// TB/s), the three blocks of the 10^6-shot job 18.6 -> 3.6 ms.  The line at 16
+// shots: a draw costs about 70 warp instructions here, the full CDF about 1000.
+__device__ __forceinline__ uint64_t quant_exact(float p, float f1, float f2, int sigma) {
+    return f1 == 0.f ? quant_pow2(p, sigma) : (uint64_t)__float2ll_rn(p * f1 * f2);
+}
+template <int NI>
+__global__ void __launch_bounds__(256) k_sample_few(
+    const float* __restrict__ marg, int b, int64_t n_parent, const int32_t* __restrict__ traj,
+    const int64_t* __restrict__ count, const int64_t* __restrict__ rank0, const int64_t* __restrict__ tmp_off,
+    int64_t tmp_cap, uint2 key, uint32_t tagw, int32_t* __restrict__ tmp_x, int64_t* __restrict__ tmp_c,
+    int64_t* __restrict__ ndist) {
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int GL = 32 / NI;                // lanes that hold the same total after the butterfly
+    const int lane = threadIdx.x & 31;
+    const int64_t n = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (n >= n_parent) return;                 // the whole warp leaves together
+    const int64_t c = count[n];
+    if (c <= 0 || c > kFewShots) {
+        if (c <= 0 && lane == 0) ndist[n] = 0;
+        return;
+    }
+    const float4* p = reinterpret_cast<const float4*>(marg + n * (128 * NI)) + lane;
+    float4 v[NI];
+    float m = 0.f;
+#pragma unroll
+    for (int i = 0; i < NI; i++) v[i] = p[32 * i];
+#pragma unroll
+    for (int i = 0; i < NI; i++) {
+        // entries that are not positive (NaN among them) count as zero
+        v[i].x = v[i].x > 0.f ? v[i].x : 0.f;
+        v[i].y = v[i].y > 0.f ? v[i].y : 0.f;
+        v[i].z = v[i].z > 0.f ? v[i].z : 0.f;
+        v[i].w = v[i].w > 0.f ? v[i].w : 0.f;
+        m = fmaxf(m, fmaxf(fmaxf(v[i].x, v[i].y), fmaxf(v[i].z, v[i].w)));
+    }
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kAll, m, o));
+    const int sigma = 52 - b - frexp_exp(m);
+    const bool fin = m < __int_as_float(0x7f800000);
+    const int s1 = sigma / 2, s2 = sigma - s1;   // |sigma| <= 200
+    const float f1 = fin ? __int_as_float((127 + s1) << 23) : 0.f, f2 = __int_as_float((127 + s2) << 23);
+    uint64_t t[NI];
+#pragma unroll
+    for (int i = 0; i < NI; i++)
+        t[i] = quant_exact(v[i].x, f1, f2, sigma) + quant_exact(v[i].y, f1, f2, sigma) +
+               quant_exact(v[i].z, f1, f2, sigma) + quant_exact(v[i].w, f1, f2, sigma);
+    // t[0] becomes the total of the 128 bins of read lane / GL
+    int o = 16;
+#pragma unroll
+    for (int w = NI / 2; w >= 1; w /= 2, o >>= 1)
+#pragma unroll
+        for (int k = 0; k < w; k++) {
+            const uint64_t keep = (lane & o) ? t[k + w] : t[k], send = (lane & o) ? t[k] : t[k + w];
+            t[k] = keep + __shfl_xor_sync(kAll, send, o);
+        }
+    for (; o > 0; o >>= 1) t[0] += __shfl_xor_sync(kAll, t[0], o);
+    uint64_t cum = t[0];                       // inclusive over the reads
+#pragma unroll
+    for (int w = GL; w < 32; w <<= 1) {
+        const uint64_t u = __shfl_up_sync(kAll, cum, w);
+        if (lane >= w) cum += u;
+    }
+    const uint64_t T = __shfl_sync(kAll, cum, 31);
+    if (T == 0) {   // zero-norm network: its shots cannot be drawn and are dropped
+        if (lane == 0) ndist[n] = 0;
+        return;
+    }
+    const uint64_t rank = (uint64_t)(rank0[n] + lane);
+    const uint64_t r_l =
+        __umul64hi(word64(philox4x32_10(make_uint4((uint32_t)rank, (uint32_t)(rank >> 32), (uint32_t)traj[n], tagw), key)), T);
+    int my_x = -1 - lane;                      // lanes without a draw match nobody
+    for (int k = 0; k < (int)c; k++) {
+        uint64_t r = __shfl_sync(kAll, r_l, k);
+        const int i = (__ffs(__ballot_sync(kAll, r < cum)) - 1) / GL;   // the read holding the draw
+        const uint64_t before = __shfl_sync(kAll, cum, i * GL - 1 < 0 ? 0 : i * GL - 1);
+        if (i) r -= before;
+        float4 q = p[32 * i];
+        const uint64_t q0 = quant_exact(q.x > 0.f ? q.x : 0.f, f1, f2, sigma);
+        const uint64_t q1 = q0 + quant_exact(q.y > 0.f ? q.y : 0.f, f1, f2, sigma);
+        const uint64_t q2 = q1 + quant_exact(q.z > 0.f ? q.z : 0.f, f1, f2, sigma);
+        const uint64_t q3 = q2 + quant_exact(q.w > 0.f ? q.w : 0.f, f1, f2, sigma);
+        const uint64_t inc = warp_incl_scan_u64(q3, lane);
+        const int l = __ffs(__ballot_sync(kAll, r < inc)) - 1;
+        const uint64_t d = r - (inc - q3);     // within lane l's four bins
+        const int x = __shfl_sync(kAll, 128 * i + 4 * lane + (d >= q0) + (d >= q1) + (d >= q2), l);
+        if (lane == k) my_x = x;
+    }
+    // distinct outcomes in increasing order with their counts
+    const unsigned peers = __match_any_sync(kAll, my_x);
+    const bool first = my_x >= 0 && __ffs(peers) - 1 == lane;
+    const unsigned firsts = __ballot_sync(kAll, first);
+    int pos = 0;
+    for (unsigned f = firsts; f; f &= f - 1) pos += __shfl_sync(kAll, my_x, __ffs(f) - 1) < my_x;
+    const int64_t q = tmp_off[n] + pos;
+    if (first && q < tmp_cap) {   // slots past tmp_cap are never written; the host reports the shortfall
+        tmp_x[q] = my_x;
+        tmp_c[q] = __popc(peers);
+    }
+    if (lane == 0) ndist[n] = __popc(firsts);
 }
 
 __global__ void k_emit_children(const int32_t* __restrict__ traj, const uint64_t* __restrict__ prefix,
@@ -604,9 +732,30 @@ int64_t run_sample_block(const float* marg, int b, int start, const int32_t* ptr
         if (b <= kSampWarpMaxBits) {
             // per warp: CDF (8 B) + histogram (4 B) per bin; 48 KB at 2^10 bins
             const size_t smem = (size_t)kSampWarps * (((size_t)1 << b) * (sizeof(uint64_t) + sizeof(unsigned)));
-            k_sample_parents_warp<<<(unsigned)((n_parent + kSampWarps - 1) / kSampWarps), kSampWarps * 32, smem, s>>>(
-                marg, b, n_parent, ptraj, pcount, sc.rank0, sc.tmp_off, child_cap, key,
-                philox_tag(STREAM_SAMPLE, circuit, block), sc.tmp_x, sc.tmp_c, sc.ndist);
+            const uint32_t tagw = philox_tag(STREAM_SAMPLE, circuit, block);
+            // rows of at least 128 bins on 16-byte boundaries: few-shot parents in registers
+            const bool few = b >= 7 && (reinterpret_cast<uintptr_t>(marg) & 15) == 0;
+            if (few) {
+                const unsigned grid = (unsigned)((n_parent + 7) / 8);
+                auto run = [&](auto kernel) {
+                    kernel<<<grid, 256, 0, s>>>(marg, b, n_parent, ptraj, pcount, sc.rank0, sc.tmp_off, child_cap, key,
+                                                tagw, sc.tmp_x, sc.tmp_c, sc.ndist);
+                };
+                count_launches(K_SAMPLE_PARENTS);
+                if (b == 7) run(k_sample_few<1>);
+                else if (b == 8) run(k_sample_few<2>);
+                else if (b == 9) run(k_sample_few<4>);
+                else run(k_sample_few<8>);
+            }
+            // the others: parents spread over all warp slots (four CTAs of 2^10 bins fit
+            // an SM), several per look only where few of them remain among many
+            const int64_t slots = 152 * 4 * kSampWarps;
+            const int grp = few ? (int)std::max<int64_t>(1, std::min<int64_t>(32, n_parent / slots)) : 1;
+            const int64_t per = (int64_t)grp * kSampWarps;
+            k_sample_parents_warp<<<(unsigned)std::min<int64_t>((n_parent + per - 1) / per, 152 * 16), kSampWarps * 32,
+                                    smem, s>>>(
+                marg, b, n_parent, ptraj, pcount, sc.rank0, sc.tmp_off, child_cap, key, tagw, sc.tmp_x, sc.tmp_c,
+                sc.ndist, few ? kFewShots : -1, grp);
         } else {
             const size_t smem = (size_t)(((int64_t)1 << b) * (sizeof(uint64_t) + sizeof(unsigned int)));
             if (smem > 32 * 1024)
