@@ -146,10 +146,15 @@ void launch_small_steps(const SmallRuns& sr, std::pair<int32_t, int32_t> parts, 
 void launch_contract_step(const StepDesc* d_step, const StepDesc& h_step, const ChunkCtx& ctx,
                           int64_t n_inst, cudaStream_t s);
 // marginal rows (real diagonal of the root) and their FP64 totals; part holds
-// n_net * finalize_tiles(b) doubles when finalize_tiles(b) > 1 (else unused)
+// n_net * finalize_tiles(b) doubles when finalize_tiles(b) > 1 (else unused);
+// rowmax (or null): zeroed, per row the bits of its largest entry
 int64_t finalize_tiles(int b);
-void launch_finalize(const RootRef* d_root, const ChunkCtx& ctx, int b, int64_t n_net, float* marg, double* Z,
-                     double* part, cudaStream_t s);
+// The block's closing elementwise or outer product, if the finalisation can form it from
+// its factors (prod, d_prod below: the step is then not launched).
+const StepDesc* closing_product(const BlockPlan& bp);
+void launch_finalize(const RootRef* d_root, const RootRef& root, const StepDesc* d_prod, const StepDesc* prod,
+                     const ChunkCtx& ctx, int b, int64_t n_net, float* marg, double* Z, double* part, unsigned* rowmax,
+                     cudaStream_t s);
 
 // ---- tensor-core steps (kernels_gemm.cu); err: device word set on a timeout
 // Networks of a chunk grouped by trajectory: group g holds networks
@@ -252,7 +257,8 @@ struct HarvestArgs {
     int circuit, block;
 };
 struct HarvestScratch {
-    unsigned* rowmax;           // [n_net]
+    unsigned* rowmax;           // [n_net] largest entries, from the finalisation
+    float* pmin;                // [n_net] smallest entry kept (exhaustive)
     unsigned long long* T;      // [n_net]
     uint64_t* tcdf;             // [n_net][harvest_cdf_tiles(b)] (direct)
     int64_t* tcnt;              // [n_net * harvest_tiles(b)]

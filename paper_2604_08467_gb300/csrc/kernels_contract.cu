@@ -911,57 +911,181 @@ bool launch_rows(const StepDesc* d_step, const StepDesc& h, const ChunkCtx& ctx,
     return true;
 }
 
-// marg[n][x] = Re(root_n[x]) (the double-layer diagonal), Z[n] = sum_x in FP64.
-// One block per (network, tile of kFinTile consecutive block outcomes x); a
-// thread takes kFinPer consecutive x and steps its root offset from x to x + 1
-// with delta[ctz(~x)] (delta[k] = stride[k] - sum of the strides below k).
-// Z is the FP64 sum of the tile (written directly when the block has one tile,
-// otherwise as a partial that k_finalize_sum adds in tile order).
-constexpr int kFinThreads = 256, kFinPer = 16, kFinTile = kFinThreads * kFinPer;
+// marg[n][x] = Re(root_n[x]) (the double-layer diagonal), or, where the block
+// ends with an elementwise or outer product (the ket-only form's |a(x)|^2, a
+// network whose last two parts share no bond), that product's real part formed
+// from the factors: the closing step is then not launched and its 8-byte
+// outputs are neither written nor read.  Z is the row's FP64 total; with
+// rowmax, the largest entry of every row is kept too.
+// A CTA takes units of 4096 outcomes (a tile of a wide block, or several
+// networks of a narrow one).  The root is read in the order of its memory
+// (outcome bits sorted by stride) and turned to outcome order in shared
+// memory, so reads and writes are both coalesced; one thread per 16 consecutive
+// outcomes read 8 bytes per 64-128 byte step, with 64 of 256 threads busy at
+// 2^10 outcomes (1.4 TB/s).  Z adds 16 consecutive outcomes per thread, a
+// shuffle tree per warp, the warps in order, the tiles in order; the 16 are
+// added as 64-bit integers scaled by the thread's largest entry (58 bits for
+// it, so the sum is closer than one of FP64 roundings), because this chip adds
+// two FP64 numbers per clock and SM.
+// Measured: 1.9 M rows of 2^10 outcomes 15.6 -> 10.0 ms with the closing |a|^2
+// (6.3 ms, 24.6 GB) gone; 24 rows of 2^28 outcomes, an outer product, 46.1 ms
+// and 13.2 ms for the product -> 22.5 ms.
+constexpr int kFinThreads = 256, kFinTileLog = 12, kFinTile = 1 << kFinTileLog;
+enum FinMode { FIN_ROOT = 0, FIN_SQUARE = 1, FIN_PRODUCT = 2 };
+struct FinArgs {
+    int32_t b, tb;                 // outcome bits; those within a unit (the rest number tiles)
+    int32_t n_it, net_log;         // elements per thread; log2 networks per unit
+    int32_t x_bit[kFinTileLog];    // outcome bit of element bit k
+    float s0, s1;                  // signs of the factors' imaginary parts
+    int64_t stride[2][kFinTileLog];   // operand strides of the element bits
+    int64_t hi_stride[2][32];         // of the outcome bits above tb
+    int64_t tiles, n_net, n_units;
+};
 
-__global__ void __launch_bounds__(kFinThreads) k_finalize(const RootRef* __restrict__ groot, const __grid_constant__ ChunkCtx c, int b,
-                                                          int64_t tiles, float* __restrict__ marg,
-                                                          double* __restrict__ Z, double* __restrict__ part) {
-    __shared__ __align__(16) RootRef r;
-    __shared__ int64_t delta[32];
-    __shared__ double red[kFinThreads / 32];
-    {
-        const int4* src = reinterpret_cast<const int4*>(groot);
-        int4* dst = reinterpret_cast<int4*>(&r);
-        for (int i = threadIdx.x; i < (int)(sizeof(RootRef) / sizeof(int4)); i += blockDim.x) dst[i] = src[i];
+// Sum of 16 floats of a thread.
+__device__ __forceinline__ double sum16(const float* v) {
+    float m = 0.f, a = 0.f;
+    for (int k = 0; k < 16; k++) {
+        m = fmaxf(m, fabsf(v[k]));
+        a += fabsf(v[k]);
     }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        int64_t below = 0;
-        for (int t = 0; t < (int)threadIdx.x && t < b; t++) below += r.x_stride[t];
-        delta[threadIdx.x] = (int)threadIdx.x < b ? r.x_stride[threadIdx.x] - below : 0;
-    }
-    __syncthreads();
-    const int64_t net = blockIdx.x / tiles, tile = blockIdx.x - net * tiles;
-    const float2* R = operand_ptr(r.op, CLS_NET, net, c);
-    const int64_t nx = (int64_t)1 << b;
-    int64_t x = tile * kFinTile + (int64_t)threadIdx.x * kFinPer;
     double acc = 0.0;
-    if (x < nx) {
-        int64_t off = 0;
-        for (int t = 0; t < b; t++)
-            if ((x >> t) & 1) off += r.x_stride[t];
-        float* out = marg + net * nx;
-        for (int k = 0; k < kFinPer && x < nx; k++, x++) {
-            const float v = R[off].x;
-            out[x] = v;
-            acc += (double)v;
-            off += delta[__ffsll(~x) - 1];
-        }
+    if (!(a <= 3.0e38f)) {         // NaN, infinite, or too large for the scale below
+        for (int k = 0; k < 16; k++) acc += (double)v[k];
+        return acc;
     }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < kFinThreads / 32; w++) t += red[w];
-        if (tiles == 1) Z[net] = t;
-        else part[blockIdx.x] = t;
+    if (m == 0.f) return 0.0;
+    const int s = 58 - frexp_exp(m), s1 = s / 2, s2 = s - s1;   // |s| <= 206
+    const float f1 = __int_as_float((127 + s1) << 23), f2 = __int_as_float((127 + s2) << 23);
+    int64_t t = 0;
+    for (int k = 0; k < 16; k++) t += __float2ll_rn(v[k] * f1 * f2);
+    return (double)t * __longlong_as_double((int64_t)(1023 - s) << 52);
+}
+
+template <int IT, int MODE>        // elements per thread (0: n_it, narrow blocks)
+__global__ void __launch_bounds__(kFinThreads) k_finalize(const OperandDesc* __restrict__ op0, const OperandDesc* __restrict__ op1,
+                                                          const __grid_constant__ ChunkCtx c,
+                                                          const __grid_constant__ FinArgs f, float* __restrict__ marg,
+                                                          double* __restrict__ Z, double* __restrict__ part,
+                                                          unsigned* __restrict__ rowmax) {
+    constexpr int NOP = MODE == FIN_PRODUCT ? 2 : 1;
+    __shared__ float sm[kFinTile + kFinTile / 16];   // outcome x at x + x / 16
+    __shared__ const float2* ptr[NOP][kFinThreads];
+    __shared__ int64_t it_off[NOP][16];
+    __shared__ int it_x[16];
+    __shared__ double red[kFinThreads / 32];
+    const int tid = threadIdx.x, n_it = IT ? IT : f.n_it, unit_log = f.tb + f.net_log;
+    // element e = it * 256 + tid: its bits below tb select the outcome in the
+    // order of the operands' memory, those above the network of the unit
+    auto place = [&](int e, int64_t* off, int& x) {
+        x = e >> f.tb << f.tb;
+#pragma unroll
+        for (int o = 0; o < NOP; o++) off[o] = 0;
+        for (int k = 0; k < f.tb; k++)
+            if ((e >> k) & 1) {
+#pragma unroll
+                for (int o = 0; o < NOP; o++) off[o] += f.stride[o][k];
+                x += 1 << f.x_bit[k];
+            }
+    };
+    int64_t off_t[NOP];
+    int x_t;
+    place(tid, off_t, x_t);
+    if (tid < 16) {
+        int64_t off[NOP];
+        place(tid << 8 & ((1 << unit_log) - 1), off, it_x[tid]);
+#pragma unroll
+        for (int o = 0; o < NOP; o++) it_off[o][tid] = off[o];
+    }
+    const int64_t nx = (int64_t)1 << f.b;
+    for (int64_t u = blockIdx.x; u < f.n_units; u += gridDim.x) {
+        const int64_t tile = u % f.tiles, net0 = (u / f.tiles) << f.net_log;
+        const int nets = (int)min((int64_t)1 << f.net_log, f.n_net - net0);
+        __syncthreads();           // the previous unit's addresses and outcomes are no longer read
+        if (tid < nets)
+#pragma unroll
+            for (int o = 0; o < NOP; o++) {
+                const float2* p = operand_ptr(o ? *op1 : *op0, CLS_NET, net0 + tid, c);
+                for (int t = f.tb; t < f.b; t++)
+                    if ((tile >> (t - f.tb)) & 1) p += f.hi_stride[o][t];
+                ptr[o][tid] = p;
+            }
+        __syncthreads();
+        const int valid = nets << f.tb;   // elements of the unit
+#pragma unroll
+        for (int it = 0; it < n_it; it++) {
+            const int e = it * kFinThreads + tid;
+            float v = 0.f;
+            if (e < valid) {
+                const float2 x = ptr[0][e >> f.tb][off_t[0] + it_off[0][it]];
+                if constexpr (MODE == FIN_ROOT) {
+                    v = x.x;
+                } else {
+                    float2 y = x;
+                    if constexpr (MODE == FIN_PRODUCT) y = ptr[NOP - 1][e >> f.tb][off_t[NOP - 1] + it_off[NOP - 1][it]];
+                    v = fmaf(-(f.s0 * x.y), f.s1 * y.y, fmaf(x.x, y.x, 0.f));   // as the SIMT kernels' single term
+                }
+            }
+            const int x = x_t + it_x[it];
+            sm[x + (x >> 4)] = v;
+        }
+        __syncthreads();
+        float* out = marg + net0 * nx + (tile << f.tb);
+#pragma unroll
+        for (int it = 0; it < n_it; it++) {
+            const int x = it * kFinThreads + tid;
+            if (x < valid) out[x] = sm[x + (x >> 4)];
+        }
+        // narrow blocks: threads past the last network drop out (whole trees of them)
+        const unsigned mask = __ballot_sync(0xffffffffu, f.tb >= 9 || 16 * tid < valid);
+        if (f.tb < 9 && 16 * tid >= valid) continue;
+        const float* row = sm + 17 * tid;
+        if (f.tb < 4) {            // several networks per thread
+            for (int g = 0; g < 16 >> f.tb && 16 * tid + (g << f.tb) < valid; g++) {
+                double acc = 0.0;
+                float m = 0.f;
+                for (int k = 0; k < 1 << f.tb; k++) {
+                    acc += (double)row[(g << f.tb) + k];
+                    m = fmaxf(m, row[(g << f.tb) + k]);
+                }
+                const int64_t net = net0 + (((16 * tid) >> f.tb) + g);
+                Z[net] = acc;
+                if (rowmax && m > 0.f) rowmax[net] = __float_as_uint(m);
+            }
+            continue;
+        }
+        double acc = 0.0;
+        float m = 0.f;
+        if (16 * tid < valid) {
+            float v[16];
+#pragma unroll
+            for (int k = 0; k < 16; k++) {
+                v[k] = row[k];
+                m = fmaxf(m, v[k]);
+            }
+            acc = sum16(v);
+        }
+        const int per = 1 << (f.tb - 4);                // threads per network
+        const int64_t net = net0 + tid / per;
+        const int width = per < 32 ? per : 32;
+        for (int o = width >> 1; o > 0; o >>= 1) {
+            acc += __shfl_down_sync(mask, acc, o, width);
+            m = fmaxf(m, __shfl_down_sync(mask, m, o, width));
+        }
+        const bool lead = (tid & (width - 1)) == 0 && 16 * tid < valid;
+        if (rowmax && lead && m > 0.f) atomicMax(&rowmax[net], __float_as_uint(m));
+        if (per <= 32) {
+            if (lead) Z[net] = acc;
+            continue;
+        }
+        if ((tid & 31) == 0) red[tid >> 5] = acc;
+        __syncthreads();
+        if (tid % per == 0 && 16 * tid < valid) {
+            double t = 0.0;
+            for (int w = 0; w < per / 32; w++) t += red[(tid >> 5) + w];
+            if (f.tiles == 1) Z[net] = t;
+            else part[net * f.tiles + tile] = t;
+        }
     }
 }
 
@@ -1158,14 +1282,81 @@ void launch_contract_step(const StepDesc* d_step, const StepDesc& h, const Chunk
 
 int64_t finalize_tiles(int b) { return (((int64_t)1 << b) + kFinTile - 1) / kFinTile; }
 
-void launch_finalize(const RootRef* d_root, const ChunkCtx& ctx, int b, int64_t n_net, float* marg, double* Z,
-                     double* part, cudaStream_t s) {
+const StepDesc* closing_product(const BlockPlan& bp) {
+    if (bp.steps.empty()) return nullptr;
+    const StepDesc& h = bp.steps.back();
+    const OperandDesc& r = bp.root.op;
+    if (h.kind != STEP_DIRECT || h.n_sum != 0 || h.virt || h.fuse_prev || bp.b != h.n_out || h.n_out > 30) return nullptr;
+    if (r.mode != OP_BUF || r.n_slice || r.arena != h.out_arena || r.arena_off != h.out_off || r.inst_size != h.out_size)
+        return nullptr;
+    for (int t = 0; t < bp.b; t++) {
+        const int64_t v = bp.root.x_stride[t];
+        if (v <= 0 || (v & (v - 1)) || v >= h.out_size) return nullptr;
+    }
+    return &h;
+}
+
+void launch_finalize(const RootRef* d_root, const RootRef& root, const StepDesc* d_prod, const StepDesc* prod,
+                     const ChunkCtx& ctx, int b, int64_t n_net, float* marg, double* Z, double* part, unsigned* rowmax,
+                     cudaStream_t s) {
     if (n_net <= 0) return;
-    const int64_t tiles = finalize_tiles(b);
-    StatScope sc(K_FINALIZE, s, (double)n_net * (double)(1ll << b) * 12.0, 0.0);
-    k_finalize<<<(unsigned)(n_net * tiles), kFinThreads, 0, s>>>(d_root, ctx, b, tiles, marg, Z, part);
-    if (tiles > 1) count_launches(K_FINALIZE);
-    if (tiles > 1) k_finalize_sum<<<(unsigned)((n_net + 127) / 128), 128, 0, s>>>(part, tiles, n_net, Z);
+    FinArgs f;
+    memset(&f, 0, sizeof f);
+    f.b = b;
+    f.tb = std::min(b, kFinTileLog);
+    f.net_log = std::min(kFinTileLog - f.tb, 8);
+    f.n_it = std::max(1, 1 << (f.tb + f.net_log) >> 8);
+    f.n_net = n_net;
+    f.tiles = finalize_tiles(b);
+    f.n_units = ((n_net + (1ll << f.net_log) - 1) >> f.net_log) * f.tiles;
+    f.s0 = f.s1 = 1.f;
+    int mode = FIN_ROOT;
+    const OperandDesc *op0 = &d_root->op, *op1 = op0;
+    if (prod) {
+        const OperandDesc &p = prod->op[0], &q = prod->op[1];
+        bool same = p.mode == OP_BUF && q.mode == OP_BUF && !p.n_slice && !q.n_slice && p.arena == q.arena &&
+                    p.cls == q.cls && p.arena_off == q.arena_off && p.inst_size == q.inst_size && p.cache == q.cache;
+        for (int t = 0; t < prod->n_out; t++) same = same && prod->out_stride[0][t] == prod->out_stride[1][t];
+        mode = same ? FIN_SQUARE : FIN_PRODUCT;
+        op0 = &d_prod->op[0];
+        op1 = &d_prod->op[1];
+        f.s0 = p.conj ? -1.f : 1.f;
+        f.s1 = q.conj ? -1.f : 1.f;
+    }
+    // stride of outcome bit t in the root, or in a factor of the closing product
+    auto stride = [&](int o, int t) {
+        const int64_t v = root.x_stride[t];
+        return prod ? prod->out_stride[o][__builtin_ctzll((unsigned long long)v)] : v;
+    };
+    // element order: along the larger operand's memory, then the other's bits
+    const int big = mode == FIN_PRODUCT && prod->op[1].inst_size >> prod->op[1].n_slice > prod->op[0].inst_size >> prod->op[0].n_slice;
+    int order[kFinTileLog];
+    for (int t = 0; t < f.tb; t++) order[t] = t;
+    auto key = [&](int t) {
+        const int64_t v = stride(big, t);
+        return v ? v : ((int64_t)1 << 40) + stride(1 - big, t);
+    };
+    std::sort(order, order + f.tb, [&](int x, int y) { return key(x) < key(y); });
+    for (int k = 0; k < f.tb; k++) {
+        f.x_bit[k] = order[k];
+        for (int o = 0; o < 2; o++) f.stride[o][k] = stride(o, order[k]);
+    }
+    for (int t = f.tb; t < b; t++)
+        for (int o = 0; o < 2; o++) f.hi_stride[o][t] = stride(o, t);
+    StatScope sc(K_FINALIZE, s, (double)n_net * (double)(1ll << b) * (mode == FIN_PRODUCT ? 4.0 : 12.0), 0.0);
+    const unsigned grid = (unsigned)std::min<int64_t>(f.n_units, 152 * 8);
+    auto run = [&](auto kernel) { kernel<<<grid, kFinThreads, 0, s>>>(op0, op1, ctx, f, marg, Z, part, rowmax); };
+    if (f.n_it == 16) {
+        if (mode == FIN_ROOT) run(k_finalize<16, FIN_ROOT>);
+        else if (mode == FIN_SQUARE) run(k_finalize<16, FIN_SQUARE>);
+        else run(k_finalize<16, FIN_PRODUCT>);
+    } else {
+        if (mode == FIN_ROOT) run(k_finalize<0, FIN_ROOT>);
+        else if (mode == FIN_SQUARE) run(k_finalize<0, FIN_SQUARE>);
+        else run(k_finalize<0, FIN_PRODUCT>);
+    }
+    if (f.tiles > 1) count_launches(K_FINALIZE);
+    if (f.tiles > 1) k_finalize_sum<<<(unsigned)((n_net + 127) / 128), 128, 0, s>>>(part, f.tiles, n_net, Z);
 }
 
 }  // namespace ptn

@@ -134,7 +134,7 @@ struct PlanWorkspace {
     DevBuf ev_steps, ev_bwd, ev_root, ev_pl, ev_dvt, ev_terms, ev_F, ev_partial, ev_iota;
     DevBuf zpart;                         // per-tile partial totals of large marginal rows
     // final-block harvest of non-proportional sampling
-    DevBuf h_rowmax, h_T, h_tcdf, h_tcnt, h_toff, h_scan, h_cnt, h_rank0, h_first;
+    DevBuf h_rowmax, h_pmin, h_T, h_tcdf, h_tcnt, h_toff, h_scan, h_cnt, h_rank0, h_first;
     // intermediate caching: key halves, hash tables, representatives, lists, counts
     DevBuf c_h, c_keys, c_first, c_rep, c_list, c_cnt;
     HostBuf h_traj, h_chunk_traj, h_net_tl, h_small, h_grp, h_ccnt;
@@ -157,7 +157,7 @@ struct PlanWorkspace {
                          &s_tmp_c, &s_scan, &zero_prefix, &pack[0], &pack[1], &err, &grp, &grp_cnt,
                          &grp_tile0, &grp_scan, &arena_x[0], &arena_x[1], &ev_steps,
                          &ev_bwd, &ev_root, &ev_pl, &ev_dvt, &ev_terms, &ev_F, &ev_partial, &ev_iota, &zpart,
-                         &h_rowmax, &h_T, &h_tcdf, &h_tcnt, &h_toff, &h_scan, &h_cnt, &h_rank0, &h_first,
+                         &h_rowmax, &h_pmin, &h_T, &h_tcdf, &h_tcnt, &h_toff, &h_scan, &h_cnt, &h_rank0, &h_first,
                          &c_h, &c_keys, &c_first, &c_rep, &c_list, &c_cnt};
         for (DevBuf* b : all) b->release();
         h_grp.release();
@@ -360,7 +360,7 @@ ptn_status ensure_nz(const ptn_traj* ctr, cudaStream_t s) {
 // Contract n_net networks of block j; marg/Z outputs are device arrays.
 ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const int32_t* d_net_traj,
                           const uint64_t* d_net_prefix, int64_t n_net, float* marg, double* Z, int max_traj_chunk,
-                          int precision, cudaStream_t s, bool graphs = false) {
+                          int precision, cudaStream_t s, bool graphs = false, unsigned* rowmax = nullptr) {
     if (n_net <= 0) return PTN_OK;
     if (precision != PTN_PREC_FP32 && precision != PTN_PREC_BF16X3 && precision != PTN_PREC_FP16X3)
         return set_error(PTN_ERR_INVALID_ARG, "unknown precision mode %d", precision);
@@ -479,6 +479,7 @@ ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const
     }
     PTN_CUDA(cudaMemsetAsync(ws->err.p, 0, sizeof(int), s));
     const RootRef* d_root = plan->d_roots + j;
+    const StepDesc* closing = closing_product(bp);
     if (graphs) {
         if (!ws->cap_stream) PTN_CUDA(cudaStreamCreateWithFlags(&ws->cap_stream, cudaStreamNonBlocking));
         if (ws->gexec.size() < plan->blocks.size()) ws->gexec.resize(plan->blocks.size(), nullptr);
@@ -554,7 +555,7 @@ ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const
         }
         for (size_t st = 0; st < bp.steps.size(); st++) {
             const StepDesc& h = bp.steps[st];
-            if (h.virt) continue;   // formed inside its consumer's operand pack
+            if (h.virt || &h == closing) continue;   // formed inside its consumer's operand pack, the finalisation
             StepTag tag(j, (int)st);
             if (const int len = launch_small_run(bp.small, bp.steps, st, plan->opts.fuse_max, ctx, c.n_traj, ls)) {
                 st += len - 1;
@@ -575,8 +576,9 @@ ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const
         }
         {
             StepTag tag(j, (int)bp.steps.size());
-            launch_finalize(d_root, ctx, bp.b, c.n_net, marg + c.net0 * ((int64_t)1 << bp.b), Z + c.net0,
-                            ws->zpart.as<double>(), ls);
+            launch_finalize(d_root, bp.root, bp.d_steps + bp.steps.size() - 1, closing, ctx, bp.b, c.n_net,
+                            marg + c.net0 * ((int64_t)1 << bp.b), Z + c.net0, ws->zpart.as<double>(),
+                            rowmax ? rowmax + c.net0 : nullptr, ls);
         }
         if (graphs) {
             // the block's executable graph takes the new chunk's parameters in
@@ -1434,6 +1436,7 @@ static ptn_status sample_nonprop(const ptn_plan* plan, const ptn_traj* traj, con
     if (n > 0) {
         if ((e = ws->marg.grow(sizeof(float) * sub * nx)) || (e = ws->Z.grow(sizeof(double) * sub)) ||
             (e = ws->h_rowmax.grow(sizeof(unsigned) * sub)) || (e = ws->h_T.grow(sizeof(uint64_t) * sub)) ||
+            (e = ws->h_pmin.grow(sizeof(float) * sub)) ||
             (e = ws->h_tcnt.grow(sizeof(int64_t) * sub * tiles)) || (e = ws->h_toff.grow(sizeof(int64_t) * sub * tiles)) ||
             (e = ws->h_scan.grow(sizeof(int64_t) * scan_tmp_elems(sub * tiles))))
             return e;
@@ -1444,6 +1447,7 @@ static ptn_status sample_nonprop(const ptn_plan* plan, const ptn_traj* traj, con
     HarvestScratch hs;
     hs.rowmax = ws->h_rowmax.as<unsigned>();
     hs.T = ws->h_T.as<unsigned long long>();
+    hs.pmin = ws->h_pmin.as<float>();
     hs.tcdf = ws->h_tcdf.as<uint64_t>();
     hs.tcnt = ws->h_tcnt.as<int64_t>();
     hs.toff = ws->h_toff.as<int64_t>();
@@ -1469,8 +1473,9 @@ static ptn_status sample_nonprop(const ptn_plan* plan, const ptn_traj* traj, con
     int64_t total = 0;
     for (int64_t a = 0; a < n; a += sub) {
         const int64_t m = std::min(sub, n - a);
+        cudaMemsetAsync(hs.rowmax, 0, sizeof(unsigned) * m, s);
         e = contract_level(plan, traj, jf, ftraj + a, fprefix + a * W, m, ws->marg.as<float>(), ws->Z.as<double>(),
-                           o->max_traj_per_chunk, o->precision, s, o->use_graphs != 0);
+                           o->max_traj_per_chunk, o->precision, s, o->use_graphs != 0, hs.rowmax);
         if (e) {
             free_parts();
             return e;
