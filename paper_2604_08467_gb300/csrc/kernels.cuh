@@ -140,9 +140,9 @@ struct CacheArgs {
 void launch_cache_tables(const CacheArgs& a, cudaStream_t s);
 
 // ---- launchers (kernels_contract.cu)
-// a run of small trajectory-class steps (small_step, fuse_prev) in one launch
+// a run of small steps of one class (fusable_step, fuse_prev) in one launch
 void launch_small_steps(const SmallRuns& sr, std::pair<int32_t, int32_t> parts, const StepDesc* h_steps, int n_steps,
-                        const ChunkCtx& ctx, int64_t n_traj, cudaStream_t s);
+                        const ChunkCtx& ctx, int64_t n_inst, cudaStream_t s);
 void launch_contract_step(const StepDesc* d_step, const StepDesc& h_step, const ChunkCtx& ctx,
                           int64_t n_inst, cudaStream_t s);
 // marginal rows (real diagonal of the root) and their FP64 totals; part holds

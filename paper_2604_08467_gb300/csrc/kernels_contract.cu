@@ -1115,12 +1115,16 @@ __global__ void k_finalize_sum(const double* __restrict__ part, int64_t tiles, i
 // Measured against the walk with two barriers and a 2.7 KB descriptor per
 // step: 689 steps of the last 30-qubit block, 131 trajectories 1.67 -> 0.09 ms;
 // 731 steps of the first, 4096 trajectories 8.2 -> 2.6 ms.
+// Runs of network-level steps (blocks lowered class by class) go the same way,
+// one CTA per network: a 100-qubit block's network, 203 launches 1.24 ms -> 2
+// launches and the finalisation 0.13 ms.
 struct SmallArgs {
     const SmallStep* steps;
     const SmallEnt* ent;
     const int32_t* lvl;
     const uint32_t* ktab;
-    int32_t n_steps, n_lvl;
+    const SmallSlice* slices;
+    int32_t n_steps, n_lvl, cls;
 };
 struct SmallRes {
     const float2 *A, *B;
@@ -1129,16 +1133,23 @@ struct SmallRes {
     int32_t ktab;
 };
 
-__device__ __forceinline__ const float2* small_operand(const SmallOp& d, int64_t tl, const ChunkCtx& c) {
+__device__ __forceinline__ const float2* small_operand(const SmallOp& d, int64_t tl, int64_t net,
+                                                       const SmallSlice* slices, const ChunkCtx& c) {
+    int64_t off = 0;
+    if (d.n_slice) {
+        const uint64_t* pre = c.net_prefix + net * c.n_words;
+        for (int s = 0; s < d.n_slice; s++)
+            off += (int64_t)bits_get(pre, slices[d.slice0 + s].qubit) * slices[d.slice0 + s].stride;
+    }
     if (d.src < 0) {
         int64_t var = 0;
         if (d.col >= 0) var = c.var_ids[(int64_t)c.chunk_traj[tl] * c.n_var_cols + d.col];
-        return c.vtab + d.base + var * d.size;
+        return c.vtab + d.base + var * d.size + off;
     }
-    int64_t oi = 0;
+    int64_t oi = d.inst == CLS_NET ? net : 0;
     if (d.inst == CLS_TRAJ)
         oi = (d.cache > 0 && c.cache_rep) ? (int64_t)c.cache_rep[(int64_t)(d.cache - 1) * c.cache_n + tl] : tl;
-    return c.arena[d.src] + d.base * c.arena_inst[d.src] + oi * d.size;
+    return c.arena[d.src] + d.base * c.arena_inst[d.src] + oi * d.size + off;
 }
 
 __device__ __forceinline__ void small_term(float2& acc, const float2 x, const float2 y, float sa, float sb) {
@@ -1152,10 +1163,10 @@ __device__ __forceinline__ void small_term(float2& acc, const float2 x, const fl
 __global__ void __launch_bounds__(1024) k_small_steps(const SmallArgs a, const __grid_constant__ ChunkCtx c) {
     extern __shared__ __align__(16) uint8_t small_smem[];
     SmallRes* res = reinterpret_cast<SmallRes*>(small_smem);
-    const int64_t tl = blockIdx.x;
+    const int64_t inst = blockIdx.x, tl = a.cls == CLS_NET ? (int64_t)c.net_tl[inst] : inst;
     for (int t = threadIdx.x; t < 2 * a.n_steps; t += blockDim.x) {
         const SmallStep& s = a.steps[t >> 1];
-        const float2* p = small_operand(s.op[t & 1], tl, c);
+        const float2* p = small_operand(s.op[t & 1], tl, inst, a.slices, c);
         SmallRes& r = res[t >> 1];
         if (t & 1) {
             r.B = p;
@@ -1163,7 +1174,7 @@ __global__ void __launch_bounds__(1024) k_small_steps(const SmallArgs a, const _
             r.ktab = s.ktab;
         } else {
             r.A = p;
-            r.out = c.arena[s.out_arena] + s.out_off * c.arena_inst[s.out_arena] + tl * s.out_size;
+            r.out = c.arena[s.out_arena] + s.out_off * c.arena_inst[s.out_arena] + inst * s.out_size;
         }
     }
     int e1 = a.lvl[0];
@@ -1202,24 +1213,27 @@ __global__ void __launch_bounds__(1024) k_small_steps(const SmallArgs a, const _
 }  // namespace
 
 void launch_small_steps(const SmallRuns& sr, std::pair<int32_t, int32_t> parts, const StepDesc* h_steps, int n_steps,
-                        const ChunkCtx& ctx, int64_t n_traj, cudaStream_t s) {
-    if (n_steps <= 0 || n_traj <= 0) return;
+                        const ChunkCtx& ctx, int64_t n_inst, cudaStream_t s) {
+    if (n_steps <= 0 || n_inst <= 0) return;
     double bytes = 0.0, flops = 0.0;
     for (int k = 0; k < n_steps; k++) {
         const StepDesc& h = h_steps[k];
-        bytes += 8.0 * (double)n_traj * (double)(h.out_size + h.op[0].inst_size + h.op[1].inst_size);
-        flops += 8.0 * (double)n_traj * (double)h.out_size * (double)(1ll << h.n_sum);
+        bytes += 8.0 * (double)n_inst * (double)(h.out_size + h.op[0].inst_size + h.op[1].inst_size);
+        flops += 8.0 * (double)n_inst * (double)h.out_size * (double)(1ll << h.n_sum);
     }
     StatScope sc(K_CONTRACT_SMALL, s, bytes, flops);
-    // up to one trajectory per SM: the levels' elements over as many threads as a
-    // CTA has (latency); more trajectories: smaller CTAs, several per SM, so that
-    // one's barriers and address chains overlap another's arithmetic
-    const int threads = n_traj <= 152 ? 1024 : (n_traj <= 304 ? 512 : 256);
+    // up to one instance per SM: the levels' elements over as many threads as a
+    // CTA has (latency); more of them: smaller CTAs, several per SM, so that
+    // one's barriers and address chains overlap another's arithmetic.  A
+    // network's levels have tens of elements.
+    const bool net = h_steps[0].out_cls == CLS_NET;
+    const int threads = n_inst <= 152 ? (net ? 512 : 1024) : (n_inst <= 304 ? (net ? 256 : 512) : (net ? 64 : 256));
     for (int p = parts.first; p < parts.second; p++) {
         const SmallPart& pt = sr.parts[p];
-        const SmallArgs a{sr.d_steps + pt.step0, sr.d_ent, sr.d_lvl + pt.lvl0, sr.d_ktab, pt.n_steps, pt.n_lvl};
+        const SmallArgs a{sr.d_steps + pt.step0, sr.d_ent, sr.d_lvl + pt.lvl0, sr.d_ktab, sr.d_slices,
+                          pt.n_steps, pt.n_lvl, pt.cls};
         if (p > parts.first) count_launches(K_CONTRACT_SMALL);
-        k_small_steps<<<(unsigned)n_traj, threads, sizeof(SmallRes) * pt.n_steps, s>>>(a, ctx);
+        k_small_steps<<<(unsigned)n_inst, threads, sizeof(SmallRes) * pt.n_steps, s>>>(a, ctx);
     }
 }
 

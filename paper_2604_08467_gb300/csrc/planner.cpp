@@ -561,8 +561,8 @@ struct ArenaAlloc {   // first-fit offsets of live buffers in one arena
 // same arena read or written earlier in the run, or one of its operands
 // overlaps, without coinciding, an output written earlier in the run.  A
 // coinciding range holds the same instance at the same addresses, which only
-// the CTA of that instance touches, in order.
-static void mark_fusable_runs(std::vector<StepDesc>& steps) {
+// the CTA of that instance touches, in order.  A run stays within one class.
+static void mark_fusable_runs(std::vector<StepDesc>& steps, bool by_class = false) {
     struct Rng {
         int32_t arena;
         int64_t off, size;
@@ -580,7 +580,7 @@ static void mark_fusable_runs(std::vector<StepDesc>& steps) {
     for (size_t i = 0; i < steps.size(); i++) {
         StepDesc& st = steps[i];
         st.fuse_prev = 0;
-        if (!small_step(st)) {
+        if (!fusable_step(st, by_class)) {
             touched.clear();
             continue;
         }
@@ -588,7 +588,8 @@ static void mark_fusable_runs(std::vector<StepDesc>& steps) {
         std::vector<Rng> ins;
         for (const OperandDesc& d : st.op)
             if (d.mode == OP_BUF) ins.push_back({d.arena, d.arena_off, d.inst_size, false});
-        bool join = i > 0 && small_step(steps[i - 1]) && !clash(out, true);
+        bool join = i > 0 && fusable_step(steps[i - 1], by_class) && steps[i - 1].out_cls == st.out_cls &&
+                    !clash(out, true);
         for (const Rng& r : ins) join = join && !clash(r, false);
         if (!join) touched.clear();
         st.fuse_prev = join ? 1 : 0;
@@ -681,7 +682,7 @@ static void mark_pack_products(BlockPlan& bp, int fuse_max) {
             if (prod_of[g][x] < 0 || G.op[x].n_slice) continue;
             const size_t k = (size_t)prod_of[g][x];
             StepDesc& P = bp.steps[k];
-            const bool fused = fuse_max > 1 && small_step(P) && (P.fuse_prev || (k + 1 < n && bp.steps[k + 1].fuse_prev));
+            const bool fused = fuse_max > 1 && fusable_step(P, bp.by_class) && (P.fuse_prev || (k + 1 < n && bp.steps[k + 1].fuse_prev));
             if (P.kind != STEP_DIRECT || P.n_sum != 0 || P.virt || fused) continue;
             if (P.op[0].inst_size > (1ll << 31) || P.op[1].inst_size > (1ll << 31)) continue;
             bool clash = false;
@@ -704,8 +705,10 @@ static void mark_pack_products(BlockPlan& bp, int fuse_max) {
 // state with every qubit open; the forward intermediates are kept (all of
 // them, or with checkpointing those crossing a segment boundary) and the
 // reversed (adjoint) path is lowered too, see the end.
+constexpr double kByClassBytes = 1 << 20;
 static ptn_status lower_block(const ptn_plan* plan, const BlockNet& net, const Searcher& s,
-                              int32_t start, int32_t b, BlockPlan& bp, bool expval = false) {
+                              int32_t start, int32_t b, BlockPlan& bp, bool expval = false, bool by_class = false) {
+    bp.by_class = by_class;
     struct Rec {
         TRef a, b, c;
     };
@@ -794,6 +797,7 @@ static ptn_status lower_block(const ptn_plan* plan, const BlockNet& net, const S
     // a released slot is not reused before the run ends: the slot's other
     // instances may still be read by other CTAs (mark_fusable_runs).
     bool in_run = false;
+    int32_t run_cls = -1;
     std::vector<std::pair<int32_t, int64_t>> deferred;
     auto release = [&](int32_t arena, int64_t off) {
         if (in_run) deferred.push_back({arena, off});
@@ -849,7 +853,19 @@ static ptn_status lower_block(const ptn_plan* plan, const BlockNet& net, const S
     };
 
     std::string summary;
-    for (const Move& mv : s.moves) {
+    // by_class: the moves of the path class by class (an operand's class is never
+    // above its result's, so this order is as valid as the path's own)
+    std::vector<const Move*> moves;
+    for (const Move& mv : s.moves) moves.push_back(&mv);
+    if (by_class)
+        std::stable_sort(moves.begin(), moves.end(), [&](const Move* x, const Move* y) {
+            // (a slice is a view: it follows the tensor it views)
+            const int cx = (int)s.t[x->type == MV_SLICE ? x->a : x->c].cls;
+            const int cy = (int)s.t[y->type == MV_SLICE ? y->a : y->c].cls;
+            return cx < cy;
+        });
+    for (const Move* pmv : moves) {
+        const Move& mv = *pmv;
         if (mv.type == MV_SLICE) {
             ref[mv.c] = ref[mv.a];       // a view: same storage, NET addressing when consumed
             if (mv.mc >= 0) ref[mv.mc] = ref[mv.ma];
@@ -924,12 +940,13 @@ static ptn_status lower_block(const ptn_plan* plan, const BlockNet& net, const S
         classify_step(st, pf, !plan->opts.simt_only);
         for (int r = 0; r < 2; r++)
             for (int k = 0; k < 3; k++) bp.pack_peak[r][k] = std::max(bp.pack_peak[r][k], pf[r][k]);
-        if (!small_step(st)) end_run();
+        if (!fusable_step(st, by_class) || st.out_cls != run_cls) end_run();
         // output buffer: allocate before releasing the operands
         BufInfo bi;
         bi.arena = C.cls;
         bi.off = arenas[C.cls].alloc(st.out_size);
-        in_run = small_step(st);
+        in_run = fusable_step(st, by_class);
+        run_cls = st.out_cls;
         bi.refs = mv.mc >= 0 ? 2 : 1;
         int32_t bid = (int32_t)bufs.size();
         bufs.push_back(bi);
@@ -1000,11 +1017,12 @@ static ptn_status lower_block(const ptn_plan* plan, const BlockNet& net, const S
         classify_step(st, pf, !plan->opts.simt_only);
         for (int r = 0; r < 2; r++)
             for (int k = 0; k < 3; k++) bp.pack_peak[r][k] = std::max(bp.pack_peak[r][k], pf[r][k]);
-        if (!small_step(st)) end_run();
+        if (!fusable_step(st, by_class) || st.out_cls != run_cls) end_run();
         BufInfo bi;
         bi.arena = cls;
         bi.off = arenas[cls].alloc(st.out_size);
-        in_run = small_step(st);
+        in_run = fusable_step(st, by_class);
+        run_cls = st.out_cls;
         bi.refs = 1;
         const int32_t bid = (int32_t)bufs.size();
         bufs.push_back(bi);
@@ -1030,7 +1048,7 @@ static ptn_status lower_block(const ptn_plan* plan, const BlockNet& net, const S
         R = rn;
     }
     end_run();
-    mark_fusable_runs(bp.steps);
+    mark_fusable_runs(bp.steps, by_class);
     ptn_status e = make_op(R, CLS_NET, bp.root.op);
     if (e) return e;
     for (int tb = 0; tb < b; tb++) bp.root.x_stride[tb] = -1;
@@ -1393,8 +1411,31 @@ static ptn_status search_and_lower(ptn_plan* plan, BlockNet& net, int j, int sta
     bp.est_time = best.time;
     bp.est_mult_traj = E;
     bp.est_mult_net = D;
+    BlockPlan alt = bp;
     ptn_status e = lower_block(plan, net, best, start, b, bp, expval);
     if (e) return e;
+    // A block of small tensors is bound by its launches: a path that goes back
+    // and forth between trajectory and network level cuts the fused runs (44
+    // runs and 159 single network steps for a 100-qubit block of the paper's
+    // family).  Listed class by class its small steps form one run per class.
+    // Buffers then live longer, so this is done only while a trajectory's take
+    // at most kByClassBytes, a network's grow by no more than a sixteenth of
+    // that, and a memory cap the caller set still holds what it held.
+    if (!expval && plan->opts.fuse_max > 1) {
+        auto bytes = [](const BlockPlan& p, int k) {
+            return 8.0 * (double)p.arena_peak[k] + 4.0 * (double)(p.pack_peak[0][k] + p.pack_peak[1][k]);
+        };
+        auto one_network = [&](const BlockPlan& p) { return bytes(p, 0) + bytes(p, 1) + bytes(p, 2) + 12.0; };
+        int n_net = 0;
+        for (const StepDesc& st : bp.steps) n_net += small_net_step(st);
+        if (n_net > 1 && bytes(bp, CLS_TRAJ) <= kByClassBytes &&
+            lower_block(plan, net, best, start, b, alt, false, true) == PTN_OK) {
+            const double cap = plan->opts.mem_cap_bytes;
+            if (bytes(alt, CLS_TRAJ) <= kByClassBytes && bytes(alt, CLS_NET) <= bytes(bp, CLS_NET) + kByClassBytes / 16 &&
+                (cap <= 0 || one_network(alt) <= cap || one_network(bp) > cap))
+                bp = std::move(alt);
+        }
+    }
     char buf[256];
     snprintf(buf, sizeof buf, "steps=%zu max_rank=%lld est_time=%.3es", bp.steps.size(), (long long)best.max_rank,
              best.time);

@@ -104,6 +104,9 @@ inline bool small_step(const StepDesc& h) {
 
 // Fused runs as k_small_steps executes them (small_runs.cpp): compact steps,
 // the output elements of every level, and summed-offset tables.
+struct SmallSlice {          // projected bit of a network-level step's operand
+    int32_t qubit, stride;
+};
 struct SmallOp {
     int64_t base;            // leaf: element of variant 0 in the variant table; buffer: arena offset per instance
     int32_t size;            // elements per variant / instance
@@ -111,6 +114,7 @@ struct SmallOp {
     int32_t inst;            // buffer: storage class (CLS_CONST: one instance)
     int32_t col;             // leaf: variant column, -1 = single variant
     int32_t cache;           // as OperandDesc.cache
+    int32_t slice0, n_slice; // its slices in SmallRuns.slices
     int32_t pad;
 };
 struct SmallStep {
@@ -128,6 +132,7 @@ struct SmallEnt {
 };
 struct SmallPart {           // at most kSmallPartSteps steps of a run: one launch
     int32_t step0, n_steps, lvl0, n_lvl;
+    int32_t cls;             // instances: trajectories or networks
 };
 constexpr int kSmallPartSteps = 1024;
 struct SmallRuns {
@@ -137,12 +142,25 @@ struct SmallRuns {
     std::vector<SmallEnt> ent;
     std::vector<int32_t> lvl;    // per part n_lvl + 1 entry positions
     std::vector<uint32_t> ktab;
+    std::vector<SmallSlice> slices;
     // device copies
     SmallStep* d_steps = nullptr;
     SmallEnt* d_ent = nullptr;
     int32_t* d_lvl = nullptr;
     uint32_t* d_ktab = nullptr;
+    SmallSlice* d_slices = nullptr;
 };
+
+// Network-level steps of blocks lowered class by class (BlockPlan.by_class)
+// that run fused, one CTA per network: at most 2^kSmallNetBits multiply-adds
+// (products without summed bits among them).
+constexpr int kSmallNetBits = 12;
+inline bool small_net_step(const StepDesc& h) {
+    return h.kind == STEP_DIRECT && h.out_cls == CLS_NET && h.n_sum <= kSmallSumBits &&
+           h.n_out + h.n_sum <= kSmallNetBits && h.op[0].inst_size <= (1ll << kSmallOpBits) &&
+           h.op[1].inst_size <= (1ll << kSmallOpBits);
+}
+inline bool fusable_step(const StepDesc& h, bool by_class) { return small_step(h) || (by_class && small_net_step(h)); }
 
 struct LeafInfo {
     int32_t gate;            // source gate, -1 for a |0> state
@@ -190,6 +208,7 @@ static_assert(sizeof(RootRef) % 16 == 0, "RootRef must be a multiple of 16 bytes
 struct BlockPlan {
     int32_t start = 0, b = 0;
     int32_t ket_only = 0;                // sampling block lowered in the ket-only network form
+    int32_t by_class = 0;                // steps listed class by class: constant, trajectory, network level
     std::vector<StepDesc> steps;
     RootRef root;
     int64_t arena_peak[N_ARENAS] = {0, 0, 0, 0, 0};   // elements per instance, per arena

@@ -211,7 +211,9 @@ ptn_status upload_small_runs(SmallRuns& sr) {
         return PTN_OK;
     };
     ptn_status e;
-    if ((e = up(sr.ent, &sr.d_ent)) || (e = up(sr.lvl, &sr.d_lvl)) || (e = up(sr.ktab, &sr.d_ktab))) return e;
+    if ((e = up(sr.ent, &sr.d_ent)) || (e = up(sr.lvl, &sr.d_lvl)) || (e = up(sr.ktab, &sr.d_ktab)) ||
+        (e = up(sr.slices, &sr.d_slices)))
+        return e;
     return up(sr.steps, &sr.d_steps);
 }
 void free_small_runs(SmallRuns& sr) {
@@ -219,14 +221,15 @@ void free_small_runs(SmallRuns& sr) {
     cudaFree(sr.d_ent);
     cudaFree(sr.d_lvl);
     cudaFree(sr.d_ktab);
+    cudaFree(sr.d_slices);
 }
 // Launches the fused run starting at step k, if one does; the number of steps it covers, else 0.
 int launch_small_run(const SmallRuns& sr, const std::vector<StepDesc>& steps, size_t k, int fuse_max,
-                     const ChunkCtx& ctx, int64_t n_traj, cudaStream_t s) {
+                     const ChunkCtx& ctx, int64_t n_inst, cudaStream_t s) {
     const auto it = sr.run_at.find((int32_t)k);
     if (it == sr.run_at.end()) return 0;
     const int len = small_run_len(steps, k, fuse_max);
-    launch_small_steps(sr, it->second, &steps[k], len, ctx, n_traj, s);
+    launch_small_steps(sr, it->second, &steps[k], len, ctx, n_inst, s);
     return len;
 }
 
@@ -557,7 +560,8 @@ ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const
             const StepDesc& h = bp.steps[st];
             if (h.virt || &h == closing) continue;   // formed inside its consumer's operand pack, the finalisation
             StepTag tag(j, (int)st);
-            if (const int len = launch_small_run(bp.small, bp.steps, st, plan->opts.fuse_max, ctx, c.n_traj, ls)) {
+            if (const int len = launch_small_run(bp.small, bp.steps, st, plan->opts.fuse_max, ctx,
+                                                 h.out_cls == CLS_NET ? c.n_net : c.n_traj, ls)) {
                 st += len - 1;
                 continue;
             }

@@ -1,5 +1,5 @@
-// Dataflow schedule of the fused runs of small trajectory-class steps
-// (k_small_steps): host side, made once per plan.
+// Dataflow schedule of the fused runs of small steps (k_small_steps): host
+// side, made once per plan.
 //
 // A run is a tree of gate-sized contractions listed in path order; its depth
 // is 15-25 levels where it has 180-730 steps (the 12- and 30-qubit brickwork
@@ -45,6 +45,7 @@ void add_part(const StepDesc* st, int n, SmallRuns& sr) {
     SmallPart part;
     part.step0 = (int32_t)sr.steps.size();
     part.n_steps = n;
+    part.cls = st[0].out_cls;
     std::vector<int> level(n, 0);
     int n_lvl = 0;
     for (int k = 0; k < n; k++) {
@@ -74,6 +75,9 @@ void add_part(const StepDesc* st, int n, SmallRuns& sr) {
                 p.inst = d.cls;
                 p.cache = d.cls == CLS_TRAJ ? d.cache : 0;
             }
+            p.slice0 = (int32_t)sr.slices.size();
+            p.n_slice = d.n_slice;
+            for (int q = 0; q < d.n_slice; q++) sr.slices.push_back({d.slice_qubit[q], (int32_t)d.slice_stride[q]});
             for (int q = 0; q < st[k].n_sum; q++) dense = dense && st[k].sum_stride[o][q] == (int64_t)1 << q;
         }
         s.out_off = st[k].out_off;
@@ -116,7 +120,6 @@ void add_part(const StepDesc* st, int n, SmallRuns& sr) {
 }  // namespace
 
 int small_run_len(const std::vector<StepDesc>& steps, size_t k, int fuse_max) {
-    if (!small_step(steps[k])) return 0;
     size_t en = k + 1;
     while (en < steps.size() && en - k < (size_t)fuse_max && steps[en].fuse_prev) en++;
     return (int)(en - k);

@@ -47,3 +47,27 @@ def test_long_and_cut_runs(fuse_max):
     assert any(sum(s["fuse_prev"] for s in b["steps"]) > 1024 for b in plan.describe(1)["blocks"])
     for a, b in zip(fused, single):
         assert torch.equal(a, b)
+
+
+# network-level runs (blocks listed class by class), past one word of prefix bits;
+# the sizes are those where the threads per network change
+@pytest.mark.parametrize("n_net", [1, 153, 400])
+def test_network_runs(n_net):
+    circ = W.paper_random_circuit(70, 420, np.random.default_rng(9))
+    fused = ptn.ptn_plan_path(circ, [10] * 7, hypersamples=8, est_traj=n_net, est_shots=n_net)
+    single = ptn.ptn_plan_path(circ, [10] * 7, hypersamples=8, est_traj=n_net, est_shots=n_net, fuse_max=1)
+    blocks = fused.describe(1)["blocks"]
+    assert any(s["out_cls"] == 2 and s["fuse_prev"] for b in blocks for s in b["steps"])
+    shots = ptn.ptn_sample_shots(fused, ptn.ptn_presample_trajectories(fused, 4, n_net), 6, shots_per_traj=1)
+    words = shots.to_torch()[1].clone()             # prefixes with weight, [n_net, 2]
+    for j in (1, 4, 6):
+        out = []
+        for plan in (fused, single):
+            tr = ptn.ptn_presample_trajectories(plan, 4, n_net)
+            marg = torch.empty((n_net, 1 << 10), device="cuda")
+            Z = torch.empty(n_net, dtype=torch.float64, device="cuda")
+            nt = torch.arange(n_net, dtype=torch.int32, device="cuda")
+            ptn.ptn_contract_batch(plan, tr, j, nt, words.reshape(-1), marg, Z)
+            out.append((marg, Z))
+        assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+        assert float(out[0][1].min()) > 0
