@@ -183,8 +183,11 @@ struct ObsTerm {
 };
 // Per trajectory: F = sum_x w(x) |psi(x)|^2 and the root adjoint w(x) conj(psi(x)),
 // w(x) = sum_t coeff_t (-1)^popc(x & zmask_t).
+// wtab (or null): w by element of the state's buffer, from launch_obs_weights
+constexpr int kObsTableBits = 20;
+void launch_obs_weights(const RootRef* d_root, int n, const ObsTerm* terms, int n_terms, double* wtab, cudaStream_t s);
 void launch_observable(const RootRef* d_root, const ChunkCtx& ctx, int n, const ObsTerm* terms, int n_terms,
-                       int64_t root_adj_off, int64_t traj0, double* F, cudaStream_t s);
+                       const double* wtab, int64_t root_adj_off, int64_t traj0, double* F, cudaStream_t s);
 // amp[t][x] = psi_t(x), bit q of x = qubit q, for the n_traj trajectories of the chunk
 void launch_amplitudes(const RootRef* d_root, const ChunkCtx& ctx, int n, int64_t n_traj, float2* amp, cudaStream_t s);
 // partial[(traj0 + i) * n_params + param] += 2 Re sum_e G_leaf[e] dLeaf[e]

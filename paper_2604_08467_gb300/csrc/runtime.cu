@@ -131,7 +131,7 @@ struct PlanWorkspace {
     DevBuf pack[2], err, grp, grp_cnt, grp_tile0, grp_scan;
     // expectation / gradient plans
     DevBuf arena_x[2];                    // ADJ, LGRAD arenas
-    DevBuf ev_steps, ev_bwd, ev_root, ev_pl, ev_dvt, ev_terms, ev_F, ev_partial, ev_iota;
+    DevBuf ev_steps, ev_bwd, ev_root, ev_pl, ev_dvt, ev_terms, ev_w, ev_F, ev_partial, ev_iota;
     DevBuf zpart;                         // per-tile partial totals of large marginal rows
     // final-block harvest of non-proportional sampling
     DevBuf h_rowmax, h_pmin, h_T, h_tcdf, h_tcnt, h_toff, h_scan, h_cnt, h_rank0, h_first;
@@ -156,7 +156,7 @@ struct PlanWorkspace {
                          &s_cap, &s_tmp_off, &s_rank0, &s_excl, &s_first, &s_ndist, &s_out_off, &s_tmp_x,
                          &s_tmp_c, &s_scan, &zero_prefix, &pack[0], &pack[1], &err, &grp, &grp_cnt,
                          &grp_tile0, &grp_scan, &arena_x[0], &arena_x[1], &ev_steps,
-                         &ev_bwd, &ev_root, &ev_pl, &ev_dvt, &ev_terms, &ev_F, &ev_partial, &ev_iota, &zpart,
+                         &ev_bwd, &ev_root, &ev_pl, &ev_dvt, &ev_terms, &ev_w, &ev_F, &ev_partial, &ev_iota, &zpart,
                          &h_rowmax, &h_pmin, &h_T, &h_tcdf, &h_tcnt, &h_toff, &h_scan, &h_cnt, &h_rank0, &h_first,
                          &c_h, &c_keys, &c_first, &c_rep, &c_list, &c_cnt};
         for (DevBuf* b : all) b->release();
@@ -1208,6 +1208,12 @@ ptn_status ptn_expval_grad(const ptn_plan* cplan, const ptn_traj* traj, const pt
         (e = ws->ev_partial.grow(sizeof(double) * E * np)) || (e = ws->ev_iota.grow(sizeof(int32_t) * E)))
         return e;
     PTN_CUDA(cudaMemcpyAsync(ws->ev_terms.p, terms.data(), sizeof(ObsTerm) * terms.size(), cudaMemcpyHostToDevice, s));
+    double* wtab = nullptr;
+    if (n <= kObsTableBits) {
+        if ((e = ws->ev_w.grow(sizeof(double) << n))) return e;
+        wtab = ws->ev_w.as<double>();
+        launch_obs_weights(ws->ev_root.as<RootRef>(), n, ws->ev_terms.as<ObsTerm>(), (int)terms.size(), wtab, s);
+    }
     PTN_CUDA(cudaMemsetAsync(ws->ev_partial.p, 0, sizeof(double) * E * np, s));
     launch_iota_i32(ws->ev_iota.as<int32_t>(), E, s);
     // chunks of trajectories that fit the memory cap
@@ -1269,7 +1275,7 @@ ptn_status ptn_expval_grad(const ptn_plan* cplan, const ptn_traj* traj, const pt
             return PTN_OK;
         };
         if ((e = run(bp.steps, ws->ev_steps.as<StepDesc>(), bp.small, -2))) return e;
-        launch_observable(ws->ev_root.as<RootRef>(), ctx, n, ws->ev_terms.as<ObsTerm>(), (int)terms.size(),
+        launch_observable(ws->ev_root.as<RootRef>(), ctx, n, ws->ev_terms.as<ObsTerm>(), (int)terms.size(), wtab,
                           bp.root_adj_off, t0, ws->ev_F.as<double>(), s);
         if ((e = run(bp.bwd, ws->ev_bwd.as<StepDesc>(), bp.small_bwd, -3))) return e;
         launch_leaf_grad(ctx, ws->ev_pl.as<ParamLeaf>(), (int)bp.pleaves.size(), ws->ev_dvt.as<float2>(), t0, nt, np,
