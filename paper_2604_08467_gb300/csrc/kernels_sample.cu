@@ -130,26 +130,39 @@ __global__ void k_var_ids(const uint8_t* __restrict__ kraus, int64_t n, int32_t 
 }
 
 // ----------------------------------------------------------------- scans --
+// Exclusive sum over the block (a multiple of 32 threads): a shuffle scan per
+// warp and one of the warp totals, three barriers (doubling steps over shared
+// memory took two per step, 20 for 1024 threads, 8 us of a 2048-entry scan).
 __device__ int64_t block_exclusive_scan(int64_t v, int64_t* sh, int64_t* total) {
-    // sh: blockDim.x + 1 elements
-    const int t = threadIdx.x;
-    sh[t] = v;
-    __syncthreads();
-    for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-        int64_t add = t >= off ? sh[t - off] : 0;
-        __syncthreads();
-        sh[t] += add;
-        __syncthreads();
+    // sh: 32 elements
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+    int64_t inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t u = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += u;
     }
-    const int64_t incl = sh[t];
-    if (total) *total = sh[blockDim.x - 1];
+    if (lane == 31) sh[warp] = inc;
     __syncthreads();
-    return incl - v;
+    if (warp == 0) {
+        int64_t w = lane < n_warps ? sh[lane] : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t u = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += u;
+        }
+        sh[lane] = w;
+    }
+    __syncthreads();
+    const int64_t before = warp ? sh[warp - 1] : 0;
+    if (total) *total = sh[n_warps - 1];
+    __syncthreads();
+    return before + inc - v;
 }
 
 __global__ void __launch_bounds__(1024) k_scan_tiles(const int64_t* __restrict__ in, int64_t* __restrict__ out,
                                                      int64_t n, int64_t* __restrict__ tile_sums) {
-    __shared__ int64_t sh[1025];
+    __shared__ int64_t sh[32];
     const int64_t base = (int64_t)blockIdx.x * kScanTile;
     const int64_t i0 = base + 2 * threadIdx.x, i1 = i0 + 1;
     const int64_t a = i0 < n ? in[i0] : 0, b = i1 < n ? in[i1] : 0;
@@ -170,7 +183,7 @@ __global__ void k_scan_add(int64_t* __restrict__ out, int64_t n, const int64_t* 
 __global__ void __launch_bounds__(1024) k_quantise_cdf(const double* __restrict__ w, int64_t n, int bits,
                                                        double* __restrict__ C) {
     __shared__ double red[1024];
-    __shared__ int64_t sh[1025];
+    __shared__ int64_t sh[32];
     __shared__ double carry;
     double m = 0.0;
     for (int64_t i = threadIdx.x; i < n; i += blockDim.x) m = fmax(m, w[i] > 0.0 ? w[i] : 0.0);
@@ -267,7 +280,8 @@ __global__ void k_rank0(const int64_t* __restrict__ excl, const int32_t* __restr
     if (i < n) rank0[i] = excl[i] - excl[first[traj[i]]];
 }
 
-// One block per parent: quantised CDF, c draws, histogram, ordered compaction
+// One block per parent (few parents, or blocks of more than 2^10 bins):
+// quantised CDF, c draws, histogram, ordered compaction
 // of the nonzero bins into the parent's slot of the temporary child list.
 __global__ void __launch_bounds__(256) k_sample_parents(const float* __restrict__ marg, int b,
                                                         const int32_t* __restrict__ traj,
@@ -280,7 +294,7 @@ __global__ void __launch_bounds__(256) k_sample_parents(const float* __restrict_
     const int64_t nb = (int64_t)1 << b;
     uint64_t* C = reinterpret_cast<uint64_t*>(smem);                   // nb
     unsigned int* hist = reinterpret_cast<unsigned int*>(C + nb);      // nb
-    __shared__ int64_t sh[257];
+    __shared__ int64_t sh[32];
     __shared__ float fred[256];
     __shared__ uint64_t carry;
     __shared__ int64_t wpos;
@@ -729,7 +743,10 @@ int64_t run_sample_block(const float* marg, int b, int start, const int32_t* ptr
     const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
     {
         StatScope st_sp(K_SAMPLE_PARENTS, s, (double)n_parent * ((double)((int64_t)1 << b) * 4.0 + 40.0), 0.0);
-        if (b <= kSampWarpMaxBits) {
+        // Up to two parents per SM: a CTA each (64 parents of 1000 shots and their
+        // children, two blocks: 90 us by one warp each, 63 us).  More: a warp each,
+        // up to 2^10 bins.
+        if (b <= kSampWarpMaxBits && n_parent > 2 * 152) {
             // per warp: CDF (8 B) + histogram (4 B) per bin; 48 KB at 2^10 bins
             const size_t smem = (size_t)kSampWarps * (((size_t)1 << b) * (sizeof(uint64_t) + sizeof(unsigned)));
             const uint32_t tagw = philox_tag(STREAM_SAMPLE, circuit, block);
