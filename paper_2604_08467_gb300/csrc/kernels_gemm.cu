@@ -126,6 +126,7 @@ struct GemmArgs {
     int32_t frag_sm[8], frag_row[8];   // place in the staged fragment, row within the 32
     int64_t frag_out[8];
     int64_t row_hi[2];           // output strides of rows 32 and 64 of a tile
+    int32_t tm_log, tn_log;      // log2 tiles along M and N (a step's sizes are powers of two)
     int64_t tiles_m, tiles_n, n_inst, n_tiles;
     const int32_t* net_tl;
     // stacked mode: the rows of all networks of one trajectory form one GEMM
@@ -915,7 +916,7 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
                  : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
         "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
@@ -925,7 +926,11 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
           "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+    tmem_ld32_issue(taddr, r);
+    tmem_ld_wait();
 }
 // Store 32 columns of this warp's 32 TMEM lanes (one register per column) and
 // wait until the stores have completed.
@@ -952,26 +957,23 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
 // set (acc_empty), and the epilogue starts after the item's last MMA
 // completes (acc_full).  Every wait is bounded.
 constexpr int kGemmThreads = 320;   // producer, MMA, 8 epilogue warps
-struct TileInfo {
-    int64_t inst, h, row_end;
-    int m0, n0, za, zb;
+struct TileInfo {              // (rows and instances are TMA coordinates: 32 bits)
+    int inst, h, row_end, m0, n0, za, zb;
 };
 __device__ __forceinline__ TileInfo decode_tile(const GemmArgs& g, int64_t tile) {
     TileInfo t;
     if (!g.stacked) {
-        const int64_t tiles = g.tiles_m * g.tiles_n;
-        const int64_t zt = tile / tiles;
-        const int64_t r = tile - zt * tiles;
-        const int64_t tm = r % g.tiles_m, tn = r / g.tiles_m;
-        t.inst = zt / g.n_h;
-        t.h = zt - t.inst * g.n_h;
+        const int64_t tm = tile & (((int64_t)1 << g.tm_log) - 1), tn = (tile >> g.tm_log) & (((int64_t)1 << g.tn_log) - 1);
+        const int64_t zt = tile >> (g.tm_log + g.tn_log);
+        t.inst = (int)(zt >> g.n_hb);
+        t.h = (int)(zt & (((int64_t)1 << g.n_hb) - 1));
         t.m0 = (int)(tm * kBM);
         t.n0 = (int)(tn * kBN);
         t.row_end = g.M;
-        const int64_t pa = g.a_pcls == g.out_cls ? t.inst : (g.a_pcls == CLS_TRAJ ? (int64_t)g.net_tl[t.inst] : 0);
-        const int64_t pb = g.b_pcls == g.out_cls ? t.inst : (g.b_pcls == CLS_TRAJ ? (int64_t)g.net_tl[t.inst] : 0);
-        t.za = (int)(pa * g.n_h + t.h);
-        t.zb = (int)(pb * g.n_h + t.h);
+        const int pa = g.a_pcls == g.out_cls ? t.inst : (g.a_pcls == CLS_TRAJ ? g.net_tl[t.inst] : 0);
+        const int pb = g.b_pcls == g.out_cls ? t.inst : (g.b_pcls == CLS_TRAJ ? g.net_tl[t.inst] : 0);
+        t.za = pa * g.n_h + t.h;
+        t.zb = pb * g.n_h + t.h;
     } else {
         // group (trajectory) of this tile: largest grp with grp_tile0[grp] <= tile
         int64_t lo = 0, hi = g.n_groups - 1;
@@ -985,14 +987,41 @@ __device__ __forceinline__ TileInfo decode_tile(const GemmArgs& g, int64_t tile)
         const int64_t tmg = (r1 - r0 + kBM - 1) / kBM;
         t.m0 = (int)(r0 + (r % tmg) * kBM);
         t.n0 = (int)((r / tmg) * kBN);
-        t.inst = lo;          // the trajectory (local index) supplies the B operand
+        t.inst = (int)lo;     // the trajectory (local index) supplies the B operand
         t.h = 0;
-        t.row_end = r1;
+        t.row_end = (int)r1;
         t.za = 0;
         t.zb = g.b_pcls == CLS_TRAJ ? (int)lo : 0;
     }
     return t;
 }
+
+// The tiles of a CTA as a warp sees them: lane l decodes the l-th of the next 32
+// at once (a stacked tile's group takes a binary search of dependent reads, so
+// one search's latency serves 32 tiles) and the warp takes them by shuffles.
+struct TileQueue {
+    TileInfo mine;
+    int64_t i = 0;
+    __device__ __forceinline__ bool next(const GemmArgs& g, int lane, TileInfo& t) {
+        const int64_t tile = blockIdx.x + i * gridDim.x;
+        if (tile >= g.n_tiles) return false;
+        const int l = (int)(i & 31);
+        if (l == 0) {
+            const int64_t ahead = tile + (int64_t)lane * gridDim.x;
+            mine = decode_tile(g, ahead < g.n_tiles ? ahead : tile);
+        }
+        t.inst = __shfl_sync(0xffffffffu, mine.inst, l);
+        t.h = __shfl_sync(0xffffffffu, mine.h, l);
+        t.row_end = __shfl_sync(0xffffffffu, mine.row_end, l);
+        t.m0 = __shfl_sync(0xffffffffu, mine.m0, l);
+        t.n0 = __shfl_sync(0xffffffffu, mine.n0, l);
+        t.za = __shfl_sync(0xffffffffu, mine.za, l);
+        t.zb = __shfl_sync(0xffffffffu, mine.zb, l);
+        i++;
+        return true;
+    }
+};
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }   // |e| <= 126
 
 template <int F>
 __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant__ CUtensorMap tmA,
@@ -1053,10 +1082,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
     const int64_t n_tiles = g.n_tiles;
 
     if (warp == 0) {
-        if (lane == 0) {
-            int64_t it = 0;
-            for (int64_t tile = blockIdx.x; tile < n_tiles && !*abort; tile += gridDim.x) {
-                const TileInfo t = decode_tile(g, tile);
+        int64_t it = 0;
+        TileQueue tq;
+        TileInfo t;
+        while (!__shfl_sync(0xffffffffu, *abort, 0) && tq.next(g, lane, t)) {
+            if (lane == 0) {
                 for (int kb = 0; kb < g.nkb; kb++, it++) {
                     const int s = (int)(it % kStages);
                     if (it >= kStages && !mbar_wait(&empty[s], (uint32_t)((it / kStages) - 1) & 1u, abort, g.wait_ns)) {
@@ -1072,6 +1102,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                     tma_load_3d(st + 2 * kTileA + kTileB, &tmB, g.Kh + kb * kBK, t.n0, t.zb, &full[s]);   // B lo
                 }
             }
+            __syncwarp();
+        }
+        if (lane == 0) {
             // let this CTA's own copies land before it exits (on every path: the
             // MMA thread may have stopped early): the last load of every stage
             // is that stage's newest phase
@@ -1157,9 +1190,22 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
             }
         int64_t lt = 0;
         bool live = true;
-        for (int64_t tile = blockIdx.x; tile < n_tiles && live; tile += gridDim.x) {
+        TileQueue tq;
+        TileInfo t, tn;
+        bool more = tq.next(g, lane, tn);
+        // FP16: this lane's row and column exponents of a tile's segment 0, read one
+        // tile ahead (their latency would precede every tile of a short contraction)
+        int ea = 0, eb = 0;
+        auto read_exps = [&](const TileInfo& x, int sg, int& a, int& b) {
+            const int64_t row = (int64_t)x.m0 + q * 32 + lane;
+            a = row < x.row_end ? g.exp_a[((int64_t)x.za * g.M + row) * n_seg + sg] : 0;
+            b = g.exp_b[((int64_t)x.zb * (g.N2 >> 1) + (x.n0 >> 1) + (c_lo >> 1) + lane) * n_seg + sg];
+        };
+        if (F == FMT_FP16 && more) read_exps(tn, 0, ea, eb);
+        while (more && live) {
             if (__shfl_sync(0xffffffffu, *abort, 0)) break;   // warp-uniform stop
-            const TileInfo t = decode_tile(g, tile);
+            t = tn;
+            more = tq.next(g, lane, tn);
             // output offsets of this warp's columns (staged: of its fragments' first columns)
             for (int c = c_lo / 2 + lane; c < c_hi / 2; c += 32) {
                 const int64_t n = (int64_t)(t.n0 / 2) + c;
@@ -1170,7 +1216,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
             }
             const int64_t row = (int64_t)t.m0 + q * 32 + lane;
             const int64_t row0 = g.staged ? (int64_t)t.m0 : row;   // staged: the tile's first row
-            int64_t m = row0, out_inst = g.out_map ? (int64_t)g.out_map[t.inst] : t.inst;
+            int64_t m = row0, out_inst = g.out_map ? g.out_map[t.inst] : t.inst;
             if (g.stacked) {
                 out_inst = row0 >> g.m_bits;
                 m = row0 & (((int64_t)1 << g.m_bits) - 1);
@@ -1181,7 +1227,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
             for (int i = 0; i < g.n_hb; i++)
                 if ((t.h >> i) & 1) moff += g.h_stride[i];
             const bool row_ok = row < t.row_end;
-            const int row_lim = (int)(t.row_end - t.m0 < 128 ? t.row_end - t.m0 : 128) - q * 32;   // valid rows of this quadrant
+            const int row_lim = min(t.row_end - t.m0, 128) - q * 32;   // valid rows of this quadrant
             float2* out = g.out + (row_ok || g.staged ? out_inst : 0) * g.out_size + moff + (g.staged ? out_l : 0);
             __syncwarp();
             for (int sg = 0; sg < n_seg; sg++, lt++) {
@@ -1194,13 +1240,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                 // column scales 2^eb; their product 2^(ea + eb) is exact
                 float urow = 1.f;
                 if (F == FMT_FP16) {
-                    for (int c = c_lo / 2 + lane; c < c_hi / 2; c += 32) {
-                        const int64_t n = (int64_t)(t.n0 / 2) + c;
-                        ucol[c] = 2 * n < g.N2
-                                      ? ldexpf(1.f, (int)g.exp_b[((int64_t)t.zb * (g.N2 >> 1) + n) * n_seg + sg])
-                                      : 0.f;
-                    }
-                    if (row_ok) urow = ldexpf(1.f, (int)g.exp_a[((int64_t)t.za * g.M + row) * n_seg + sg]);
+                    if (sg > 0) read_exps(t, sg, ea, eb);
+                    ucol[c_lo / 2 + lane] = pow2f(eb);
+                    urow = pow2f(ea);
+                    if (sg + 1 == n_seg && more) read_exps(tn, 0, ea, eb);
                     __syncwarp();
                 }
                 // one lane waits and the warp follows its outcome (lanes polling on
@@ -1252,15 +1295,33 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                 if (n_seg == 1) {
 #pragma unroll 1
                     for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
+                        // accumulators two at a time, added in order
                         float v[32];
-                        uint32_t r[32];
-                        tmem_ld32(acc0 + (uint32_t)c0, r);
+                        uint32_t r[32], r2[32];
+                        tmem_ld32_issue(acc0 + (uint32_t)c0, r);
+                        if (n_acc > 1) tmem_ld32_issue(acc0 + (uint32_t)(kBN + c0), r2);
+                        tmem_ld_wait();
 #pragma unroll
                         for (int j = 0; j < 32; j++) v[j] = __uint_as_float(r[j]);
-                        for (int a = 1; a < n_acc; a++) {
-                            tmem_ld32(acc0 + (uint32_t)(a * kBN + c0), r);
+                        if (n_acc > 1) {
+#pragma unroll
+                            for (int j = 0; j < 32; j++) v[j] += __uint_as_float(r2[j]);
+                        }
+                        if (n_acc > 2) {
+                            tmem_ld32_issue(acc0 + (uint32_t)(2 * kBN + c0), r);
+                            if (n_acc > 3) tmem_ld32_issue(acc0 + (uint32_t)(3 * kBN + c0), r2);
+                            tmem_ld_wait();
 #pragma unroll
                             for (int j = 0; j < 32; j++) v[j] += __uint_as_float(r[j]);
+                            if (n_acc > 3) {
+#pragma unroll
+                                for (int j = 0; j < 32; j++) v[j] += __uint_as_float(r2[j]);
+                            }
+                        }
+                        if (c0 + 32 >= c_hi) {   // everything read: the set may take its next item while the tile is stored
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(&acc_empty[set]);
                         }
                         if (F == FMT_FP16) {
 #pragma unroll
@@ -1305,9 +1366,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                         }
                     }
                 }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&acc_empty[set]);   // accumulators read: this set may take the next item
+                if (n_seg > 1) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&acc_empty[set]);   // accumulators read: this set may take the next item
+                }
             }
         }
     }
@@ -1582,6 +1645,8 @@ ptn_status run_gemm(const StepDesc& st, const ChunkCtx& ctx, int64_t n_inst, voi
     ga.n_hb = nh;
     ga.tiles_m = (M + kBM - 1) / kBM;
     ga.tiles_n = (2 * N + kBN - 1) / kBN;
+    while ((1ll << ga.tm_log) < ga.tiles_m) ga.tm_log++;
+    while ((1ll << ga.tn_log) < ga.tiles_n) ga.tn_log++;
     ga.n_inst = n_inst;
     ga.net_tl = ctx.net_tl;
     ga.out = ctx.arena[st.out_arena] + st.out_off * ctx.arena_inst[st.out_arena];
