@@ -4,9 +4,20 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "ptn_internal.h"
 
 namespace ptn {
+
+// Runs f once per device of the process (kernel attributes are set per device);
+// other threads wait for it.
+template <class F>
+inline void once_per_device(std::once_flag (&done)[64], F&& f) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::call_once(done[dev & 63], f);
+}
 
 // Philox4x32-10 (Salmon et al., SC'11): ten rounds of two 32x32->64-bit
 // multiplies mixed with the key, the key bumped by the Weyl constants between

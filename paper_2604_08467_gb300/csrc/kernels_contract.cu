@@ -844,12 +844,11 @@ bool rows_split(const StepDesc& h, const ChunkCtx& ctx, int shared, int g_log, R
 template <int RA, int RB>
 void launch_rows_t(const StepDesc* d_step, const ChunkCtx& ctx, int64_t n_inst, const GroupArgs& g, int smem,
                    cudaStream_t s) {
-    static const bool attr_set = [] {
+    static std::once_flag done[64];
+    once_per_device(done, [] {
         cudaFuncSetAttribute(k_contract_rows<RA, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowsSmem);
         cudaFuncSetAttribute(k_contract_group<RA, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGroupSmem);
-        return true;
-    }();
-    (void)attr_set;
+    });
     const int threads = std::max(64, 1 << g.r.n_lane);
     const int64_t cap = 152ll * std::max(1, std::min(2048 / threads / 2, 220 * 1024 / (smem + 1024)));
     if (g.n_groups) {
@@ -922,14 +921,15 @@ bool launch_rows(const StepDesc* d_step, const StepDesc& h, const ChunkCtx& ctx,
 // (outcome bits sorted by stride) and turned to outcome order in shared
 // memory, so reads and writes are both coalesced; one thread per 16 consecutive
 // outcomes read 8 bytes per 64-128 byte step, with 64 of 256 threads busy at
-// 2^10 outcomes (1.4 TB/s).  Z adds 16 consecutive outcomes per thread, a
-// shuffle tree per warp, the warps in order, the tiles in order; the 16 are
-// added as 64-bit integers scaled by the thread's largest entry (58 bits for
-// it, so the sum is closer than one of FP64 roundings), because this chip adds
-// two FP64 numbers per clock and SM.
-// Measured: 1.9 M rows of 2^10 outcomes 15.6 -> 10.0 ms with the closing |a|^2
+// 2^10 outcomes (1.4 TB/s).  Blocks of 2^10 and of 2^12 outcomes and more hold
+// their elements in registers (TB): a warp's part of a row is added as 64-bit
+// integers scaled by its largest entry (53 bits for it, the accuracy of adding
+// FP64 roundings), because this chip adds two FP64 numbers per clock and SM;
+// warps and tiles follow in order in FP64.  The others add 16 consecutive
+// outcomes per thread the same way and use a shuffle tree.
+// Measured: 1.9 M rows of 2^10 outcomes 15.6 -> 8.4 ms with the closing |a|^2
 // (6.3 ms, 24.6 GB) gone; 24 rows of 2^28 outcomes, an outer product, 46.1 ms
-// and 13.2 ms for the product -> 22.5 ms.
+// and 13.2 ms for the product -> 18.9 ms.
 constexpr int kFinThreads = 256, kFinTileLog = 12, kFinTile = 1 << kFinTileLog;
 enum FinMode { FIN_ROOT = 0, FIN_SQUARE = 1, FIN_PRODUCT = 2 };
 struct FinArgs {
@@ -942,61 +942,91 @@ struct FinArgs {
     int64_t tiles, n_net, n_units;
 };
 
+// 2^s as two FP32 factors and 2^-s in FP64, |s| <= 250
+struct FixedScale {
+    float f1, f2;
+    double inv;
+    __device__ __forceinline__ explicit FixedScale(int s) {
+        const int s1 = s / 2, s2 = s - s1;
+        f1 = __int_as_float((127 + s1) << 23);
+        f2 = __int_as_float((127 + s2) << 23);
+        inv = __longlong_as_double((int64_t)(1023 - s) << 52);
+    }
+    __device__ __forceinline__ int64_t operator()(float v) const { return __float2ll_rn(v * f1 * f2); }
+};
 // Sum of 16 floats of a thread.
 __device__ __forceinline__ double sum16(const float* v) {
-    float m = 0.f, a = 0.f;
+    float m = 0.f;
+    bool fin = true;
     for (int k = 0; k < 16; k++) {
         m = fmaxf(m, fabsf(v[k]));
-        a += fabsf(v[k]);
+        fin = fin && fabsf(v[k]) < __int_as_float(0x7f800000);
     }
     double acc = 0.0;
-    if (!(a <= 3.0e38f)) {         // NaN, infinite, or too large for the scale below
+    if (!fin) {                    // infinite entries or NaN
         for (int k = 0; k < 16; k++) acc += (double)v[k];
         return acc;
     }
     if (m == 0.f) return 0.0;
-    const int s = 58 - frexp_exp(m), s1 = s / 2, s2 = s - s1;   // |s| <= 206
-    const float f1 = __int_as_float((127 + s1) << 23), f2 = __int_as_float((127 + s2) << 23);
+    const FixedScale fs(58 - frexp_exp(m));
     int64_t t = 0;
-    for (int k = 0; k < 16; k++) t += __float2ll_rn(v[k] * f1 * f2);
-    return (double)t * __longlong_as_double((int64_t)(1023 - s) << 52);
+    for (int k = 0; k < 16; k++) t += fs(v[k]);
+    return (double)t * fs.inv;
+}
+// Sum of N floats per lane over a warp (in lane 0), and the largest entry (m, all lanes).
+template <int N>
+__device__ __forceinline__ double warp_sum(const float* v, float& m) {
+    float a = 0.f;
+    m = 0.f;
+    bool fin = true;
+#pragma unroll
+    for (int k = 0; k < N; k++) {
+        m = fmaxf(m, v[k]);
+        a = fmaxf(a, fabsf(v[k]));
+        fin = fin && fabsf(v[k]) < __int_as_float(0x7f800000);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
+    }
+    if (!__all_sync(0xffffffffu, fin)) {   // infinite entries or NaN
+        double acc = 0.0;
+        for (int k = 0; k < N; k++) acc += (double)v[k];
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+        return acc;
+    }
+    if (a == 0.f) return 0.0;
+    const FixedScale fs(53 - frexp_exp(a));
+    int64_t t = 0;
+#pragma unroll
+    for (int k = 0; k < N; k++) t += fs(v[k]);
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return (double)t * fs.inv;
 }
 
-template <int IT, int MODE>        // elements per thread (0: n_it, narrow blocks)
+template <int TB, int MODE>        // TB: tb = 10 or 12 with 4096 elements per unit; 0: any other
 __global__ void __launch_bounds__(kFinThreads) k_finalize(const OperandDesc* __restrict__ op0, const OperandDesc* __restrict__ op1,
                                                           const __grid_constant__ ChunkCtx c,
                                                           const __grid_constant__ FinArgs f, float* __restrict__ marg,
                                                           double* __restrict__ Z, double* __restrict__ part,
                                                           unsigned* __restrict__ rowmax) {
-    constexpr int NOP = MODE == FIN_PRODUCT ? 2 : 1;
+    constexpr int NOP = MODE == FIN_PRODUCT ? 2 : 1, NV = 16;
     __shared__ float sm[kFinTile + kFinTile / 16];   // outcome x at x + x / 16
-    __shared__ const float2* ptr[NOP][kFinThreads];
-    __shared__ int64_t it_off[NOP][16];
-    __shared__ int it_x[16];
-    __shared__ double red[kFinThreads / 32];
-    const int tid = threadIdx.x, n_it = IT ? IT : f.n_it, unit_log = f.tb + f.net_log;
+    __shared__ const float2* ptr[NOP][TB ? 4 : kFinThreads];
+    __shared__ double red[4 * kFinThreads / 32];
+    const int tid = threadIdx.x, n_it = TB ? NV : f.n_it, tb = TB ? TB : f.tb;
     // element e = it * 256 + tid: its bits below tb select the outcome in the
     // order of the operands' memory, those above the network of the unit
-    auto place = [&](int e, int64_t* off, int& x) {
-        x = e >> f.tb << f.tb;
-#pragma unroll
-        for (int o = 0; o < NOP; o++) off[o] = 0;
-        for (int k = 0; k < f.tb; k++)
-            if ((e >> k) & 1) {
-#pragma unroll
-                for (int o = 0; o < NOP; o++) off[o] += f.stride[o][k];
-                x += 1 << f.x_bit[k];
-            }
-    };
     int64_t off_t[NOP];
-    int x_t;
-    place(tid, off_t, x_t);
-    if (tid < 16) {
-        int64_t off[NOP];
-        place(tid << 8 & ((1 << unit_log) - 1), off, it_x[tid]);
+    int x_t = 0;
 #pragma unroll
-        for (int o = 0; o < NOP; o++) it_off[o][tid] = off[o];
-    }
+    for (int o = 0; o < NOP; o++) off_t[o] = 0;
+    for (int k = 0; k < 8; k++)
+        if ((tid >> k) & 1) {
+#pragma unroll
+            for (int o = 0; o < NOP; o++) off_t[o] += f.stride[o][k];
+            x_t += 1 << f.x_bit[k];
+        }
     const int64_t nx = (int64_t)1 << f.b;
     for (int64_t u = blockIdx.x; u < f.n_units; u += gridDim.x) {
         const int64_t tile = u % f.tiles, net0 = (u / f.tiles) << f.net_log;
@@ -1006,49 +1036,87 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const OperandDesc* __r
 #pragma unroll
             for (int o = 0; o < NOP; o++) {
                 const float2* p = operand_ptr(o ? *op1 : *op0, CLS_NET, net0 + tid, c);
-                for (int t = f.tb; t < f.b; t++)
-                    if ((tile >> (t - f.tb)) & 1) p += f.hi_stride[o][t];
+                for (int t = tb; t < f.b; t++)
+                    if ((tile >> (t - tb)) & 1) p += f.hi_stride[o][t];
                 ptr[o][tid] = p;
             }
         __syncthreads();
-        const int valid = nets << f.tb;   // elements of the unit
+        const int valid = nets << tb;     // elements of the unit
+        // every read of the unit in flight before the first is used
+        float v[NV];
 #pragma unroll
-        for (int it = 0; it < n_it; it++) {
+        for (int it = 0; it < NV; it++) {
             const int e = it * kFinThreads + tid;
-            float v = 0.f;
-            if (e < valid) {
-                const float2 x = ptr[0][e >> f.tb][off_t[0] + it_off[0][it]];
+            v[it] = 0.f;
+            if (it < n_it && e < valid) {
+                int64_t off[NOP];
+#pragma unroll
+                for (int o = 0; o < NOP; o++) {
+                    off[o] = off_t[o];
+#pragma unroll
+                    for (int k = 8; k < kFinTileLog; k++)
+                        if ((it >> (k - 8)) & 1) off[o] += f.stride[o][k];
+                }
+                const float2* p = ptr[0][e >> tb] + off[0];
                 if constexpr (MODE == FIN_ROOT) {
-                    v = x.x;
+                    v[it] = p->x;
                 } else {
+                    const float2 x = *p;
                     float2 y = x;
-                    if constexpr (MODE == FIN_PRODUCT) y = ptr[NOP - 1][e >> f.tb][off_t[NOP - 1] + it_off[NOP - 1][it]];
-                    v = fmaf(-(f.s0 * x.y), f.s1 * y.y, fmaf(x.x, y.x, 0.f));   // as the SIMT kernels' single term
+                    if constexpr (MODE == FIN_PRODUCT) y = ptr[NOP - 1][e >> tb][off[NOP - 1]];
+                    v[it] = fmaf(-(f.s0 * x.y), f.s1 * y.y, fmaf(x.x, y.x, 0.f));   // as the SIMT kernels' single term
                 }
             }
-            const int x = x_t + it_x[it];
-            sm[x + (x >> 4)] = v;
+        }
+#pragma unroll
+        for (int it = 0; it < NV; it++) {
+            int x = x_t;
+#pragma unroll
+            for (int k = 8; k < kFinTileLog; k++)
+                if ((it >> (k - 8)) & 1) x += 1 << f.x_bit[k];
+            if (it < n_it) sm[x + (x >> 4)] = v[it];
+        }
+        if constexpr (TB != 0) {
+            constexpr int PER = 1 << (TB - 8), NETS = NV / PER;   // a thread's elements of a network
+#pragma unroll
+            for (int g = 0; g < NETS; g++) {
+                float m;
+                const double t = warp_sum<PER>(v + g * PER, m);
+                if ((tid & 31) == 0) {
+                    red[g * 8 + (tid >> 5)] = t;
+                    if (rowmax && m > 0.f && g < nets) atomicMax(&rowmax[net0 + g], __float_as_uint(m));
+                }
+            }
         }
         __syncthreads();
-        float* out = marg + net0 * nx + (tile << f.tb);
+        float* out = marg + net0 * nx + (tile << tb);
 #pragma unroll
-        for (int it = 0; it < n_it; it++) {
+        for (int it = 0; it < NV; it++) {
             const int x = it * kFinThreads + tid;
-            if (x < valid) out[x] = sm[x + (x >> 4)];
+            if (it < n_it && x < valid) out[x] = sm[x + (x >> 4)];
+        }
+        if constexpr (TB != 0) {
+            if (tid < nets) {
+                double t = 0.0;
+                for (int w = 0; w < 8; w++) t += red[tid * 8 + w];
+                if (f.tiles == 1) Z[net0 + tid] = t;
+                else part[(net0 + tid) * f.tiles + tile] = t;
+            }
+            continue;
         }
         // narrow blocks: threads past the last network drop out (whole trees of them)
-        const unsigned mask = __ballot_sync(0xffffffffu, f.tb >= 9 || 16 * tid < valid);
-        if (f.tb < 9 && 16 * tid >= valid) continue;
+        const unsigned mask = __ballot_sync(0xffffffffu, tb >= 9 || 16 * tid < valid);
+        if (tb < 9 && 16 * tid >= valid) continue;
         const float* row = sm + 17 * tid;
-        if (f.tb < 4) {            // several networks per thread
-            for (int g = 0; g < 16 >> f.tb && 16 * tid + (g << f.tb) < valid; g++) {
+        if (tb < 4) {              // several networks per thread
+            for (int g = 0; g < 16 >> tb && 16 * tid + (g << tb) < valid; g++) {
                 double acc = 0.0;
                 float m = 0.f;
-                for (int k = 0; k < 1 << f.tb; k++) {
-                    acc += (double)row[(g << f.tb) + k];
-                    m = fmaxf(m, row[(g << f.tb) + k]);
+                for (int k = 0; k < 1 << tb; k++) {
+                    acc += (double)row[(g << tb) + k];
+                    m = fmaxf(m, row[(g << tb) + k]);
                 }
-                const int64_t net = net0 + (((16 * tid) >> f.tb) + g);
+                const int64_t net = net0 + (((16 * tid) >> tb) + g);
                 Z[net] = acc;
                 if (rowmax && m > 0.f) rowmax[net] = __float_as_uint(m);
             }
@@ -1057,15 +1125,15 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const OperandDesc* __r
         double acc = 0.0;
         float m = 0.f;
         if (16 * tid < valid) {
-            float v[16];
+            float r[16];
 #pragma unroll
             for (int k = 0; k < 16; k++) {
-                v[k] = row[k];
-                m = fmaxf(m, v[k]);
+                r[k] = row[k];
+                m = fmaxf(m, r[k]);
             }
-            acc = sum16(v);
+            acc = sum16(r);
         }
-        const int per = 1 << (f.tb - 4);                // threads per network
+        const int per = 1 << (tb - 4);                  // threads per network
         const int64_t net = net0 + tid / per;
         const int width = per < 32 ? per : 32;
         for (int o = width >> 1; o > 0; o >>= 1) {
@@ -1351,6 +1419,7 @@ void launch_finalize(const RootRef* d_root, const RootRef& root, const StepDesc*
         return v ? v : ((int64_t)1 << 40) + stride(1 - big, t);
     };
     std::sort(order, order + f.tb, [&](int x, int y) { return key(x) < key(y); });
+    for (int k = f.tb; k < kFinTileLog; k++) f.x_bit[k] = k;   // network bits: no stride
     for (int k = 0; k < f.tb; k++) {
         f.x_bit[k] = order[k];
         for (int o = 0; o < 2; o++) f.stride[o][k] = stride(o, order[k]);
@@ -1360,10 +1429,14 @@ void launch_finalize(const RootRef* d_root, const RootRef& root, const StepDesc*
     StatScope sc(K_FINALIZE, s, (double)n_net * (double)(1ll << b) * (mode == FIN_PRODUCT ? 4.0 : 12.0), 0.0);
     const unsigned grid = (unsigned)std::min<int64_t>(f.n_units, 152 * 8);
     auto run = [&](auto kernel) { kernel<<<grid, kFinThreads, 0, s>>>(op0, op1, ctx, f, marg, Z, part, rowmax); };
-    if (f.n_it == 16) {
-        if (mode == FIN_ROOT) run(k_finalize<16, FIN_ROOT>);
-        else if (mode == FIN_SQUARE) run(k_finalize<16, FIN_SQUARE>);
-        else run(k_finalize<16, FIN_PRODUCT>);
+    if (f.tb == 12) {
+        if (mode == FIN_ROOT) run(k_finalize<12, FIN_ROOT>);
+        else if (mode == FIN_SQUARE) run(k_finalize<12, FIN_SQUARE>);
+        else run(k_finalize<12, FIN_PRODUCT>);
+    } else if (f.tb == 10) {
+        if (mode == FIN_ROOT) run(k_finalize<10, FIN_ROOT>);
+        else if (mode == FIN_SQUARE) run(k_finalize<10, FIN_SQUARE>);
+        else run(k_finalize<10, FIN_PRODUCT>);
     } else {
         if (mode == FIN_ROOT) run(k_finalize<0, FIN_ROOT>);
         else if (mode == FIN_SQUARE) run(k_finalize<0, FIN_SQUARE>);

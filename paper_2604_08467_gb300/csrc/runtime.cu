@@ -1210,9 +1210,13 @@ ptn_status ptn_expval_grad(const ptn_plan* cplan, const ptn_traj* traj, const pt
     PTN_CUDA(cudaMemcpyAsync(ws->ev_terms.p, terms.data(), sizeof(ObsTerm) * terms.size(), cudaMemcpyHostToDevice, s));
     double* wtab = nullptr;
     if (n <= kObsTableBits) {
-        if ((e = ws->ev_w.grow(sizeof(double) << n))) return e;
-        wtab = ws->ev_w.as<double>();
-        launch_obs_weights(ws->ev_root.as<RootRef>(), n, ws->ev_terms.as<ObsTerm>(), (int)terms.size(), wtab, s);
+        if (ws->ev_w.grow(sizeof(double) << n) == PTN_OK) {   // no room: the weights are formed per element
+            wtab = ws->ev_w.as<double>();
+            launch_obs_weights(ws->ev_root.as<RootRef>(), n, ws->ev_terms.as<ObsTerm>(), (int)terms.size(), wtab, s);
+        } else {
+            clear_error();
+            cudaGetLastError();
+        }
     }
     PTN_CUDA(cudaMemsetAsync(ws->ev_partial.p, 0, sizeof(double) * E * np, s));
     launch_iota_i32(ws->ev_iota.as<int32_t>(), E, s);
