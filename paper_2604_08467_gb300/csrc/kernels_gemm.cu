@@ -35,7 +35,6 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
-#include <vector>
 
 #include "kernels.cuh"
 #include "stats.h"
@@ -51,6 +50,7 @@ constexpr int kStages = 3;        // pipeline depth (4 tiles of 16 KB per stage)
 constexpr int kTileA = kBM * kRowBytes;
 constexpr int kTileB = kBN * kRowBytes;
 constexpr int kStageBytes = 2 * kTileA + 2 * kTileB;
+constexpr int kPairN = 2 * kBN;   // columns of a CTA pair's tile (k_gemm<F, true>): 128 B rows staged by each CTA
 // epilogue staging: per epilogue warp a fragment of 32 rows x 8 complex columns,
 // rows padded to 9 slots (the 8-byte writes of a column and most reads hit
 // different banks)
@@ -126,6 +126,8 @@ struct GemmArgs {
     int32_t frag_sm[8], frag_row[8];   // place in the staged fragment, row within the 32
     int64_t frag_out[8];
     int64_t row_hi[2];           // output strides of rows 32 and 64 of a tile
+    int32_t pair;                // CTA pairs: an M tile and its odd neighbour run together
+    int32_t bn;                  // columns of a tile
     int32_t tm_log, tn_log;      // log2 tiles along M and N (a step's sizes are powers of two)
     int64_t tiles_m, tiles_n, n_inst, n_tiles;
     const int32_t* net_tl;
@@ -830,12 +832,30 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}\n"
         : "=r"(ok)
         : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
     return ok != 0;
+}
+// the same barrier of CTA `rank` of the cluster (a shared::cluster address)
+__device__ __forceinline__ uint32_t mbar_of(uint64_t* bar, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(bar)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ uint64_t global_ns() {
     uint64_t t;
@@ -870,6 +890,13 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, in
         ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
         : "memory");
 }
+// the same load by a CTA of a pair, its bytes counted by the leader's barrier
+__device__ __forceinline__ void tma_load_3d_pair(void* dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -885,35 +912,60 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
     return d;
 }
 
-// Instruction descriptor: D = F32, A = B = format F, both K-major, M = 128, N = kBN.
-template <int F>
+// Instruction descriptor: D = F32, A = B = format F, both K-major, M = 128 (a
+// pair: 256, 128 rows per CTA), N = kBN (a pair: kPairN).
+template <int F, bool PAIR>
 __host__ __device__ constexpr uint32_t idesc() {
-    return (1u << 4) | (Fmt<F>::kAB << 7) | (Fmt<F>::kAB << 10) | ((uint32_t)(kBN >> 3) << 17) |
-           ((uint32_t)(kBM >> 4) << 24);
+    return (1u << 4) | (Fmt<F>::kAB << 7) | (Fmt<F>::kAB << 10) | ((uint32_t)((PAIR ? kPairN : kBN) >> 3) << 17) |
+           ((uint32_t)((PAIR ? 2 * kBM : kBM) >> 4) << 24);
 }
 
 // One MMA over 32 bytes of K (8 TF32 or 16 BF16/FP16 elements).
-template <int F>
+template <int F, bool PAIR>
 __device__ __forceinline__ void umma(uint32_t taddr, uint64_t ad, uint64_t bd, uint32_t acc) {
-    if constexpr (F == FMT_TF32) {
+    if constexpr (F == FMT_TF32 && !PAIR) {
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
             "setp.ne.b32 p, %4, 0;\n\t"
             "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(taddr),
-            "l"(ad), "l"(bd), "r"(idesc<F>()), "r"(acc)
+            "l"(ad), "l"(bd), "r"(idesc<F, PAIR>()), "r"(acc)
+            : "memory");
+    } else if constexpr (F == FMT_TF32) {
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(taddr),
+            "l"(ad), "l"(bd), "r"(idesc<F, PAIR>()), "r"(acc)
+            : "memory");
+    } else if constexpr (!PAIR) {
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(taddr),
+            "l"(ad), "l"(bd), "r"(idesc<F, PAIR>()), "r"(acc)
             : "memory");
     } else {
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
             "setp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(taddr),
-            "l"(ad), "l"(bd), "r"(idesc<F>()), "r"(acc)
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(taddr),
+            "l"(ad), "l"(bd), "r"(idesc<F, PAIR>()), "r"(acc)
             : "memory");
     }
 }
+// bar (a pair: this barrier of both CTAs) arrives when the MMAs issued so far are done
+template <bool PAIR>
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
+    if constexpr (PAIR) {
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+                smem_u32(bar)),
+            "h"((uint16_t)3)
+            : "memory");
+    } else {
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+                     : "memory");
+    }
 }
 
 __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&r)[32]) {
@@ -957,6 +1009,7 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
 // set (acc_empty), and the epilogue starts after the item's last MMA
 // completes (acc_full).  Every wait is bounded.
 constexpr int kGemmThreads = 320;   // producer, MMA, 8 epilogue warps
+constexpr int64_t kPairRows = 4;    // least M tiles per trajectory of a stacked GEMM run by CTA pairs
 struct TileInfo {              // (rows and instances are TMA coordinates: 32 bits)
     int inst, h, row_end, m0, n0, za, zb;
 };
@@ -968,7 +1021,7 @@ __device__ __forceinline__ TileInfo decode_tile(const GemmArgs& g, int64_t tile)
         t.inst = (int)(zt >> g.n_hb);
         t.h = (int)(zt & (((int64_t)1 << g.n_hb) - 1));
         t.m0 = (int)(tm * kBM);
-        t.n0 = (int)(tn * kBN);
+        t.n0 = (int)(tn * g.bn);
         t.row_end = g.M;
         const int pa = g.a_pcls == g.out_cls ? t.inst : (g.a_pcls == CLS_TRAJ ? g.net_tl[t.inst] : 0);
         const int pb = g.b_pcls == g.out_cls ? t.inst : (g.b_pcls == CLS_TRAJ ? g.net_tl[t.inst] : 0);
@@ -984,9 +1037,9 @@ __device__ __forceinline__ TileInfo decode_tile(const GemmArgs& g, int64_t tile)
         }
         const int64_t r = tile - g.grp_tile0[lo];
         const int64_t r0 = (int64_t)g.grp_net0[lo] << g.m_bits, r1 = (int64_t)g.grp_net0[lo + 1] << g.m_bits;
-        const int64_t tmg = (r1 - r0 + kBM - 1) / kBM;
+        const int64_t tmg = ((r1 - r0 + kBM - 1) / kBM + g.pair) & ~(int64_t)g.pair;   // pairs: an even number
         t.m0 = (int)(r0 + (r % tmg) * kBM);
-        t.n0 = (int)((r / tmg) * kBN);
+        t.n0 = (int)((r / tmg) * g.bn);
         t.inst = (int)lo;     // the trajectory (local index) supplies the B operand
         t.h = 0;
         t.row_end = (int)r1;
@@ -1023,7 +1076,24 @@ struct TileQueue {
 };
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }   // |e| <= 126
 
-template <int F>
+// PAIR: two CTAs of a cluster work on 256 x 256 tiles (cta_group::2): each
+// stages its own 128 A rows and half of the B rows, both tensor cores read both
+// halves.  A 128 x 128 tile is bound by shared memory: per k-block its 12 MMAs
+// read 96 KB and TMA writes 64 KB, 1280 clocks at 128 bytes each, and takes 1370
+// to 1430 where the MMAs alone take 768 (64 clocks each with resident operands);
+// a pair of 128 columns measured the same 1380.  With 256 columns a CTA's k-block
+// has twice the work for the same 64 KB written.  The accumulator and the running
+// sum then fill TMEM, so only segmented tiles run so: one accumulator set, freed
+// for the next segment as soon as it is added to the sum (the last segment too,
+// before the tile is stored from the sum).  The even CTA leads: its producer
+// counts both CTAs' bytes, its MMA thread issues for both and signals freed
+// stages and finished accumulators to both, and both CTAs' epilogue warps free
+// the accumulator at its barrier.  The products, their order and the segments are
+// those of one CTA, so every output is the same.  Measured: the middle 30-qubit
+// block's step of 4096 terms (FP16 hi/lo) 64.3 -> 53.3 ms (518 TFLOP/s, 0.95 of
+// the sustained peak / 3 with its padded rows), 512 terms of the 16-qubit state
+// (TF32) 9.57 -> 6.63 ms (331 TFLOP/s).
+template <int F, bool PAIR>
 __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant__ CUtensorMap tmA,
                                                           const __grid_constant__ CUtensorMap tmB,
                                                           const __grid_constant__ GemmArgs g) {
@@ -1031,16 +1101,18 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* stage0 = smem;
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
-    uint64_t* empty = full + kStages;
-    uint64_t* acc_full = empty + kStages;   // per accumulator set
-    uint64_t* acc_empty = acc_full + 2;
+    constexpr int NST = kStages, TN = PAIR ? kPairN : kBN;   // columns of a tile
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);   // a pair: the leader's count
+    uint64_t* empty = full + NST;
+    uint64_t* acc_full = empty + NST;       // per accumulator set
+    uint64_t* acc_empty = acc_full + 2;     // a pair: the leader's count
     uint64_t* drain = acc_empty + 2;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
     int64_t* noff_all = reinterpret_cast<int64_t*>(tslot + 4);   // 8 epilogue warps x kBN / 2 column offsets
     float* ucol_all = reinterpret_cast<float*>(noff_all + 8 * (kBN / 2));   // FP16: column scales 2^eb
     float2* stg_all = reinterpret_cast<float2*>(smem + kStages * kStageBytes + kTabBytes);   // staged fragments
+    const uint32_t rank = PAIR ? cluster_rank() : 0u;
     // Work items are (tile, K segment) pairs.  A tile's k-blocks run in
     // segments of at most kSegKb; the tensor core's accumulation truncates, so
     // long chains drift: every segment is accumulated on its own and the
@@ -1048,35 +1120,51 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
     // running sum kept in TMEM columns [2 kBN, 3 kBN), then writes the tile
     // once.  Segmented tiles use two accumulator sets of one accumulator, short
     // contractions (at most 8 k-blocks) two sets of kAcc / 2 (the epilogue of
-    // one item overlaps the MMAs of the next); the others one set of kAcc.
+    // one item overlaps the MMAs of the next); the others one set of kAcc.  A
+    // pair's accumulator takes columns [0, kPairN), its running sum the rest.
     const int seg_kb = g.nkb > kSegKb ? kSegKb : g.nkb;
     const int n_seg = (g.nkb + seg_kb - 1) / seg_kb;
-    const int n_sets = (g.nkb <= 8 || n_seg > 1) ? 2 : 1;
+    const int n_sets = !PAIR && (g.nkb <= 8 || n_seg > 1) ? 2 : 1;
     const int acc_per = n_seg > 1 ? 1 : kAcc / n_sets;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 32) {
-        for (int s = 0; s < kStages; s++) {
+        for (int s = 0; s < NST; s++) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
         for (int k = 0; k < 2; k++) {
             mbar_init(&acc_full[k], 1);
-            mbar_init(&acc_empty[k], 8);   // one arrival per epilogue warp
+            mbar_init(&acc_empty[k], PAIR ? 16 : 8);   // one arrival per epilogue warp
         }
         mbar_init(drain, 1);
         *abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
-                     "r"(kTmemCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (PAIR) {
+        // both CTAs' barriers exist before either signals the other's
+        __syncthreads();
+        cluster_sync();
+        if (warp == 0) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                         "r"(kTmemCols)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        }
+        tc_fence_before();
+        __syncthreads();
+        cluster_sync();              // the peer's accumulators are allocated too
+    } else {
+        if (warp == 0) {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
+                         "r"(kTmemCols)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
+        tc_fence_before();
+        __syncthreads();
     }
-    tc_fence_before();
-    __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
     const int64_t n_tiles = g.n_tiles;
@@ -1088,18 +1176,28 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
         while (!__shfl_sync(0xffffffffu, *abort, 0) && tq.next(g, lane, t)) {
             if (lane == 0) {
                 for (int kb = 0; kb < g.nkb; kb++, it++) {
-                    const int s = (int)(it % kStages);
-                    if (it >= kStages && !mbar_wait(&empty[s], (uint32_t)((it / kStages) - 1) & 1u, abort, g.wait_ns)) {
+                    const int s = (int)(it % NST);
+                    if (it >= NST && !mbar_wait(&empty[s], (uint32_t)((it / NST) - 1) & 1u, abort, g.wait_ns)) {
                         atomicExch(g.err, 1);
                         *abort = 1;
                         break;
                     }
                     uint8_t* st = stage0 + s * kStageBytes;
-                    mbar_expect_tx(&full[s], (uint32_t)kStageBytes);
-                    tma_load_3d(st, &tmA, kb * kBK, t.m0, t.za, &full[s]);                          // A hi
-                    tma_load_3d(st + kTileA, &tmA, g.Kh + kb * kBK, t.m0, t.za, &full[s]);          // A lo
-                    tma_load_3d(st + 2 * kTileA, &tmB, kb * kBK, t.n0, t.zb, &full[s]);             // B hi
-                    tma_load_3d(st + 2 * kTileA + kTileB, &tmB, g.Kh + kb * kBK, t.n0, t.zb, &full[s]);   // B lo
+                    if constexpr (PAIR) {
+                        if (rank == 0) mbar_expect_tx(&full[s], (uint32_t)(2 * kStageBytes));   // both CTAs' copies
+                        const uint32_t bar = mbar_of(&full[s], 0);
+                        const int n0 = t.n0 + (int)rank * kBN;                                   // this CTA's half of B
+                        tma_load_3d_pair(st, &tmA, kb * kBK, t.m0, t.za, bar);
+                        tma_load_3d_pair(st + kTileA, &tmA, g.Kh + kb * kBK, t.m0, t.za, bar);
+                        tma_load_3d_pair(st + 2 * kTileA, &tmB, kb * kBK, n0, t.zb, bar);
+                        tma_load_3d_pair(st + 2 * kTileA + kTileB, &tmB, g.Kh + kb * kBK, n0, t.zb, bar);
+                    } else {
+                        mbar_expect_tx(&full[s], (uint32_t)kStageBytes);
+                        tma_load_3d(st, &tmA, kb * kBK, t.m0, t.za, &full[s]);                          // A hi
+                        tma_load_3d(st + kTileA, &tmA, g.Kh + kb * kBK, t.m0, t.za, &full[s]);          // A lo
+                        tma_load_3d(st + 2 * kTileA, &tmB, kb * kBK, t.n0, t.zb, &full[s]);             // B hi
+                        tma_load_3d(st + 2 * kTileA + kTileB, &tmB, g.Kh + kb * kBK, t.n0, t.zb, &full[s]);   // B lo
+                    }
                 }
             }
             __syncwarp();
@@ -1108,12 +1206,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
             // let this CTA's own copies land before it exits (on every path: the
             // MMA thread may have stopped early): the last load of every stage
             // is that stage's newest phase
-            const int64_t first = it > kStages ? it - kStages : 0;
-            for (int64_t j = first; j < it; j++) mbar_wait_plain(&full[j % kStages], (uint32_t)(j / kStages) & 1u);
+            const int64_t first = it > NST ? it - NST : 0;
+            if (!PAIR)
+                for (int64_t j = first; j < it; j++) mbar_wait_plain(&full[j % NST], (uint32_t)(j / NST) & 1u);
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (lane == 0 && rank == 0) {
             int64_t it = 0, lt = 0;
             bool ok = true;
             for (int64_t tile = blockIdx.x; tile < n_tiles && !*abort && ok; tile += gridDim.x) {
@@ -1130,8 +1229,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                     tc_fence_after();
                     const int kb0 = sg * seg_kb, kb1 = kb0 + seg_kb < g.nkb ? kb0 + seg_kb : g.nkb;
                     for (int kb = kb0; kb < kb1; kb++, it++) {
-                        const int s = (int)(it % kStages);
-                        if (!mbar_wait(&full[s], (uint32_t)(it / kStages) & 1u, abort, g.wait_ns)) {
+                        const int s = (int)(it % NST);
+                        if (!mbar_wait(&full[s], (uint32_t)(it / NST) & 1u, abort, g.wait_ns)) {
                             atomicExch(g.err, 2);
                             *abort = 1;
                             ok = false;
@@ -1141,24 +1240,24 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                         const uint32_t sa = smem_u32(stage0 + s * kStageBytes);
                         const uint32_t sal = sa + kTileA, sb = sa + 2 * kTileA, sbl = sb + kTileB;
                         const int j = kb - kb0;
-                        const uint32_t acc = tmem + (uint32_t)((set * acc_per + j % acc_per) * kBN);
+                        const uint32_t acc = tmem + (uint32_t)((set * acc_per + j % acc_per) * TN);
                         const bool fresh = j < acc_per;
 #pragma unroll
                         for (int kk = 0; kk < kRowBytes / 32; kk++) {   // 32 bytes of K per MMA
                             const uint32_t o = kk * 32;
-                            umma<F>(acc, sdesc_sw128(sa + o), sdesc_sw128(sb + o), (fresh && kk == 0) ? 0u : 1u);
-                            umma<F>(acc, sdesc_sw128(sa + o), sdesc_sw128(sbl + o), 1u);
-                            umma<F>(acc, sdesc_sw128(sal + o), sdesc_sw128(sb + o), 1u);
+                            umma<F, PAIR>(acc, sdesc_sw128(sa + o), sdesc_sw128(sb + o), (fresh && kk == 0) ? 0u : 1u);
+                            umma<F, PAIR>(acc, sdesc_sw128(sa + o), sdesc_sw128(sbl + o), 1u);
+                            umma<F, PAIR>(acc, sdesc_sw128(sal + o), sdesc_sw128(sb + o), 1u);
                         }
-                        umma_commit(&empty[s]);   // stage free once these MMAs have read it
+                        umma_commit<PAIR>(&empty[s]);   // stage free once these MMAs have read it
                     }
                     if (!ok) break;
-                    umma_commit(&acc_full[set]);  // accumulators complete for this item
+                    umma_commit<PAIR>(&acc_full[set]);  // accumulators complete for this item
                 }
             }
             // MMAs still in flight finish before TMEM is freed (on every path: the
             // epilogue may have stopped early)
-            umma_commit(drain);
+            umma_commit<PAIR>(drain);
             mbar_wait_plain(drain, 0u);
         }
         __syncwarp();
@@ -1176,9 +1275,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
         // block: that step 23.9 -> 16.1 ms, one with four hyper bits (55 GB)
         // 12.7 -> 9.1 ms (6.0 TB/s); all GEMMs of the 10^6-shot job 149 -> 132 ms.
         const int ew = warp - 2, q = warp & 3;
-        const int c_lo = (ew >> 2) * (kBN / 2), c_hi = c_lo + kBN / 2;
-        int64_t* noff = noff_all + ew * (kBN / 2);
-        float* ucol = ucol_all + ew * (kBN / 2);
+        const int c_lo = (ew >> 2) * (TN / 2), c_hi = c_lo + TN / 2;
+        // this warp's columns, from c_lo / 2 on (a single CTA's tables have room for all)
+        int64_t* noff = noff_all + ew * (kBN / 2) - (PAIR ? c_lo / 2 : 0);
+        float* ucol = ucol_all + ew * (kBN / 2) - (PAIR ? c_lo / 2 : 0);
         float2* stg = stg_all + ew * 32 * kStgPitch;
         int sm_l = 0, row_l = 0;
         int64_t out_l = (q & 1 ? g.row_hi[0] : 0) + (q & 2 ? g.row_hi[1] : 0);
@@ -1190,18 +1290,24 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
             }
         int64_t lt = 0;
         bool live = true;
+        auto release_set = [&](int set) {
+            if constexpr (PAIR) mbar_arrive_cluster(mbar_of(&acc_empty[set], 0));
+            else mbar_arrive(&acc_empty[set]);
+        };
         TileQueue tq;
         TileInfo t, tn;
         bool more = tq.next(g, lane, tn);
         // FP16: this lane's row and column exponents of a tile's segment 0, read one
         // tile ahead (their latency would precede every tile of a short contraction)
-        int ea = 0, eb = 0;
-        auto read_exps = [&](const TileInfo& x, int sg, int& a, int& b) {
+        int ea = 0, eb = 0, eb1 = 0;   // (a pair's warp has 64 columns)
+        auto read_exps = [&](const TileInfo& x, int sg, int& a, int& b, int& b1) {
             const int64_t row = (int64_t)x.m0 + q * 32 + lane;
             a = row < x.row_end ? g.exp_a[((int64_t)x.za * g.M + row) * n_seg + sg] : 0;
-            b = g.exp_b[((int64_t)x.zb * (g.N2 >> 1) + (x.n0 >> 1) + (c_lo >> 1) + lane) * n_seg + sg];
+            const int64_t col = (int64_t)x.zb * (g.N2 >> 1) + (x.n0 >> 1) + (c_lo >> 1) + lane;
+            b = g.exp_b[col * n_seg + sg];
+            if (PAIR) b1 = g.exp_b[(col + 32) * n_seg + sg];
         };
-        if (F == FMT_FP16 && more) read_exps(tn, 0, ea, eb);
+        if (F == FMT_FP16 && more) read_exps(tn, 0, ea, eb, eb1);
         while (more && live) {
             if (__shfl_sync(0xffffffffu, *abort, 0)) break;   // warp-uniform stop
             t = tn;
@@ -1232,7 +1338,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
             __syncwarp();
             for (int sg = 0; sg < n_seg; sg++, lt++) {
                 const int set = (int)(lt % n_sets);
-                const uint32_t acc0 = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(set * acc_per * kBN);
+                const uint32_t acc0 = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(set * acc_per * TN);
                 const int seg_len = (sg + 1) * seg_kb < g.nkb ? seg_kb : g.nkb - sg * seg_kb;
                 const int n_acc = seg_len < acc_per ? seg_len : acc_per;
                 const bool add = sg > 0;   // later segments add to the running sum
@@ -1240,10 +1346,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                 // column scales 2^eb; their product 2^(ea + eb) is exact
                 float urow = 1.f;
                 if (F == FMT_FP16) {
-                    if (sg > 0) read_exps(t, sg, ea, eb);
+                    if (sg > 0) read_exps(t, sg, ea, eb, eb1);
                     ucol[c_lo / 2 + lane] = pow2f(eb);
+                    if (PAIR) ucol[c_lo / 2 + 32 + lane] = pow2f(eb1);
                     urow = pow2f(ea);
-                    if (sg + 1 == n_seg && more) read_exps(tn, 0, ea, eb);
+                    if (sg + 1 == n_seg && more) read_exps(tn, 0, ea, eb, eb1);
                     __syncwarp();
                 }
                 // one lane waits and the warp follows its outcome (lanes polling on
@@ -1292,7 +1399,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                         for (int j = 0; j < 16; j++) out[noff[(c0 >> 1) + j]] = make_float2(v[2 * j], v[2 * j + 1]);
                     }
                 };
-                if (n_seg == 1) {
+                if (!PAIR && n_seg == 1) {
 #pragma unroll 1
                     for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
                         // accumulators two at a time, added in order
@@ -1321,7 +1428,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                         if (c0 + 32 >= c_hi) {   // everything read: the set may take its next item while the tile is stored
                             tc_fence_before();
                             __syncwarp();
-                            if (lane == 0) mbar_arrive(&acc_empty[set]);
+                            if (lane == 0) release_set(set);
                         }
                         if (F == FMT_FP16) {
 #pragma unroll
@@ -1351,13 +1458,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                                 v[2 * j + 1] *= u;
                             }
                         }
-                        const uint32_t sa = tmem + ((uint32_t)(q * 32) << 16) + 2 * kBN + (uint32_t)c0;
+                        const uint32_t sa = tmem + ((uint32_t)(q * 32) << 16) + 2 * kBN + (uint32_t)c0;   // = kPairN
                         if (add) {
                             tmem_ld32(sa, r);
 #pragma unroll
                             for (int j = 0; j < 32; j++) v[j] += __uint_as_float(r[j]);
                         }
-                        if (sg + 1 < n_seg) {
+                        if (PAIR || sg + 1 < n_seg) {
 #pragma unroll
                             for (int j = 0; j < 32; j++) r[j] = __float_as_uint(v[j]);
                             tmem_st32(sa, r);
@@ -1366,25 +1473,54 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                         }
                     }
                 }
-                if (n_seg > 1) {
+                if (PAIR || n_seg > 1) {
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&acc_empty[set]);   // accumulators read: this set may take the next item
+                    if (lane == 0) release_set(set);   // accumulators read: this set may take the next item
+                }
+                if (PAIR && sg + 1 == n_seg) {         // the tile, from the running sum
+#pragma unroll 1
+                    for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
+                        float v[32];
+                        uint32_t r[32];
+                        tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(kPairN + c0), r);
+#pragma unroll
+                        for (int j = 0; j < 32; j++) v[j] = __uint_as_float(r[j]);
+                        store_chunk(c0, v);
+                    }
                 }
             }
         }
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) {
+        // The peer's MMAs read this CTA's shared memory and write its TMEM, and its
+        // barriers are signalled from here: both CTAs are done before either
+        // frees or leaves.  After a wait that ran out, copies may be in flight
+        // that no barrier of this CTA counts; a millisecond lets them land.
+        if (threadIdx.x == 0 && *abort)
+            for (const uint64_t t0 = global_ns(); global_ns() - t0 < 1000000ull;) {
+            }
+        __syncthreads();
+        cluster_sync();
+    }
     if (warp == 0) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+        if constexpr (PAIR)
+            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+        else
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    }
+    if constexpr (PAIR) {
+        __syncthreads();
+        cluster_sync();
     }
 }
 
 // Tiles of every trajectory group of a stacked GEMM (cnt[n_groups] = 0, so the
 // exclusive scan of cnt ends with the total).
-__global__ void k_group_tiles(const int32_t* __restrict__ net0, int64_t n_groups, int m_bits, int64_t tiles_n,
+__global__ void k_group_tiles(const int32_t* __restrict__ net0, int64_t n_groups, int m_bits, int64_t tiles_n, int pair,
                               int64_t* __restrict__ cnt) {
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g > n_groups) return;
@@ -1393,7 +1529,7 @@ __global__ void k_group_tiles(const int32_t* __restrict__ net0, int64_t n_groups
         return;
     }
     const int64_t r = (int64_t)(net0[g + 1] - net0[g]) << m_bits;
-    cnt[g] = ((r + kBM - 1) / kBM) * tiles_n;
+    cnt[g] = (((r + kBM - 1) / kBM + pair) & ~(int64_t)pair) * tiles_n;
 }
 
 // ---------------------------------------------------------- host helpers --
@@ -1478,19 +1614,17 @@ bool pack_tile_split(const PackArgs& p, int role, TileArgs& t) {
     struct Bit {
         int64_t stride, dst;
         bool k, in;
-    };
-    std::vector<Bit> bits;           // store order: summed bits, then rows
-    for (int i = 0; i < p.n_kb; i++) bits.push_back({p.k_stride[i], (int64_t)2 << i, true, i < 6});
-    for (int i = 0; i < p.n_rb; i++) bits.push_back({p.r_stride[i], row << i, false, false});
-    std::vector<int> order;
-    for (size_t i = 0; i < bits.size(); i++) order.push_back((int)i);
-    std::sort(order.begin(), order.end(), [&](int x, int y) { return bits[x].stride < bits[y].stride; });
-    if (order.size() < 5) return false;
+    } bits[2 * kMaxPackBits];        // store order: summed bits, then rows
+    int order[2 * kMaxPackBits], place[2 * kMaxPackBits] = {}, nb = 0;
+    for (int i = 0; i < p.n_kb; i++) bits[nb++] = {p.k_stride[i], (int64_t)2 << i, true, i < 6};
+    for (int i = 0; i < p.n_rb; i++) bits[nb++] = {p.r_stride[i], row << i, false, false};
+    for (int i = 0; i < nb; i++) order[i] = i;
+    std::sort(order, order + nb, [&](int x, int y) { return bits[x].stride < bits[y].stride; });
+    if (nb < 5) return false;
     for (int i = 0; i < 4; i++)
         if (bits[order[i]].stride != (int64_t)1 << i || bits[order[i]].k) return false;
     for (int i = 0; i < 5; i++) bits[order[i]].in = true;
-    std::vector<int> place(bits.size(), 0);
-    for (size_t i = 0; i < bits.size(); i++) {
+    for (int i = 0; i < nb; i++) {
         if (bits[i].in) {
             place[i] = 1 << t.nt;
             t.st_dst[t.nt++] = bits[i].dst;
@@ -1500,10 +1634,10 @@ bool pack_tile_split(const PackArgs& p, int role, TileArgs& t) {
         }
     }
     int n = 0;
-    for (int i : order)
-        if (bits[i].in) {
-            t.ld_stride[n] = bits[i].stride;
-            t.ld_place[n++] = place[i];
+    for (int i = 0; i < nb; i++)
+        if (bits[order[i]].in) {
+            t.ld_stride[n] = bits[order[i]].stride;
+            t.ld_place[n++] = place[order[i]];
         }
     return true;
 }
@@ -1644,7 +1778,13 @@ ptn_status run_gemm(const StepDesc& st, const ChunkCtx& ctx, int64_t n_inst, voi
     ga.n_nb = nn;
     ga.n_hb = nh;
     ga.tiles_m = (M + kBM - 1) / kBM;
-    ga.tiles_n = (2 * N + kBN - 1) / kBN;
+    // CTA pairs: segmented tiles with 256 columns, where every M tile has a
+    // neighbour or (stacked) the trajectories average at least kPairRows tiles of
+    // rows, so that few pairs are half empty
+    ga.pair = ga.nkb > kSegKb && 2 * N >= kPairN &&
+              (stacked ? n_inst * M >= kPairRows * kBM * grp.n_groups : ga.tiles_m >= 2);
+    ga.bn = ga.pair ? kPairN : kBN;
+    ga.tiles_n = (2 * N + ga.bn - 1) / ga.bn;
     while ((1ll << ga.tm_log) < ga.tiles_m) ga.tm_log++;
     while ((1ll << ga.tn_log) < ga.tiles_n) ga.tn_log++;
     ga.n_inst = n_inst;
@@ -1729,22 +1869,22 @@ ptn_status run_gemm(const StepDesc& st, const ChunkCtx& ctx, int64_t n_inst, voi
         int64_t acc = 0;   // the same count the device tile table ends with
         for (int64_t gi = 0; gi < grp.n_groups; gi++) {
             const int64_t r = (int64_t)(grp.h_net0[gi + 1] - grp.h_net0[gi]) * M;
-            acc += ((r + kBM - 1) / kBM) * ga.tiles_n;
+            acc += (((r + kBM - 1) / kBM + ga.pair) & ~(int64_t)ga.pair) * ga.tiles_n;
         }
         blocks = acc;
         count_launches(K_MISC);
         k_group_tiles<<<(unsigned)((grp.n_groups + 256) / 256), 256, 0, s>>>(grp.d_net0, grp.n_groups, nm,
-                                                                              ga.tiles_n, grp.d_cnt);
+                                                                              ga.tiles_n, ga.pair, grp.d_cnt);
         launch_exclusive_scan(grp.d_cnt, grp.d_tile0, grp.n_groups + 1, grp.d_scan, s);
     }
     if (ps) return ps;
     ps = make_map(&mB, pack_b, dt, kEB, 2 * Kh, 2 * N, pb.n_pinst * (1ll << nh), kBN);
     if (ps) return ps;
-    static const bool attr_set = [] {
-        cudaFuncSetAttribute(k_gemm<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
-        return true;
-    }();
-    (void)attr_set;
+    static std::once_flag done[64];
+    once_per_device(done, [] {
+        cudaFuncSetAttribute(k_gemm<F, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
+        cudaFuncSetAttribute(k_gemm<F, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem);
+    });
     if (blocks <= 0) return PTN_OK;
     const double flops = 8.0 * (double)n_inst * (double)(1ll << nh) * (double)M * (double)N * (double)Kc;
     const double bytes = 8.0 * ((double)n_inst * (1ll << nh) * M * N) +
@@ -1758,7 +1898,23 @@ ptn_status run_gemm(const StepDesc& st, const ChunkCtx& ctx, int64_t n_inst, voi
         return n > 0 ? n : 148;
     }();
     const int64_t grid = blocks < n_sm ? blocks : n_sm;
-    k_gemm<F><<<(unsigned)grid, kGemmThreads, kGemmSmem, s>>>(mA, mB, ga);
+    if (ga.pair) {
+        cudaLaunchConfig_t lc{};
+        lc.gridDim = dim3((unsigned)(grid & ~(int64_t)1));
+        lc.blockDim = dim3(kGemmThreads);
+        lc.dynamicSmemBytes = kGemmSmem;
+        lc.stream = s;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = 2;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        lc.attrs = &at;
+        lc.numAttrs = 1;
+        e = cudaLaunchKernelEx(&lc, k_gemm<F, true>, mA, mB, ga);
+        if (e != cudaSuccess) return set_error(PTN_ERR_CUDA, "gemm launch: %s", cudaGetErrorString(e));
+    } else {
+        k_gemm<F, false><<<(unsigned)grid, kGemmThreads, kGemmSmem, s>>>(mA, mB, ga);
+    }
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(PTN_ERR_CUDA, "gemm launch: %s", cudaGetErrorString(e));
     return PTN_OK;
