@@ -1011,7 +1011,7 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
 constexpr int kGemmThreads = 320;   // producer, MMA, 8 epilogue warps
 constexpr int64_t kPairRows = 4;    // least M tiles per trajectory of a stacked GEMM run by CTA pairs
 struct TileInfo {              // (rows and instances are TMA coordinates: 32 bits)
-    int inst, h, row_end, m0, n0, za, zb;
+    int inst, h, row_end, m0, n0, za, zb, out;   // out: instance written (unstacked)
 };
 __device__ __forceinline__ TileInfo decode_tile(const GemmArgs& g, int64_t tile) {
     TileInfo t;
@@ -1023,6 +1023,7 @@ __device__ __forceinline__ TileInfo decode_tile(const GemmArgs& g, int64_t tile)
         t.m0 = (int)(tm * kBM);
         t.n0 = (int)(tn * g.bn);
         t.row_end = g.M;
+        t.out = g.out_map ? g.out_map[t.inst] : t.inst;
         const int pa = g.a_pcls == g.out_cls ? t.inst : (g.a_pcls == CLS_TRAJ ? g.net_tl[t.inst] : 0);
         const int pb = g.b_pcls == g.out_cls ? t.inst : (g.b_pcls == CLS_TRAJ ? g.net_tl[t.inst] : 0);
         t.za = pa * g.n_h + t.h;
@@ -1041,7 +1042,7 @@ __device__ __forceinline__ TileInfo decode_tile(const GemmArgs& g, int64_t tile)
         t.m0 = (int)(r0 + (r % tmg) * kBM);
         t.n0 = (int)((r / tmg) * g.bn);
         t.inst = (int)lo;     // the trajectory (local index) supplies the B operand
-        t.h = 0;
+        t.h = t.out = 0;
         t.row_end = (int)r1;
         t.za = 0;
         t.zb = g.b_pcls == CLS_TRAJ ? (int)lo : 0;
@@ -1070,6 +1071,7 @@ struct TileQueue {
         t.n0 = __shfl_sync(0xffffffffu, mine.n0, l);
         t.za = __shfl_sync(0xffffffffu, mine.za, l);
         t.zb = __shfl_sync(0xffffffffu, mine.zb, l);
+        t.out = __shfl_sync(0xffffffffu, mine.out, l);
         i++;
         return true;
     }
@@ -1109,7 +1111,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
     uint64_t* drain = acc_empty + 2;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
-    int64_t* noff_all = reinterpret_cast<int64_t*>(tslot + 4);   // 8 epilogue warps x kBN / 2 column offsets
+    // tables of the 8 epilogue warps, 16-byte aligned (the scales are read four at
+    // a time; the barriers before them end 8 bytes past a boundary)
+    constexpr int kTabOff = (int)(((2 * NST + 5) * 8 + 16 + 15) & ~15);
+    static_assert(kTabOff % 16 == 0 && kTabOff + 8 * (kBN / 2) * 12 <= kTabBytes, "epilogue tables");
+    int64_t* noff_all = reinterpret_cast<int64_t*>(smem + kStages * kStageBytes + kTabOff);   // kBN / 2 column offsets each
     float* ucol_all = reinterpret_cast<float*>(noff_all + 8 * (kBN / 2));   // FP16: column scales 2^eb
     float2* stg_all = reinterpret_cast<float2*>(smem + kStages * kStageBytes + kTabBytes);   // staged fragments
     const uint32_t rank = PAIR ? cluster_rank() : 0u;
@@ -1322,7 +1328,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
             }
             const int64_t row = (int64_t)t.m0 + q * 32 + lane;
             const int64_t row0 = g.staged ? (int64_t)t.m0 : row;   // staged: the tile's first row
-            int64_t m = row0, out_inst = g.out_map ? g.out_map[t.inst] : t.inst;
+            int64_t m = row0, out_inst = t.out;
             if (g.stacked) {
                 out_inst = row0 >> g.m_bits;
                 m = row0 & (((int64_t)1 << g.m_bits) - 1);
@@ -1432,10 +1438,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                         }
                         if (F == FMT_FP16) {
 #pragma unroll
-                            for (int j = 0; j < 16; j++) {
-                                const float u = urow * ucol[(c0 >> 1) + j];
-                                v[2 * j] *= u;
-                                v[2 * j + 1] *= u;
+                            for (int j = 0; j < 16; j += 4) {
+                                const float4 u4 = *reinterpret_cast<const float4*>(ucol + (c0 >> 1) + j);
+                                const float u[4] = {urow * u4.x, urow * u4.y, urow * u4.z, urow * u4.w};
+#pragma unroll
+                                for (int i = 0; i < 4; i++) {
+                                    v[2 * (j + i)] *= u[i];
+                                    v[2 * (j + i) + 1] *= u[i];
+                                }
                             }
                         }
                         store_chunk(c0, v);
@@ -1452,10 +1462,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                         for (int j = 0; j < 32; j++) v[j] = __uint_as_float(r[j]);
                         if (F == FMT_FP16) {
 #pragma unroll
-                            for (int j = 0; j < 16; j++) {
-                                const float u = urow * ucol[(c0 >> 1) + j];
-                                v[2 * j] *= u;
-                                v[2 * j + 1] *= u;
+                            for (int j = 0; j < 16; j += 4) {
+                                const float4 u4 = *reinterpret_cast<const float4*>(ucol + (c0 >> 1) + j);
+                                const float u[4] = {urow * u4.x, urow * u4.y, urow * u4.z, urow * u4.w};
+#pragma unroll
+                                for (int i = 0; i < 4; i++) {
+                                    v[2 * (j + i)] *= u[i];
+                                    v[2 * (j + i) + 1] *= u[i];
+                                }
                             }
                         }
                         const uint32_t sa = tmem + ((uint32_t)(q * 32) << 16) + 2 * kBN + (uint32_t)c0;   // = kPairN
