@@ -337,13 +337,11 @@ static void launch_micro(const StepDesc* d_step, const ChunkCtx& ctx, int64_t n_
     k_contract_micro<RA, RB><<<(unsigned)blocks, kDirThreads, 0, s>>>(d_step, ctx, n_inst, mb);
 }
 
-// SIMT contraction with both operands' summed axis contiguous (every step whose
-// operands were laid out for it): the rows a CTA needs are staged in shared
-// memory 16 terms at a time.  The kernels above let each thread walk its own
-// rows, and neighbouring lanes' rows lie a whole row apart: at 64 terms (512
-// bytes) the lines of all resident threads exceed L1 and every 8-byte read
-// fetches a sector again (the middle 30-qubit block's network step read at 131
-// GB/s).  Here a row chunk is copied once by consecutive 16-byte cp.async and
+// SIMT contraction staged in shared memory: the rows a CTA needs, 16 terms at a
+// time.  The kernels above let each thread walk its own rows, and neighbouring
+// lanes' rows lie a whole row apart: at 64 terms (512 bytes) the lines of all
+// resident threads exceed L1 and every 8-byte read fetches a sector again (the
+// middle 30-qubit block's network step read at 131 GB/s).  Here a row chunk is copied once by consecutive 16-byte cp.async and
 // read back two terms at a time; rows are pitched by one extra 16-byte slot, so
 // the eight lanes of a 128-bit shared read hit different banks.  Three stages,
 // one barrier per chunk: the copies of the chunk after next are in flight while
@@ -354,6 +352,11 @@ static void launch_micro(const StepDesc* d_step, const ChunkCtx& ctx, int64_t n_
 // increasing order within 256, blocks of 256 in Gray-code order.  Measured
 // against the micro-tiles: 1024 terms, 4096 trajectories 5.47 -> 1.81 ms (5.3
 // TB/s); 64 terms, 1024 outputs, 10,240 networks 0.65 -> 0.18 ms.
+// GATHER: an operand whose summed axis is not contiguous (a mirrored buffer, an
+// adjoint step) has no 16-byte pieces; its rows are copied 8 bytes at a time,
+// lanes over rows, whose strides are the low ones there.  32 terms, 2^14 outputs,
+// 1024 trajectories 0.49 -> 0.166 ms.  A variant of its own: the plain copy loop keeps
+// its registers.
 constexpr int kRowsMax = 10;          // row bits per operand, sub-tile bits, thread-tile bits
 constexpr int kRowsChunk = 16;        // terms per stage
 constexpr int kRowsStages = 3;
@@ -365,6 +368,8 @@ struct RowsArgs {
     int32_t rb[2];                     // log2 rows staged per operand
     int32_t r_stride[2][kRowsMax];     // operand stride of each row bit
     int32_t n_sub, n_lane, n_sum, kc_log;
+    int32_t k_stride[2][8];            // summed strides of an operand whose summed axis is not contiguous
+    int32_t gather[2];                 // that operand: its rows are copied 8 bytes at a time
     int32_t sub_stride[2][kMaxOut];    // sub-tile bits: operand strides, output strides
     int64_t sub_out[kMaxOut];
     int32_t lane_row[2][kRowsMax];     // thread index bits: row weights, output strides
@@ -372,6 +377,9 @@ struct RowsArgs {
     int32_t tile_row_a[2], tile_row_b[2], tile_out_a[2], tile_out_b[2];   // micro-tile bits
 };
 
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
@@ -388,7 +396,7 @@ __device__ __forceinline__ void rows_terms(float2& acc, const float4& a, const f
     acc.y = fmaf(a.w, b.z, acc.y);
 }
 
-template <int RA, int RB>
+template <int RA, int RB, bool GATHER>
 __global__ void __launch_bounds__(256) k_contract_rows(const StepDesc* __restrict__ s, const __grid_constant__ ChunkCtx c,
                                                        const int64_t n_inst, const __grid_constant__ RowsArgs r) {
     extern __shared__ __align__(16) uint8_t rows_smem[];
@@ -433,13 +441,35 @@ __global__ void __launch_bounds__(256) k_contract_rows(const StepDesc* __restric
                 const int hi = k0 >> 8;
                 k0 = ((hi ^ (hi >> 1)) << 8) | (k0 & 255);
             }
-            const float2* pa = ptr[u & 3][0] + k0;
-            const float2* pb = ptr[u & 3][1] + k0;
             const uint32_t st = static_cast<uint32_t>(__cvta_generic_to_shared(stage0 + (int)(it % kRowsStages) * stage_elems));
-            const int n = rows << piece_log;
-            for (int i = threadIdx.x; i < n; i += blockDim.x) {
-                const int row = i >> piece_log, pc = i & ((1 << piece_log) - 1);
-                cp_async16(st + (uint32_t)(row * pitch + 2 * pc) * 8u, (row < rows_a ? pa : pb) + row_off[row] + 2 * pc);
+            if constexpr (!GATHER) {
+                const float2* pa = ptr[u & 3][0] + k0;
+                const float2* pb = ptr[u & 3][1] + k0;
+                const int n = rows << piece_log;
+                for (int i = threadIdx.x; i < n; i += blockDim.x) {
+                    const int row = i >> piece_log, pc = i & ((1 << piece_log) - 1);
+                    cp_async16(st + (uint32_t)(row * pitch + 2 * pc) * 8u, (row < rows_a ? pa : pb) + row_off[row] + 2 * pc);
+                }
+            } else {
+                for (int o = 0; o < 2; o++) {
+                    const float2* p = ptr[u & 3][o];
+                    const int row0 = o ? rows_a : 0, n_rows = 1 << r.rb[o];
+                    if (!r.gather[o]) {
+                        for (int i = threadIdx.x; i < n_rows << piece_log; i += blockDim.x) {
+                            const int row = row0 + (i >> piece_log), pc = i & ((1 << piece_log) - 1);
+                            cp_async16(st + (uint32_t)(row * pitch + 2 * pc) * 8u, p + k0 + row_off[row] + 2 * pc);
+                        }
+                    } else {               // lanes over rows: their strides are the low ones here
+                        for (int i = threadIdx.x; i < n_rows << r.kc_log; i += blockDim.x) {
+                            const int row = row0 + (i & (n_rows - 1)), k = i >> r.rb[o];
+                            int ko = 0;
+#pragma unroll
+                            for (int b = 0; b < 8; b++)
+                                if (b < r.n_sum && (((k0 + k) >> b) & 1)) ko += r.k_stride[o][b];
+                            cp_async8(st + (uint32_t)(row * pitch + k) * 8u, p + row_off[row] + ko);
+                        }
+                    }
+                }
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -727,8 +757,8 @@ __global__ void __launch_bounds__(256) k_contract_group(const StepDesc* __restri
 
 // Split of a step for k_contract_rows (shared < 0) or, with operand `shared`
 // kept for a group of 2^g_log networks, k_contract_group; false where it does
-// not apply: a summed axis that is not contiguous in both operands, 16-byte
-// misaligned rows, or more bits than the tables hold.
+// not apply: 16-byte misaligned rows, more bits than the tables hold, or (a
+// group, or more than 256 terms) a summed axis that is not contiguous.
 bool rows_split(const StepDesc& h, const ChunkCtx& ctx, int shared, int g_log, RowsArgs& r, int& ra, int& rb, int& smem) {
     memset(&r, 0, sizeof r);
     if (h.n_sum < kRowsMinSum || h.n_out < 1 || h.out_size >= (1ll << 31)) return false;
@@ -738,10 +768,16 @@ bool rows_split(const StepDesc& h, const ChunkCtx& ctx, int shared, int g_log, R
     if (h.n_sum == 3 && h.n_out < 9) return false;
     for (int o = 0; o < 2; o++) {
         const OperandDesc& d = h.op[o];
+        if (d.inst_size >= (1ll << 31)) return false;
         for (int q = 0; q < h.n_sum; q++)
-            if (h.sum_stride[o][q] != (int64_t)1 << q) return false;
+            if (h.sum_stride[o][q] != (int64_t)1 << q) r.gather[o] = 1;
+        if (r.gather[o]) {
+            if (shared >= 0 || h.n_sum > 8) return false;
+            for (int q = 0; q < h.n_sum; q++) r.k_stride[o][q] = (int32_t)h.sum_stride[o][q];
+            continue;
+        }
         const int64_t base = d.mode == OP_LEAF ? d.leaf_base : d.arena_off * ctx.arena_inst[d.arena];
-        if ((base | d.inst_size) & 1 || d.inst_size >= (1ll << 31)) return false;
+        if ((base | d.inst_size) & 1) return false;
         for (int p = 0; p < h.n_out; p++)
             if (h.out_stride[o][p] & 1) return false;
         for (int p = 0; p < d.n_slice; p++)
@@ -846,7 +882,8 @@ void launch_rows_t(const StepDesc* d_step, const ChunkCtx& ctx, int64_t n_inst, 
                    cudaStream_t s) {
     static std::once_flag done[64];
     once_per_device(done, [] {
-        cudaFuncSetAttribute(k_contract_rows<RA, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowsSmem);
+        cudaFuncSetAttribute(k_contract_rows<RA, RB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowsSmem);
+        cudaFuncSetAttribute(k_contract_rows<RA, RB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowsSmem);
         cudaFuncSetAttribute(k_contract_group<RA, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGroupSmem);
     });
     const int threads = std::max(64, 1 << g.r.n_lane);
@@ -856,7 +893,11 @@ void launch_rows_t(const StepDesc* d_step, const ChunkCtx& ctx, int64_t n_inst, 
         k_contract_group<RA, RB><<<(unsigned)std::min(units, cap), threads, smem, s>>>(d_step, ctx, g);
     } else {
         const int64_t units = n_inst << g.r.n_sub;
-        k_contract_rows<RA, RB><<<(unsigned)std::min(units, cap), threads, smem, s>>>(d_step, ctx, n_inst, g.r);
+        const unsigned grid = (unsigned)std::min(units, cap);
+        if (g.r.gather[0] | g.r.gather[1])
+            k_contract_rows<RA, RB, true><<<grid, threads, smem, s>>>(d_step, ctx, n_inst, g.r);
+        else
+            k_contract_rows<RA, RB, false><<<grid, threads, smem, s>>>(d_step, ctx, n_inst, g.r);
     }
 }
 
