@@ -1009,6 +1009,7 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
 // set (acc_empty), and the epilogue starts after the item's last MMA
 // completes (acc_full).  Every wait is bounded.
 constexpr int kGemmThreads = 320;   // producer, MMA, 8 epilogue warps
+constexpr int kPairKb = 8;          // least k-blocks run by CTA pairs (2 segments of 4)
 constexpr int64_t kPairRows = 4;    // least M tiles per trajectory of a stacked GEMM run by CTA pairs
 struct TileInfo {              // (rows and instances are TMA coordinates: 32 bits)
     int inst, h, row_end, m0, n0, za, zb, out;   // out: instance written (unstacked)
@@ -1084,17 +1085,21 @@ __device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) 
 // read 96 KB and TMA writes 64 KB, 1280 clocks at 128 bytes each, and takes 1370
 // to 1430 where the MMAs alone take 768 (64 clocks each with resident operands);
 // a pair of 128 columns measured the same 1380.  With 256 columns a CTA's k-block
-// has twice the work for the same 64 KB written.  The accumulator and the running
-// sum then fill TMEM, so only segmented tiles run so: one accumulator set, freed
-// for the next segment as soon as it is added to the sum (the last segment too,
-// before the tile is stored from the sum).  The even CTA leads: its producer
-// counts both CTAs' bytes, its MMA thread issues for both and signals freed
-// stages and finished accumulators to both, and both CTAs' epilogue warps free
-// the accumulator at its barrier.  The products, their order and the segments are
-// those of one CTA, so every output is the same.  Measured: the middle 30-qubit
-// block's step of 4096 terms (FP16 hi/lo) 64.3 -> 53.3 ms (518 TFLOP/s, 0.95 of
-// the sustained peak / 3 with its padded rows), 512 terms of the 16-qubit state
-// (TF32) 9.57 -> 6.63 ms (331 TFLOP/s).
+// has twice the work for the same 64 KB written.  Two accumulators of a pair fill
+// TMEM, so its tiles are summed from segments of one accumulator: the first one
+// stays where it is, the others are accumulated beside it and added to it, and the
+// two regions change places from tile to tile, so that a tile is stored while the
+// next one's first segment runs.  Long contractions have segments anyway; those of
+// 8 and 16 k-blocks run their 2 and 4 accumulators (every second, every fourth
+// k-block) one after the other.  The even CTA leads: its producer counts both
+// CTAs' bytes, its MMA thread issues for both and signals freed stages and finished
+// accumulators to both, and both CTAs' epilogue warps free a region at its barrier.
+// The products, their order and the order of the sums are those of one CTA, so
+// every output is the same.  Measured: the middle 30-qubit block's step of 4096
+// terms (FP16 hi/lo) 64.3 -> 51.8 to 53.5 ms (516 to 533 TFLOP/s, 0.95 of the
+// sustained peak / 3 with its padded rows), its 256 terms by 2^18 outputs 4.34 ->
+// 3.79 ms; of the 16-qubit state (TF32) 512 terms 9.57 -> 6.20 ms (355 TFLOP/s),
+// 256 terms 11.26 -> 8.53 ms.
 template <int F, bool PAIR>
 __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant__ CUtensorMap tmA,
                                                           const __grid_constant__ CUtensorMap tmB,
@@ -1126,9 +1131,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
     // running sum kept in TMEM columns [2 kBN, 3 kBN), then writes the tile
     // once.  Segmented tiles use two accumulator sets of one accumulator, short
     // contractions (at most 8 k-blocks) two sets of kAcc / 2 (the epilogue of
-    // one item overlaps the MMAs of the next); the others one set of kAcc.  A
-    // pair's accumulator takes columns [0, kPairN), its running sum the rest.
-    const int seg_kb = g.nkb > kSegKb ? kSegKb : g.nkb;
+    // one item overlaps the MMAs of the next); the others one set of kAcc.
+    // A pair runs the accumulators of a short contraction (k-blocks j, j + n_seg,
+    // ... of accumulator j) one after the other, as segments (`split`).
+    const bool split = PAIR && g.nkb <= kSegKb;
+    const int n_scale = (g.nkb + kSegKb - 1) / kSegKb;   // FP16 scales per row and column
+    const int split_acc = g.nkb <= 8 ? kAcc / 2 : kAcc;
+    const int seg_kb = split ? g.nkb / split_acc : (g.nkb > kSegKb ? kSegKb : g.nkb);
     const int n_seg = (g.nkb + seg_kb - 1) / seg_kb;
     const int n_sets = !PAIR && (g.nkb <= 8 || n_seg > 1) ? 2 : 1;
     const int acc_per = n_seg > 1 ? 1 : kAcc / n_sets;
@@ -1181,7 +1190,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
         TileInfo t;
         while (!__shfl_sync(0xffffffffu, *abort, 0) && tq.next(g, lane, t)) {
             if (lane == 0) {
-                for (int kb = 0; kb < g.nkb; kb++, it++) {
+                for (int i = 0; i < g.nkb; i++, it++) {
+                    const int kb = split ? i % seg_kb * n_seg + i / seg_kb : i;
                     const int s = (int)(it % NST);
                     if (it >= NST && !mbar_wait(&empty[s], (uint32_t)((it / NST) - 1) & 1u, abort, g.wait_ns)) {
                         atomicExch(g.err, 1);
@@ -1221,12 +1231,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
         if (lane == 0 && rank == 0) {
             int64_t it = 0, lt = 0;
             bool ok = true;
+            uint32_t used = 0, phase = 0, x = 1;   // a pair: regions used, their waits' parities, the tile's sum
             for (int64_t tile = blockIdx.x; tile < n_tiles && !*abort && ok; tile += gridDim.x) {
+                x ^= 1;
                 for (int sg = 0; sg < n_seg && ok; sg++, lt++) {
-                    const int set = (int)(lt % n_sets);
+                    const int set = PAIR ? (int)(sg ? x ^ 1 : x) : (int)(lt % n_sets);
+                    const bool again = PAIR ? (used >> set) & 1 : lt >= n_sets;
+                    const uint32_t parity = PAIR ? (phase >> set) & 1 : (uint32_t)((lt / n_sets - 1) & 1);
+                    if (again) phase ^= 1u << set;
+                    used |= 1u << set;
                     // this set's previous item has been drained by the epilogue
-                    if (lt >= n_sets &&
-                        !mbar_wait(&acc_empty[set], (uint32_t)((lt / n_sets - 1) & 1), abort, g.wait_ns)) {
+                    if (again && !mbar_wait(&acc_empty[set], parity, abort, g.wait_ns)) {
                         atomicExch(g.err, 4);
                         *abort = 1;
                         ok = false;
@@ -1295,6 +1310,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                 out_l += g.frag_out[b + 1];
             }
         int64_t lt = 0;
+        uint32_t phase = 0, x = 1;   // a pair: parities of the regions' waits, the tile's running sum
         bool live = true;
         auto release_set = [&](int set) {
             if constexpr (PAIR) mbar_arrive_cluster(mbar_of(&acc_empty[set], 0));
@@ -1308,10 +1324,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
         int ea = 0, eb = 0, eb1 = 0;   // (a pair's warp has 64 columns)
         auto read_exps = [&](const TileInfo& x, int sg, int& a, int& b, int& b1) {
             const int64_t row = (int64_t)x.m0 + q * 32 + lane;
-            a = row < x.row_end ? g.exp_a[((int64_t)x.za * g.M + row) * n_seg + sg] : 0;
+            a = row < x.row_end ? g.exp_a[((int64_t)x.za * g.M + row) * n_scale + sg] : 0;
             const int64_t col = (int64_t)x.zb * (g.N2 >> 1) + (x.n0 >> 1) + (c_lo >> 1) + lane;
-            b = g.exp_b[col * n_seg + sg];
-            if (PAIR) b1 = g.exp_b[(col + 32) * n_seg + sg];
+            b = g.exp_b[col * n_scale + sg];
+            if (PAIR) b1 = g.exp_b[(col + 32) * n_scale + sg];
         };
         if (F == FMT_FP16 && more) read_exps(tn, 0, ea, eb, eb1);
         while (more && live) {
@@ -1342,27 +1358,31 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
             const int row_lim = min(t.row_end - t.m0, 128) - q * 32;   // valid rows of this quadrant
             float2* out = g.out + (row_ok || g.staged ? out_inst : 0) * g.out_size + moff + (g.staged ? out_l : 0);
             __syncwarp();
+            x ^= 1;
+            float urow = 1.f;
             for (int sg = 0; sg < n_seg; sg++, lt++) {
-                const int set = (int)(lt % n_sets);
+                const int set = PAIR ? (int)(sg ? x ^ 1 : x) : (int)(lt % n_sets);
                 const uint32_t acc0 = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(set * acc_per * TN);
                 const int seg_len = (sg + 1) * seg_kb < g.nkb ? seg_kb : g.nkb - sg * seg_kb;
                 const int n_acc = seg_len < acc_per ? seg_len : acc_per;
                 const bool add = sg > 0;   // later segments add to the running sum
                 // FP16: the segment's A row scale 2^ea (packed row za * M + row) and
                 // column scales 2^eb; their product 2^(ea + eb) is exact
-                float urow = 1.f;
-                if (F == FMT_FP16) {
+                if (F == FMT_FP16 && !(split && sg)) {
                     if (sg > 0) read_exps(t, sg, ea, eb, eb1);
+                    __syncwarp();        // the previous segment's scales are no longer read
                     ucol[c_lo / 2 + lane] = pow2f(eb);
                     if (PAIR) ucol[c_lo / 2 + 32 + lane] = pow2f(eb1);
                     urow = pow2f(ea);
-                    if (sg + 1 == n_seg && more) read_exps(tn, 0, ea, eb, eb1);
+                    if ((split || sg + 1 == n_seg) && more) read_exps(tn, 0, ea, eb, eb1);
                     __syncwarp();
                 }
                 // one lane waits and the warp follows its outcome (lanes polling on
                 // their own could disagree when a wait gives up)
                 int ok = 1;
-                if (lane == 0) ok = mbar_wait(&acc_full[set], (uint32_t)((lt / n_sets) & 1), abort, g.wait_ns) ? 1 : 0;
+                const uint32_t parity = PAIR ? (phase >> set) & 1 : (uint32_t)((lt / n_sets) & 1);
+                phase ^= 1u << set;
+                if (lane == 0) ok = mbar_wait(&acc_full[set], parity, abort, g.wait_ns) ? 1 : 0;
                 ok = __shfl_sync(0xffffffffu, ok, 0);
                 if (!ok) {
                     if (lane == 0) {
@@ -1405,7 +1425,67 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                         for (int j = 0; j < 16; j++) out[noff[(c0 >> 1) + j]] = make_float2(v[2 * j], v[2 * j + 1]);
                     }
                 };
-                if (!PAIR && n_seg == 1) {
+                auto scale_chunk = [&](int c0, float (&v)[32]) {   // FP16: by the row's and the columns' scales
+#pragma unroll
+                    for (int j = 0; j < 16; j += 4) {
+                        const float4 u4 = *reinterpret_cast<const float4*>(ucol + (c0 >> 1) + j);
+                        const float u[4] = {urow * u4.x, urow * u4.y, urow * u4.z, urow * u4.w};
+#pragma unroll
+                        for (int i = 0; i < 4; i++) {
+                            v[2 * (j + i)] *= u[i];
+                            v[2 * (j + i) + 1] *= u[i];
+                        }
+                    }
+                };
+                if constexpr (PAIR) {
+                    // the tile's first segment stays where it is and the others are
+                    // added to it; the other region is free again after each
+                    const uint32_t sum = tmem + ((uint32_t)(q * 32) << 16) + x * TN;
+                    const bool scale = F == FMT_FP16 && !split;   // per segment (else once, before the stores)
+                    if (sg > 0 || scale) {
+#pragma unroll 1
+                        for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
+                            float v[32];
+                            uint32_t r[32], r2[32];
+                            tmem_ld32_issue(acc0 + (uint32_t)c0, r);
+                            if (sg > 0) tmem_ld32_issue(sum + (uint32_t)c0, r2);
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int j = 0; j < 32; j++) v[j] = __uint_as_float(r[j]);
+                            if (scale) scale_chunk(c0, v);
+                            if (sg > 0) {
+#pragma unroll
+                                for (int j = 0; j < 32; j++) v[j] += __uint_as_float(r2[j]);
+                            }
+#pragma unroll
+                            for (int j = 0; j < 32; j++) r[j] = __float_as_uint(v[j]);
+                            tmem_st32(sum + (uint32_t)c0, r);
+                        }
+                    }
+                    if (sg > 0) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) release_set(set);
+                    }
+                    if (sg + 1 < n_seg) continue;
+#pragma unroll 1
+                    for (int c0 = c_lo; c0 < c_hi; c0 += 32) {   // the tile, while the next one starts
+                        float v[32];
+                        uint32_t r[32];
+                        tmem_ld32(sum + (uint32_t)c0, r);
+                        if (c0 + 32 >= c_hi) {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) release_set((int)x);
+                        }
+#pragma unroll
+                        for (int j = 0; j < 32; j++) v[j] = __uint_as_float(r[j]);
+                        if (F == FMT_FP16 && split) scale_chunk(c0, v);
+                        store_chunk(c0, v);
+                    }
+                    continue;
+                }
+                if (n_seg == 1) {
 #pragma unroll 1
                     for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
                         // accumulators two at a time, added in order
@@ -1436,18 +1516,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                             __syncwarp();
                             if (lane == 0) release_set(set);
                         }
-                        if (F == FMT_FP16) {
-#pragma unroll
-                            for (int j = 0; j < 16; j += 4) {
-                                const float4 u4 = *reinterpret_cast<const float4*>(ucol + (c0 >> 1) + j);
-                                const float u[4] = {urow * u4.x, urow * u4.y, urow * u4.z, urow * u4.w};
-#pragma unroll
-                                for (int i = 0; i < 4; i++) {
-                                    v[2 * (j + i)] *= u[i];
-                                    v[2 * (j + i) + 1] *= u[i];
-                                }
-                            }
-                        }
+                        if (F == FMT_FP16) scale_chunk(c0, v);
                         store_chunk(c0, v);
                     }
                 } else {
@@ -1460,25 +1529,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                         tmem_ld32(acc0 + (uint32_t)c0, r);
 #pragma unroll
                         for (int j = 0; j < 32; j++) v[j] = __uint_as_float(r[j]);
-                        if (F == FMT_FP16) {
-#pragma unroll
-                            for (int j = 0; j < 16; j += 4) {
-                                const float4 u4 = *reinterpret_cast<const float4*>(ucol + (c0 >> 1) + j);
-                                const float u[4] = {urow * u4.x, urow * u4.y, urow * u4.z, urow * u4.w};
-#pragma unroll
-                                for (int i = 0; i < 4; i++) {
-                                    v[2 * (j + i)] *= u[i];
-                                    v[2 * (j + i) + 1] *= u[i];
-                                }
-                            }
-                        }
-                        const uint32_t sa = tmem + ((uint32_t)(q * 32) << 16) + 2 * kBN + (uint32_t)c0;   // = kPairN
+                        if (F == FMT_FP16) scale_chunk(c0, v);
+                        const uint32_t sa = tmem + ((uint32_t)(q * 32) << 16) + 2 * kBN + (uint32_t)c0;
                         if (add) {
                             tmem_ld32(sa, r);
 #pragma unroll
                             for (int j = 0; j < 32; j++) v[j] += __uint_as_float(r[j]);
                         }
-                        if (PAIR || sg + 1 < n_seg) {
+                        if (sg + 1 < n_seg) {
 #pragma unroll
                             for (int j = 0; j < 32; j++) r[j] = __float_as_uint(v[j]);
                             tmem_st32(sa, r);
@@ -1487,21 +1545,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                         }
                     }
                 }
-                if (PAIR || n_seg > 1) {
+                if (n_seg > 1) {
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) release_set(set);   // accumulators read: this set may take the next item
-                }
-                if (PAIR && sg + 1 == n_seg) {         // the tile, from the running sum
-#pragma unroll 1
-                    for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
-                        float v[32];
-                        uint32_t r[32];
-                        tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(kPairN + c0), r);
-#pragma unroll
-                        for (int j = 0; j < 32; j++) v[j] = __uint_as_float(r[j]);
-                        store_chunk(c0, v);
-                    }
                 }
             }
         }
@@ -1792,10 +1839,18 @@ ptn_status run_gemm(const StepDesc& st, const ChunkCtx& ctx, int64_t n_inst, voi
     ga.n_nb = nn;
     ga.n_hb = nh;
     ga.tiles_m = (M + kBM - 1) / kBM;
-    // CTA pairs: segmented tiles with 256 columns, where every M tile has a
-    // neighbour or (stacked) the trajectories average at least kPairRows tiles of
-    // rows, so that few pairs are half empty
-    ga.pair = ga.nkb > kSegKb && 2 * N >= kPairN &&
+    // CTA pairs: at least two segments of 4 k-blocks and 256 columns, more 128 x 128
+    // tiles than SMs (fewer finish in one wave, where a pair's tile takes longer),
+    // and every M tile has a neighbour or (stacked) the trajectories average at
+    // least kPairRows tiles of rows, so that few pairs are half empty
+    static const int n_sm = [] {
+        int dev = 0, n = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        return n > 0 ? n : 148;
+    }();
+    const int64_t rows_all = stacked ? n_inst * M : ga.tiles_m * kBM * (n_inst << nh);
+    ga.pair = ga.nkb >= kPairKb && 2 * N >= kPairN && rows_all / kBM * (2 * N / kBN) > n_sm &&
               (stacked ? n_inst * M >= kPairRows * kBM * grp.n_groups : ga.tiles_m >= 2);
     ga.bn = ga.pair ? kPairN : kBN;
     ga.tiles_n = (2 * N + ga.bn - 1) / ga.bn;
@@ -1905,12 +1960,6 @@ ptn_status run_gemm(const StepDesc& st, const ChunkCtx& ctx, int64_t n_inst, voi
                          (double)kEB * 2 * Kh * ((double)pa.n_pinst * M + (double)pb.n_pinst * 2 * N) * (1ll << nh);
     StatScope sc(K_CONTRACT_GEMM, s, bytes, flops);
     ga.n_tiles = blocks;
-    static const int n_sm = [] {
-        int dev = 0, n = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        return n > 0 ? n : 148;
-    }();
     const int64_t grid = blocks < n_sm ? blocks : n_sm;
     if (ga.pair) {
         cudaLaunchConfig_t lc{};
