@@ -51,11 +51,14 @@ constexpr int kTileA = kBM * kRowBytes;
 constexpr int kTileB = kBN * kRowBytes;
 constexpr int kStageBytes = 2 * kTileA + 2 * kTileB;
 constexpr int kPairN = 2 * kBN;   // columns of a CTA pair's tile (k_gemm<F, true>): 128 B rows staged by each CTA
-// epilogue staging: per epilogue warp a fragment of 32 rows x 8 complex columns,
-// rows padded to 9 slots (the 8-byte writes of a column and most reads hit
-// different banks)
-constexpr int kStgPitch = 9;
-constexpr int kStgBytes = 8 * 32 * kStgPitch * 8;
+// epilogue staging: per epilogue warp a fragment of 32 rows x 8 complex columns.
+// Its elements are placed so that a half-warp's 8-byte accesses hit 16 different
+// bank pairs both when written by row and when read in the order of the output
+// (run_gemm): a 128 x 128 tile's operands already take 1280 clocks of shared memory
+// per k-block, and with rows padded to 9 slots 9.1 of 16.5 million wavefronts of
+// the 2^20 outputs by 128 terms were conflicts (14.2 -> 13.4 ms).
+constexpr int kStgElems = 32 * 8;
+constexpr int kStgBytes = 8 * kStgElems * 8;
 constexpr int kTabBytes = 8192;   // barriers, TMEM slot, per-warp column offsets and FP16 column scales
 constexpr int kGemmSmem = 1024 + kStages * kStageBytes + kTabBytes + kStgBytes;   // align slack + stages + tables + staging
 constexpr int kMaxPackBits = 40;
@@ -123,7 +126,8 @@ struct GemmArgs {
     // over the lanes, bits 6-7 over its four stores.
     int32_t staged;              // 0: the lowest five output bits are row bits, lanes store their own rows
     int32_t frag_vec;            // bit 0 has stride 1 and every address is even: 16-byte stores
-    int32_t frag_sm[8], frag_row[8];   // place in the staged fragment, row within the 32
+    int32_t frag_sm[8], frag_row[8];   // place in the staged fragment (XOR of the words), row within the 32
+    int32_t row_sm[5], col_sm[3];      // places of a fragment's row and column bits
     int64_t frag_out[8];
     int64_t row_hi[2];           // output strides of rows 32 and 64 of a tile
     int32_t pair;                // CTA pairs: an M tile and its odd neighbour run together
@@ -1008,7 +1012,16 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
 // starts an item only after the epilogue has released that item's accumulator
 // set (acc_empty), and the epilogue starts after the item's last MMA
 // completes (acc_full).  Every wait is bounded.
-constexpr int kGemmThreads = 320;   // producer, MMA, 8 epilogue warps
+// A warpgroup with the producer and the MMA warp (the other two idle) and two of
+// epilogue warps.  At launch 12 warps have 168 registers a thread; the first
+// warpgroup keeps kRegsFew and each epilogue thread takes kRegsEpi.  With 168 for
+// all (10 warps) the epilogue spilled 28 to 240 bytes, and every step bound by its
+// output slowed with the spills, staged or not (16 terms by 2^17 outputs 1.06 ms
+// at 68 bytes, 1.15 at 240, 0.97 without); all GEMMs of the 10^6-shot job 113.4 ->
+// 110.1 ms together with the conflict-free fragments.
+constexpr int kGemmThreads = 384;
+constexpr int kRegsFew = 72, kRegsEpi = 208;
+static_assert(128 * kRegsFew + 256 * kRegsEpi <= kGemmThreads * 168, "registers of the launch");
 constexpr int kPairKb = 8;          // least k-blocks run by CTA pairs (2 segments of 4)
 constexpr int64_t kPairRows = 4;    // least M tiles per trajectory of a stacked GEMM run by CTA pairs
 struct TileInfo {              // (rows and instances are TMA coordinates: 32 bits)
@@ -1184,106 +1197,110 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
     const uint32_t tmem = *tslot;
     const int64_t n_tiles = g.n_tiles;
 
-    if (warp == 0) {
-        int64_t it = 0;
-        TileQueue tq;
-        TileInfo t;
-        while (!__shfl_sync(0xffffffffu, *abort, 0) && tq.next(g, lane, t)) {
-            if (lane == 0) {
-                for (int i = 0; i < g.nkb; i++, it++) {
-                    const int kb = split ? i % seg_kb * n_seg + i / seg_kb : i;
-                    const int s = (int)(it % NST);
-                    if (it >= NST && !mbar_wait(&empty[s], (uint32_t)((it / NST) - 1) & 1u, abort, g.wait_ns)) {
-                        atomicExch(g.err, 1);
-                        *abort = 1;
-                        break;
-                    }
-                    uint8_t* st = stage0 + s * kStageBytes;
-                    if constexpr (PAIR) {
-                        if (rank == 0) mbar_expect_tx(&full[s], (uint32_t)(2 * kStageBytes));   // both CTAs' copies
-                        const uint32_t bar = mbar_of(&full[s], 0);
-                        const int n0 = t.n0 + (int)rank * kBN;                                   // this CTA's half of B
-                        tma_load_3d_pair(st, &tmA, kb * kBK, t.m0, t.za, bar);
-                        tma_load_3d_pair(st + kTileA, &tmA, g.Kh + kb * kBK, t.m0, t.za, bar);
-                        tma_load_3d_pair(st + 2 * kTileA, &tmB, kb * kBK, n0, t.zb, bar);
-                        tma_load_3d_pair(st + 2 * kTileA + kTileB, &tmB, g.Kh + kb * kBK, n0, t.zb, bar);
-                    } else {
-                        mbar_expect_tx(&full[s], (uint32_t)kStageBytes);
-                        tma_load_3d(st, &tmA, kb * kBK, t.m0, t.za, &full[s]);                          // A hi
-                        tma_load_3d(st + kTileA, &tmA, g.Kh + kb * kBK, t.m0, t.za, &full[s]);          // A lo
-                        tma_load_3d(st + 2 * kTileA, &tmB, kb * kBK, t.n0, t.zb, &full[s]);             // B hi
-                        tma_load_3d(st + 2 * kTileA + kTileB, &tmB, g.Kh + kb * kBK, t.n0, t.zb, &full[s]);   // B lo
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsFew));
+        if (warp == 0) {
+            int64_t it = 0;
+            TileQueue tq;
+            TileInfo t;
+            while (!__shfl_sync(0xffffffffu, *abort, 0) && tq.next(g, lane, t)) {
+                if (lane == 0) {
+                    for (int i = 0; i < g.nkb; i++, it++) {
+                        const int kb = split ? i % seg_kb * n_seg + i / seg_kb : i;
+                        const int s = (int)(it % NST);
+                        if (it >= NST && !mbar_wait(&empty[s], (uint32_t)((it / NST) - 1) & 1u, abort, g.wait_ns)) {
+                            atomicExch(g.err, 1);
+                            *abort = 1;
+                            break;
+                        }
+                        uint8_t* st = stage0 + s * kStageBytes;
+                        if constexpr (PAIR) {
+                            if (rank == 0) mbar_expect_tx(&full[s], (uint32_t)(2 * kStageBytes));   // both CTAs' copies
+                            const uint32_t bar = mbar_of(&full[s], 0);
+                            const int n0 = t.n0 + (int)rank * kBN;                                   // this CTA's half of B
+                            tma_load_3d_pair(st, &tmA, kb * kBK, t.m0, t.za, bar);
+                            tma_load_3d_pair(st + kTileA, &tmA, g.Kh + kb * kBK, t.m0, t.za, bar);
+                            tma_load_3d_pair(st + 2 * kTileA, &tmB, kb * kBK, n0, t.zb, bar);
+                            tma_load_3d_pair(st + 2 * kTileA + kTileB, &tmB, g.Kh + kb * kBK, n0, t.zb, bar);
+                        } else {
+                            mbar_expect_tx(&full[s], (uint32_t)kStageBytes);
+                            tma_load_3d(st, &tmA, kb * kBK, t.m0, t.za, &full[s]);                          // A hi
+                            tma_load_3d(st + kTileA, &tmA, g.Kh + kb * kBK, t.m0, t.za, &full[s]);          // A lo
+                            tma_load_3d(st + 2 * kTileA, &tmB, kb * kBK, t.n0, t.zb, &full[s]);             // B hi
+                            tma_load_3d(st + 2 * kTileA + kTileB, &tmB, g.Kh + kb * kBK, t.n0, t.zb, &full[s]);   // B lo
+                        }
                     }
                 }
+                __syncwarp();
+            }
+            if (lane == 0) {
+                // let this CTA's own copies land before it exits (on every path: the
+                // MMA thread may have stopped early): the last load of every stage
+                // is that stage's newest phase
+                const int64_t first = it > NST ? it - NST : 0;
+                if (!PAIR)
+                    for (int64_t j = first; j < it; j++) mbar_wait_plain(&full[j % NST], (uint32_t)(j / NST) & 1u);
             }
             __syncwarp();
-        }
-        if (lane == 0) {
-            // let this CTA's own copies land before it exits (on every path: the
-            // MMA thread may have stopped early): the last load of every stage
-            // is that stage's newest phase
-            const int64_t first = it > NST ? it - NST : 0;
-            if (!PAIR)
-                for (int64_t j = first; j < it; j++) mbar_wait_plain(&full[j % NST], (uint32_t)(j / NST) & 1u);
-        }
-        __syncwarp();
-    } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
-            int64_t it = 0, lt = 0;
-            bool ok = true;
-            uint32_t used = 0, phase = 0, x = 1;   // a pair: regions used, their waits' parities, the tile's sum
-            for (int64_t tile = blockIdx.x; tile < n_tiles && !*abort && ok; tile += gridDim.x) {
-                x ^= 1;
-                for (int sg = 0; sg < n_seg && ok; sg++, lt++) {
-                    const int set = PAIR ? (int)(sg ? x ^ 1 : x) : (int)(lt % n_sets);
-                    const bool again = PAIR ? (used >> set) & 1 : lt >= n_sets;
-                    const uint32_t parity = PAIR ? (phase >> set) & 1 : (uint32_t)((lt / n_sets - 1) & 1);
-                    if (again) phase ^= 1u << set;
-                    used |= 1u << set;
-                    // this set's previous item has been drained by the epilogue
-                    if (again && !mbar_wait(&acc_empty[set], parity, abort, g.wait_ns)) {
-                        atomicExch(g.err, 4);
-                        *abort = 1;
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const int kb0 = sg * seg_kb, kb1 = kb0 + seg_kb < g.nkb ? kb0 + seg_kb : g.nkb;
-                    for (int kb = kb0; kb < kb1; kb++, it++) {
-                        const int s = (int)(it % NST);
-                        if (!mbar_wait(&full[s], (uint32_t)(it / NST) & 1u, abort, g.wait_ns)) {
-                            atomicExch(g.err, 2);
+        } else if (warp == 1) {
+            if (lane == 0 && rank == 0) {
+                int64_t it = 0, lt = 0;
+                bool ok = true;
+                uint32_t used = 0, phase = 0, x = 1;   // a pair: regions used, their waits' parities, the tile's sum
+                for (int64_t tile = blockIdx.x; tile < n_tiles && !*abort && ok; tile += gridDim.x) {
+                    x ^= 1;
+                    for (int sg = 0; sg < n_seg && ok; sg++, lt++) {
+                        const int set = PAIR ? (int)(sg ? x ^ 1 : x) : (int)(lt % n_sets);
+                        const bool again = PAIR ? (used >> set) & 1 : lt >= n_sets;
+                        const uint32_t parity = PAIR ? (phase >> set) & 1 : (uint32_t)((lt / n_sets - 1) & 1);
+                        if (again) phase ^= 1u << set;
+                        used |= 1u << set;
+                        // this set's previous item has been drained by the epilogue
+                        if (again && !mbar_wait(&acc_empty[set], parity, abort, g.wait_ns)) {
+                            atomicExch(g.err, 4);
                             *abort = 1;
                             ok = false;
                             break;
                         }
                         tc_fence_after();
-                        const uint32_t sa = smem_u32(stage0 + s * kStageBytes);
-                        const uint32_t sal = sa + kTileA, sb = sa + 2 * kTileA, sbl = sb + kTileB;
-                        const int j = kb - kb0;
-                        const uint32_t acc = tmem + (uint32_t)((set * acc_per + j % acc_per) * TN);
-                        const bool fresh = j < acc_per;
-#pragma unroll
-                        for (int kk = 0; kk < kRowBytes / 32; kk++) {   // 32 bytes of K per MMA
-                            const uint32_t o = kk * 32;
-                            umma<F, PAIR>(acc, sdesc_sw128(sa + o), sdesc_sw128(sb + o), (fresh && kk == 0) ? 0u : 1u);
-                            umma<F, PAIR>(acc, sdesc_sw128(sa + o), sdesc_sw128(sbl + o), 1u);
-                            umma<F, PAIR>(acc, sdesc_sw128(sal + o), sdesc_sw128(sb + o), 1u);
+                        const int kb0 = sg * seg_kb, kb1 = kb0 + seg_kb < g.nkb ? kb0 + seg_kb : g.nkb;
+                        for (int kb = kb0; kb < kb1; kb++, it++) {
+                            const int s = (int)(it % NST);
+                            if (!mbar_wait(&full[s], (uint32_t)(it / NST) & 1u, abort, g.wait_ns)) {
+                                atomicExch(g.err, 2);
+                                *abort = 1;
+                                ok = false;
+                                break;
+                            }
+                            tc_fence_after();
+                            const uint32_t sa = smem_u32(stage0 + s * kStageBytes);
+                            const uint32_t sal = sa + kTileA, sb = sa + 2 * kTileA, sbl = sb + kTileB;
+                            const int j = kb - kb0;
+                            const uint32_t acc = tmem + (uint32_t)((set * acc_per + j % acc_per) * TN);
+                            const bool fresh = j < acc_per;
+    #pragma unroll
+                            for (int kk = 0; kk < kRowBytes / 32; kk++) {   // 32 bytes of K per MMA
+                                const uint32_t o = kk * 32;
+                                umma<F, PAIR>(acc, sdesc_sw128(sa + o), sdesc_sw128(sb + o), (fresh && kk == 0) ? 0u : 1u);
+                                umma<F, PAIR>(acc, sdesc_sw128(sa + o), sdesc_sw128(sbl + o), 1u);
+                                umma<F, PAIR>(acc, sdesc_sw128(sal + o), sdesc_sw128(sb + o), 1u);
+                            }
+                            umma_commit<PAIR>(&empty[s]);   // stage free once these MMAs have read it
                         }
-                        umma_commit<PAIR>(&empty[s]);   // stage free once these MMAs have read it
+                        if (!ok) break;
+                        umma_commit<PAIR>(&acc_full[set]);  // accumulators complete for this item
                     }
-                    if (!ok) break;
-                    umma_commit<PAIR>(&acc_full[set]);  // accumulators complete for this item
                 }
+                // MMAs still in flight finish before TMEM is freed (on every path: the
+                // epilogue may have stopped early)
+                umma_commit<PAIR>(drain);
+                mbar_wait_plain(drain, 0u);
             }
-            // MMAs still in flight finish before TMEM is freed (on every path: the
-            // epilogue may have stopped early)
-            umma_commit<PAIR>(drain);
-            mbar_wait_plain(drain, 0u);
+            __syncwarp();
         }
-        __syncwarp();
     } else {
-        // epilogue warps 2..9: TMEM lane quadrant q = warp % 4 holds tile rows
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
+        // epilogue warps 4..11: TMEM lane quadrant q = warp % 4 holds tile rows
         // 32q..32q+31; two warps per quadrant drain half of the tile's columns
         // each (one warp per SM sub-partition leaves its load and store
         // latencies exposed).  Where the lowest five output bits are row bits a
@@ -1295,17 +1312,18 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
         // warps staging 16 columns.  4096 trajectories of the middle 30-qubit
         // block: that step 23.9 -> 16.1 ms, one with four hyper bits (55 GB)
         // 12.7 -> 9.1 ms (6.0 TB/s); all GEMMs of the 10^6-shot job 149 -> 132 ms.
-        const int ew = warp - 2, q = warp & 3;
+        const int ew = warp - 4, q = warp & 3;
         const int c_lo = (ew >> 2) * (TN / 2), c_hi = c_lo + TN / 2;
         // this warp's columns, from c_lo / 2 on (a single CTA's tables have room for all)
         int64_t* noff = noff_all + ew * (kBN / 2) - (PAIR ? c_lo / 2 : 0);
         float* ucol = ucol_all + ew * (kBN / 2) - (PAIR ? c_lo / 2 : 0);
-        float2* stg = stg_all + ew * 32 * kStgPitch;
-        int sm_l = 0, row_l = 0;
+        float2* stg = stg_all + ew * kStgElems;
+        int sm_l = 0, row_l = 0, st_l = 0;
         int64_t out_l = (q & 1 ? g.row_hi[0] : 0) + (q & 2 ? g.row_hi[1] : 0);
         for (int b = 0; b < 5; b++)
             if ((lane >> b) & 1) {
-                sm_l += g.frag_sm[b + 1];
+                sm_l ^= g.frag_sm[b + 1];
+                st_l ^= g.row_sm[b];
                 row_l += g.frag_row[b + 1];
                 out_l += g.frag_out[b + 1];
             }
@@ -1402,15 +1420,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                         for (int f = 0; f < 2; f++) {
 #pragma unroll
                             for (int j = 0; j < 8; j++)
-                                stg[lane * kStgPitch + j] = make_float2(v[16 * f + 2 * j], v[16 * f + 2 * j + 1]);
+                                stg[st_l ^ (j & 1 ? g.col_sm[0] : 0) ^ (j & 2 ? g.col_sm[1] : 0) ^ (j & 4 ? g.col_sm[2] : 0)] =
+                                    make_float2(v[16 * f + 2 * j], v[16 * f + 2 * j + 1]);
                             __syncwarp();
                             float2* o = out + noff[(c0 >> 1) + 8 * f];
 #pragma unroll
                             for (int i = 0; i < 4; i++) {
-                                const int sm = sm_l + (i & 1 ? g.frag_sm[6] : 0) + (i & 2 ? g.frag_sm[7] : 0);
+                                const int sm = sm_l ^ (i & 1 ? g.frag_sm[6] : 0) ^ (i & 2 ? g.frag_sm[7] : 0);
                                 const int rr = row_l + (i & 1 ? g.frag_row[6] : 0) + (i & 2 ? g.frag_row[7] : 0);
                                 float2* d = o + ((i & 1 ? g.frag_out[6] : 0) + (i & 2 ? g.frag_out[7] : 0));
-                                const float2 x = stg[sm], y = stg[sm + g.frag_sm[0]];
+                                const float2 x = stg[sm], y = stg[sm ^ g.frag_sm[0]];
                                 if (g.frag_vec && rr + g.frag_row[0] < row_lim) {
                                     *reinterpret_cast<float4*>(d) = make_float4(x.x, x.y, y.x, y.y);
                                 } else {
@@ -1870,16 +1889,35 @@ ptn_status run_gemm(const StepDesc& st, const ChunkCtx& ctx, int64_t n_inst, voi
         ga.staged = direct ? 0 : 1;
         struct Bit {
             int64_t out;
-            int32_t sm, row;
+            int32_t id;   // 0..4 row bits, 5..7 column bits
         } bit[8];
-        for (int i = 0; i < 5; i++) bit[i] = {row_stride(i), kStgPitch << i, 1 << i};
-        for (int i = 0; i < 3; i++) bit[5 + i] = {ga.n_stride[i], 1 << i, 0};
+        for (int i = 0; i < 8; i++) bit[i] = {i < 5 ? row_stride(i) : ga.n_stride[i - 5], i};
         std::sort(bit, bit + 8, [](const Bit& x, const Bit& y) { return x.out < y.out; });
+        // place of a fragment's element: the XOR of its bits' words.  The low four
+        // bits of a place choose the bank pair; row bits 0..3 (a half-warp's lanes
+        // when it writes) and the sorted bits 1..4 (when it reads) both span them:
+        // a sorted bit that is not among those row bits shares the bank bit of a row
+        // bit that is not among the sorted ones.
+        int32_t place[8];
+        for (int i = 0; i < 8; i++) place[i] = 1 << i;
+        int spare = 0;   // next row bit 0..3 that is not a sorted bit 1..4
+        for (int i = 1; i <= 4; i++) {
+            if (bit[i].id < 4) continue;
+            auto sorted = [&](int r) {
+                for (int k = 1; k <= 4; k++)
+                    if (bit[k].id == r) return true;
+                return false;
+            };
+            while (sorted(spare)) spare++;
+            place[bit[i].id] |= 1 << spare++;
+        }
         for (int i = 0; i < 8; i++) {
             ga.frag_out[i] = bit[i].out;
-            ga.frag_sm[i] = bit[i].sm;
-            ga.frag_row[i] = bit[i].row;
+            ga.frag_sm[i] = place[bit[i].id];
+            ga.frag_row[i] = bit[i].id < 5 ? 1 << bit[i].id : 0;
         }
+        for (int i = 0; i < 5; i++) ga.row_sm[i] = place[i];
+        for (int i = 0; i < 3; i++) ga.col_sm[i] = place[5 + i];
         ga.row_hi[0] = row_stride(5);
         ga.row_hi[1] = row_stride(6);
         // every bit above stride 1 is even; so must the instances' bases be
