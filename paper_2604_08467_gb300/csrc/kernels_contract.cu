@@ -1117,6 +1117,16 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const OperandDesc* __r
                 if ((it >> (k - 8)) & 1) x += 1 << f.x_bit[k];
             if (it < n_it) sm[x + (x >> 4)] = v[it];
         }
+        __syncthreads();
+        float* out = marg + net0 * nx + (tile << tb);
+#pragma unroll
+        for (int it = 0; it < NV; it++) {
+            const int x = it * kFinThreads + tid;
+            if (it < n_it) v[it] = sm[x + (x >> 4)];
+            if (it < n_it && x < valid) out[x] = v[it];
+        }
+        // the totals take the outcomes in their own order, whatever the order of the
+        // operands' memory: the same row gives the same total in every plan
         if constexpr (TB != 0) {
             constexpr int PER = 1 << (TB - 8), NETS = NV / PER;   // a thread's elements of a network
 #pragma unroll
@@ -1128,15 +1138,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const OperandDesc* __r
                     if (rowmax && m > 0.f && g < nets) atomicMax(&rowmax[net0 + g], __float_as_uint(m));
                 }
             }
-        }
-        __syncthreads();
-        float* out = marg + net0 * nx + (tile << tb);
-#pragma unroll
-        for (int it = 0; it < NV; it++) {
-            const int x = it * kFinThreads + tid;
-            if (it < n_it && x < valid) out[x] = sm[x + (x >> 4)];
-        }
-        if constexpr (TB != 0) {
+            __syncthreads();
             if (tid < nets) {
                 double t = 0.0;
                 for (int w = 0; w < 8; w++) t += red[tid * 8 + w];
