@@ -186,6 +186,11 @@ struct GroupTable {
 ptn_status launch_gemm_step(const StepDesc& st, const ChunkCtx& ctx, int64_t n_inst, void* pack_a, void* pack_b,
                             int* err, const GroupTable& grp, int precision, cudaStream_t s,
                             const StepDesc* prod_src = nullptr);
+// Hash of the forms (pairs of CTAs or single ones) of the calling thread's GEMM
+// launches since the last reset: a recorded graph whose forms differ has nodes of
+// other cluster sizes, which are not exchanged in an executable graph.
+void gemm_forms_reset();
+uint64_t gemm_forms();
 
 // ---- expectation values and gradients (kernels_expval.cu)
 struct ObsTerm {

@@ -1614,6 +1614,7 @@ __global__ void k_group_tiles(const int32_t* __restrict__ net0, int64_t n_groups
 
 // ---------------------------------------------------------- host helpers --
 std::atomic<uint64_t> g_wait_ns{2000000000ull};   // limit of the GEMM's pipeline waits
+thread_local uint64_t t_gemm_forms = 0;   // this thread's launches since gemm_forms_reset: pairs or single CTAs
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -1998,6 +1999,7 @@ ptn_status run_gemm(const StepDesc& st, const ChunkCtx& ctx, int64_t n_inst, voi
                          (double)kEB * 2 * Kh * ((double)pa.n_pinst * M + (double)pb.n_pinst * 2 * N) * (1ll << nh);
     StatScope sc(K_CONTRACT_GEMM, s, bytes, flops);
     ga.n_tiles = blocks;
+    t_gemm_forms = (t_gemm_forms ^ (uint64_t)(1 + ga.pair)) * 1099511628211ull;
     const int64_t grid = blocks < n_sm ? blocks : n_sm;
     if (ga.pair) {
         cudaLaunchConfig_t lc{};
@@ -2022,6 +2024,9 @@ ptn_status run_gemm(const StepDesc& st, const ChunkCtx& ctx, int64_t n_inst, voi
 }
 
 }  // namespace
+
+void gemm_forms_reset() { t_gemm_forms = 14695981039346656037ull; }
+uint64_t gemm_forms() { return t_gemm_forms; }
 
 ptn_status launch_gemm_step(const StepDesc& st, const ChunkCtx& ctx, int64_t n_inst, void* pack_a, void* pack_b,
                             int* err, const GroupTable& grp, int precision,

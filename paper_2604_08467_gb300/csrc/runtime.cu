@@ -142,10 +142,12 @@ struct PlanWorkspace {
     // capture stream and one executable graph per block, updated in place
     cudaStream_t cap_stream = nullptr;
     std::vector<cudaGraphExec_t> gexec;
+    std::vector<uint64_t> gforms;   // gemm_forms of each
     void release_graphs() {
         for (auto& x : gexec)
             if (x) cudaGraphExecDestroy(x);
         gexec.clear();
+        gforms.clear();
         if (cap_stream) cudaStreamDestroy(cap_stream);
         cap_stream = nullptr;
     }
@@ -486,6 +488,7 @@ ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const
     if (graphs) {
         if (!ws->cap_stream) PTN_CUDA(cudaStreamCreateWithFlags(&ws->cap_stream, cudaStreamNonBlocking));
         if (ws->gexec.size() < plan->blocks.size()) ws->gexec.resize(plan->blocks.size(), nullptr);
+        ws->gforms.resize(ws->gexec.size(), 0);
     }
     for (size_t ci = 0; ci < chunks.size(); ci++) {
         const Chunk& c = chunks[ci];
@@ -522,6 +525,7 @@ ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const
         if (graphs) {
             PTN_CUDA(cudaStreamBeginCapture(ws->cap_stream, cudaStreamCaptureModeRelaxed));
             ls = ws->cap_stream;
+            gemm_forms_reset();
         }
         auto end_capture = [&]() {
             if (!graphs) return;
@@ -587,13 +591,15 @@ ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const
         if (graphs) {
             // the block's executable graph takes the new chunk's parameters in
             // place; a chunk whose launch sequence differs in shape (other
-            // launch counts) gets a fresh executable
+            // launch counts, other GEMMs on CTA pairs) gets a fresh executable
             cudaGraph_t g = nullptr;
             PTN_CUDA(cudaStreamEndCapture(ws->cap_stream, &g));
             cudaGraphExec_t& x = ws->gexec[j];
+            const bool forms = ws->gforms[j] == gemm_forms();
+            ws->gforms[j] = gemm_forms();
             if (x) {
                 cudaGraphExecUpdateResultInfo info;
-                if (cudaGraphExecUpdate(x, g, &info) != cudaSuccess) {
+                if (!forms || cudaGraphExecUpdate(x, g, &info) != cudaSuccess) {
                     cudaGetLastError();
                     cudaGraphExecDestroy(x);
                     x = nullptr;
