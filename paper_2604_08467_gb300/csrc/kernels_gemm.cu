@@ -55,8 +55,9 @@ constexpr int kPairN = 2 * kBN;   // columns of a CTA pair's tile (k_gemm<F, tru
 // Its elements are placed so that a half-warp's 8-byte accesses hit 16 different
 // bank pairs both when written by row and when read in the order of the output
 // (run_gemm): a 128 x 128 tile's operands already take 1280 clocks of shared memory
-// per k-block, and with rows padded to 9 slots 9.1 of 16.5 million wavefronts of
-// the 2^20 outputs by 128 terms were conflicts (14.2 -> 13.4 ms).
+// per k-block.  Against rows padded to 9 slots, 2^20 outputs by 128 terms, 40
+// trajectories: 16.5 -> 13.9 million wavefronts, 9.8 -> 7.0 million of them counted
+// as conflicts; 4096 trajectories 14.2 -> 13.4 ms.
 constexpr int kStgElems = 32 * 8;
 constexpr int kStgBytes = 8 * kStgElems * 8;
 constexpr int kTabBytes = 8192;   // barriers, TMEM slot, per-warp column offsets and FP16 column scales
@@ -1018,7 +1019,7 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
 // all (10 warps) the epilogue spilled 28 to 240 bytes, and every step bound by its
 // output slowed with the spills, staged or not (16 terms by 2^17 outputs 1.06 ms
 // at 68 bytes, 1.15 at 240, 0.97 without); all GEMMs of the 10^6-shot job 113.4 ->
-// 110.1 ms together with the conflict-free fragments.
+// 110.1 ms together with the placed fragments.
 constexpr int kGemmThreads = 384;
 constexpr int kRegsFew = 72, kRegsEpi = 208;
 static_assert(128 * kRegsFew + 256 * kRegsEpi <= kGemmThreads * 168, "registers of the launch");
