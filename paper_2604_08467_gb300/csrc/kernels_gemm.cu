@@ -1007,7 +1007,7 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
 // Persistent warp-specialised GEMM: each CTA (one per SM) walks the tiles
 // blockIdx.x, blockIdx.x + gridDim.x, ...  Warp 0 lane 0 streams the K-blocks
 // of all its tiles through the kStages shared-memory ring by TMA; warp 1
-// lane 0 issues tcgen05.mma into the TMEM accumulators; warps 2-5 (one per
+// lane 0 issues tcgen05.mma into the TMEM accumulators; warps 4-11 (two per
 // TMEM lane quadrant) drain a finished item (a tile, or one K segment of a
 // long tile) while the producer already loads the next one.  The MMA warp
 // starts an item only after the epilogue has released that item's accumulator
