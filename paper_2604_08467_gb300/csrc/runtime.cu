@@ -547,7 +547,7 @@ ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const
         ctx.n_words = (plan->n_qubits + 63) / 64;
         ctx.chunk_traj = ws->chunk_traj.as<int32_t>() + c.traj0;
         ctx.net_tl = ws->net_tl.as<int32_t>() + c.net0;
-        ctx.net_prefix = d_net_prefix + c.net0;
+        ctx.net_prefix = d_net_prefix + c.net0 * ctx.n_words;
         for (int a = 0; a < 3; a++) ctx.arena[a] = ws->arena[a].as<float2>();
         ctx.arena[ARENA_ADJ] = ctx.arena[ARENA_LGRAD] = nullptr;
         ctx.arena_inst[ARENA_ADJ] = ctx.arena_inst[ARENA_LGRAD] = 0;
