@@ -830,6 +830,10 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
+// takes `bytes` that no copy will bring off the current phase of this CTA's barrier
+__device__ __forceinline__ void mbar_complete_tx(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -849,6 +853,14 @@ __device__ __forceinline__ uint32_t mbar_of(uint64_t* bar, uint32_t rank) {
     uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(bar)), "r"(rank));
     return r;
+}
+// a 64-bit word of CTA `rank`'s shared memory
+__device__ __forceinline__ int64_t load_of(const int64_t* p, uint32_t rank) {
+    uint32_t a;
+    int64_t v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+    return v;
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
@@ -1130,6 +1142,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
     uint64_t* drain = acc_empty + 2;
     uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* abort = reinterpret_cast<volatile int*>(tslot + 1);
+    int64_t* issued = reinterpret_cast<int64_t*>(tslot + 2);   // a pair: stages this CTA's producer loaded
     // tables of the 8 epilogue warps, 16-byte aligned (the scales are read four at
     // a time; the barriers before them end 8 bytes past a boundary)
     constexpr int kTabOff = (int)(((2 * NST + 5) * 8 + 16 + 15) & ~15);
@@ -1238,8 +1251,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
                 // let this CTA's own copies land before it exits (on every path: the
                 // MMA thread may have stopped early): the last load of every stage
                 // is that stage's newest phase
+                // (a pair's are counted by the leader: below, when both producers have stopped)
                 const int64_t first = it > NST ? it - NST : 0;
-                if (!PAIR)
+                if (PAIR) *issued = it;
+                else
                     for (int64_t j = first; j < it; j++) mbar_wait_plain(&full[j % NST], (uint32_t)(j / NST) & 1u);
             }
             __syncwarp();
@@ -1576,15 +1591,29 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm(const __grid_constant_
     tc_fence_before();
     __syncthreads();
     if constexpr (PAIR) {
-        // The peer's MMAs read this CTA's shared memory and write its TMEM, and its
-        // barriers are signalled from here: both CTAs are done before either
-        // frees or leaves.  After a wait that ran out, copies may be in flight
-        // that no barrier of this CTA counts; a millisecond lets them land.
-        if (threadIdx.x == 0 && *abort)
-            for (const uint64_t t0 = global_ns(); global_ns() - t0 < 1000000ull;) {
+        // The peer's MMAs read this CTA's shared memory and write its TMEM, its
+        // barriers are signalled from here, and the leader's count the copies of
+        // both: neither frees or leaves before all of that has ended.
+        cluster_sync();              // no wait, load or MMA is started by either from here on
+        if (threadIdx.x == 0) {
+            if (rank == 0) {
+                // After a wait that ran out the producers may have stopped at different
+                // stages.  A stage that one of them alone loaded (at most NST: both wait
+                // for the same MMAs) is settled for the half that is missing; then the
+                // newest phase of every stage ends with the last copy in flight.
+                const int64_t mine = *issued, peer = load_of(issued, 1);
+                const int64_t lo = mine < peer ? mine : peer, hi = mine < peer ? peer : mine;
+                for (int64_t j = lo; j < hi; j++) {
+                    if (mine > peer) mbar_complete_tx(&full[j % NST], (uint32_t)kStageBytes);
+                    else mbar_expect_tx(&full[j % NST], (uint32_t)kStageBytes);
+                }
+                for (int64_t j = hi > NST ? hi - NST : 0; j < hi; j++)
+                    mbar_wait_plain(&full[j % NST], (uint32_t)(j / NST) & 1u);
+            } else {
+                mbar_wait_plain(drain, 0u);   // the leader's last commit, signalled to both
             }
-        __syncthreads();
-        cluster_sync();
+        }
+        __syncwarp();
     }
     if (warp == 0) {
         tc_fence_after();
