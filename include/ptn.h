@@ -562,11 +562,13 @@ ptn_status ptn_tune_block_sizes(const ptn_circuit* circuit, const ptn_noise* noi
  * the plain direct kernel).  Every block is contracted once on a probe of
  * min(n_probe, unique trajectories, what one chunk holds) networks (one per
  * trajectory, prefix 0) to fill its intermediates; then each step is launched
- * under every feasible (ra, rb), timed over `reps` launches with CUDA events
- * on the stream after one warm-up, and the fastest shape is stored in the
- * plan for later calls if it beats the default shape (the most tile bits) by
- * more than 5%.  The probe should be as large as the chunks of the intended
- * runs: a shape that wins on few instances can lose on many.
+ * as it runs by default (staged through shared memory where that applies, else
+ * the most tile bits) and under every feasible (ra, rb), timed over `reps`
+ * launches with CUDA events on the stream after one warm-up, and the fastest
+ * shape is stored in the plan for later calls if it beats the default by more
+ * than 5%.  Steps that run fused with others or in the finalisation are left
+ * out.  The probe should be as large as the chunks of the intended runs: a
+ * shape that wins on few instances can lose on many.
  * Timing does not depend on the data, and a step's output never aliases its
  * operands, so the repeated launches leave the intermediates intact.  The
  * arithmetic of each output (its multiply-add chain over the summed bits) is

@@ -156,6 +156,8 @@ void launch_small_steps(const SmallRuns& sr, std::pair<int32_t, int32_t> parts, 
                         const ChunkCtx& ctx, int64_t n_inst, cudaStream_t s);
 void launch_contract_step(const StepDesc* d_step, const StepDesc& h_step, const ChunkCtx& ctx,
                           int64_t n_inst, cudaStream_t s);
+// whether a step without a tuned tile is staged through shared memory (no micro-tile)
+bool staged_step(const StepDesc& h, const ChunkCtx& ctx, int64_t n_inst);
 // marginal rows (real diagonal of the root) and their FP64 totals; part holds
 // n_net * finalize_tiles(b) doubles when finalize_tiles(b) > 1 (else unused);
 // rowmax (or null): zeroed, per row the bits of its largest entry

@@ -901,15 +901,13 @@ void launch_rows_t(const StepDesc* d_step, const ChunkCtx& ctx, int64_t n_inst, 
     }
 }
 
-// Runs a step by k_contract_group or k_contract_rows where one of them applies.
-bool launch_rows(const StepDesc* d_step, const StepDesc& h, const ChunkCtx& ctx, int64_t n_inst, cudaStream_t s) {
-    GroupArgs g;
+// Arguments of k_contract_group (n_groups set) or k_contract_rows for a step;
+// false where neither applies.
+bool choose_rows(const StepDesc& h, const ChunkCtx& ctx, int64_t n_inst, GroupArgs& g, int& ra, int& rb, int& smem) {
     memset(&g, 0, sizeof g);
-    int ra, rb, smem;
     // shared operand: a trajectory- or circuit-level buffer, the one with more
     // elements per network; grouped where a unit finds at least kGroupMin
     // networks on average
-    bool ok = false;
     if (h.out_cls == CLS_NET && ctx.grp_net0 && h.n_sum <= 8) {
         int p = -1;
         int64_t best = 0;
@@ -933,10 +931,15 @@ bool launch_rows(const StepDesc* d_step, const StepDesc& h, const ChunkCtx& ctx,
             while ((groups << (g.r.n_sub + g.ns + g.seg_log)) < 152 * 6 &&
                    n_inst >= 2 * kGroupMin * (groups << (g.ns + g.seg_log)))
                 g.seg_log++;
-            ok = true;
+            return true;
         }
     }
-    if (!ok && !rows_split(h, ctx, -1, 0, g.r, ra, rb, smem)) return false;
+    return rows_split(h, ctx, -1, 0, g.r, ra, rb, smem);
+}
+bool launch_rows(const StepDesc* d_step, const StepDesc& h, const ChunkCtx& ctx, int64_t n_inst, cudaStream_t s) {
+    GroupArgs g;
+    int ra, rb, smem;
+    if (!choose_rows(h, ctx, n_inst, g, ra, rb, smem)) return false;
     switch (ra * 3 + rb) {
         case 0: launch_rows_t<0, 0>(d_step, ctx, n_inst, g, smem, s); break;
         case 1: launch_rows_t<0, 1>(d_step, ctx, n_inst, g, smem, s); break;
@@ -1347,6 +1350,12 @@ void launch_small_steps(const SmallRuns& sr, std::pair<int32_t, int32_t> parts, 
         if (p > parts.first) count_launches(K_CONTRACT_SMALL);
         k_small_steps<<<(unsigned)n_inst, threads, sizeof(SmallRes) * pt.n_steps, s>>>(a, ctx);
     }
+}
+
+bool staged_step(const StepDesc& h, const ChunkCtx& ctx, int64_t n_inst) {
+    GroupArgs g;
+    int ra, rb, smem;
+    return choose_rows(h, ctx, n_inst, g, ra, rb, smem);
 }
 
 void launch_contract_step(const StepDesc* d_step, const StepDesc& h, const ChunkCtx& ctx, int64_t n_inst,

@@ -1936,10 +1936,10 @@ static void json_steps(std::string& s, const std::vector<StepDesc>& steps) {
         const StepDesc& st = steps[i];
         snprintf(buf, sizeof buf,
                  "%s{\"out_cls\":%d,\"n_out\":%d,\"n_sum\":%d,\"kind\":%d,\"gemm_a\":%d,\"out_arena\":%d,"
-                 "\"out_off\":%lld,\"fuse_prev\":%d,\"cache\":%d,\"virt\":%d,\"prod\":%d,\"prod_src\":%d,"
+                 "\"out_off\":%lld,\"fuse_prev\":%d,\"cache\":%d,\"virt\":%d,\"prod\":%d,\"prod_src\":%d,\"tile\":%d,"
                  "\"ops\":[",
                  i ? "," : "", st.out_cls, st.n_out, st.n_sum, st.kind, st.gemm_a, st.out_arena, (long long)st.out_off,
-                 st.fuse_prev, st.cache, st.virt, st.prod, st.prod_src);
+                 st.fuse_prev, st.cache, st.virt, st.prod, st.prod_src, st.tile);
         s += buf;
         json_op(s, st.op[0]);
         s += ",";

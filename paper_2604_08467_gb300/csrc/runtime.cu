@@ -975,17 +975,15 @@ ptn_status ptn_tune_tiles(ptn_plan* plan, const ptn_traj* traj, int64_t n_probe,
         ctx.arena_inst[CLS_CONST] = 1;
         ctx.arena_inst[CLS_TRAJ] = nt;
         ctx.arena_inst[CLS_NET] = nn;
+        ctx.grp_net0 = ws->grp.as<int32_t>();   // (the probe is one chunk: its trajectories' first networks)
+        const StepDesc* closing = closing_product(bp);
         for (size_t st = 0; st < bp.steps.size(); st++) {
             StepDesc& h = bp.steps[st];
-            if (small_step(h)) {   // fused runs are not tuned (one launch walks the whole run)
-                size_t en = st + 1;
-                while (en < bp.steps.size() && en - st < (size_t)plan->opts.fuse_max && bp.steps[en].fuse_prev) en++;
-                if (en - st >= 2) {
-                    st = en - 1;
-                    continue;
-                }
+            if (bp.small.run_at.count((int32_t)st)) {   // fused runs are not tuned (one launch walks the whole run)
+                st += small_run_len(bp.steps, st, plan->opts.fuse_max) - 1;
+                continue;
             }
-            if (h.kind != STEP_DIRECT || h.virt) continue;
+            if (h.kind != STEP_DIRECT || h.virt || &h == closing) continue;   // not launched on their own
             int ra_av = 0, rb_av = 0;
             for (int q = 0; q < h.n_out; q++) {
                 const bool va = h.out_stride[0][q] != 0, vb = h.out_stride[1][q] != 0;
@@ -995,16 +993,18 @@ ptn_status ptn_tune_tiles(ptn_plan* plan, const ptn_traj* traj, int64_t n_probe,
             ra_av = std::min(ra_av, 2);
             rb_av = std::min(rb_av, 2);
             const int64_t ni = h.out_cls == CLS_CONST ? 1 : (h.out_cls == CLS_TRAJ ? nt : nn);
-            // the default shape first; another shape replaces it only if it is
-            // more than 5% faster (timing noise does not move the choice)
-            const int def = 1 + 3 * ra_av + rb_av;
-            int best = def;
+            // the default first, as calls run it (a micro-tile of the most bits, unless
+            // the step is staged); another shape replaces it only if it is more than
+            // 5% faster (timing noise does not move the choice)
+            StepDesc h2 = h;
+            h2.tile = 0;
+            const bool staged = staged_step(h2, ctx, ni);
+            int best = 0;
             float best_ms = INFINITY, def_ms = INFINITY;
             for (int cand = -1; cand < (ra_av + 1) * (rb_av + 1); cand++) {
                 const int ra = cand < 0 ? ra_av : cand / (rb_av + 1), rb = cand < 0 ? rb_av : cand % (rb_av + 1);
-                if (cand >= 0 && ra == ra_av && rb == rb_av) continue;
-                StepDesc h2 = h;
-                h2.tile = 1 + 3 * ra + rb;
+                if (cand >= 0 && ra == ra_av && rb == rb_av && !staged) continue;
+                h2.tile = cand < 0 ? 0 : 1 + 3 * ra + rb;
                 launch_contract_step(bp.d_steps + st, h2, ctx, ni, s);   // warm-up
                 cudaEventRecord(e0, s);
                 for (int r = 0; r < reps; r++) launch_contract_step(bp.d_steps + st, h2, ctx, ni, s);
@@ -1019,9 +1019,9 @@ ptn_status ptn_tune_tiles(ptn_plan* plan, const ptn_traj* traj, int64_t n_probe,
                     best = h2.tile;
                 }
             }
-            if (best_ms > 0.95f * def_ms) best = def;
+            if (best_ms > 0.95f * def_ms) best = 0;
             tuned++;
-            if (best != def) changed++;
+            if (best) changed++;
             h.tile = best;
         }
         release_probe();
