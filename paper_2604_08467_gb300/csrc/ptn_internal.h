@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <map>
+#include <memory>
 #include <string>
 #include <utility>
 #include <vector>
@@ -209,6 +210,7 @@ struct BlockPlan {
     int32_t start = 0, b = 0;
     int32_t ket_only = 0;                // sampling block lowered in the ket-only network form
     int32_t by_class = 0;                // steps listed class by class: constant, trajectory, network level
+    std::shared_ptr<BlockPlan> path_order;   // (by_class) the same steps in the path's order: smaller buffers
     std::vector<StepDesc> steps;
     RootRef root;
     int64_t arena_peak[N_ARENAS] = {0, 0, 0, 0, 0};   // elements per instance, per arena
@@ -226,8 +228,9 @@ struct BlockPlan {
     std::vector<uint32_t> cache_bits;
     uint32_t* d_cache_bits = nullptr;
     SmallRuns small, small_bwd;          // fused runs of `steps` and (gradient plans) of `bwd`
-    // device copy
+    // device copies
     StepDesc* d_steps = nullptr;
+    RootRef* d_root = nullptr;
     // expectation/gradient plans only: the reversed path and its targets
     std::vector<StepDesc> bwd;
     int64_t root_adj_off = 0;            // ADJ arena offset of the root adjoint
@@ -267,7 +270,6 @@ struct ptn_plan {
     int32_t* d_leaf_site_ptr = nullptr;
     int32_t* d_leaf_site_idx = nullptr;
     int32_t* d_leaf_site_mul = nullptr;
-    ptn::RootRef* d_roots = nullptr;     // root descriptor of every block
     double mem_cap = 0;
 };
 
