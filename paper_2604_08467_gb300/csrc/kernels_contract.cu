@@ -580,7 +580,9 @@ __global__ void __launch_bounds__(256) k_contract_rows(const StepDesc* __restric
 // Batches of 8 have to be mostly full: with 5 networks per unit 0.053 ms by
 // k_contract_rows became 0.130, with 6.6 it went from 0.115 to 0.053.
 constexpr int kGroupWin = 512;         // networks scanned at a time
-constexpr int kGroupSmem = 72 * 1024;  // stages of one CTA (three per SM)
+// stages of one CTA: three per SM, but for 4 x 4 micro-tiles (wide steps), whose 194
+// registers leave room for two CTAs of 128 threads or one of 256
+constexpr int kGroupSmem = 72 * 1024;
 struct GroupArgs {
     RowsArgs r;                        // thread, micro-tile and sub-tile bits; the private operand's row
                                        // index has the network's place in the batch above its own rows
@@ -970,7 +972,11 @@ bool launch_rows(const StepDesc* d_step, const StepDesc& h, const ChunkCtx& ctx,
 // integers scaled by its largest entry (53 bits for it, the accuracy of adding
 // FP64 roundings), because this chip adds two FP64 numbers per clock and SM;
 // warps and tiles follow in order in FP64.  The others add 16 consecutive
-// outcomes per thread the same way and use a shuffle tree.
+// outcomes per thread the same way and use a shuffle tree; their form takes 107 to
+// 128 registers where the two take 64.  The two run through it would take, per
+// entry of 16,384 rows, at 2^10 outcomes 5.8 ps for the root (4.6 here), 6.0 for
+// |a|^2 (6.2), 8.5 for an outer product (5.4), at 2^12 5.3 (3.0), 5.4 (4.7) and 8.5
+// (4.3); 512 rows of 2^20 as an outer product 5.42 ms (2.21).
 // Measured: 1.9 M rows of 2^10 outcomes 15.6 -> 8.4 ms with the closing |a|^2
 // (6.3 ms, 24.6 GB) gone; 24 rows of 2^28 outcomes, an outer product, 46.1 ms
 // and 13.2 ms for the product -> 18.9 ms.

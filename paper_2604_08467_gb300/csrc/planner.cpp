@@ -1418,11 +1418,12 @@ static ptn_status search_and_lower(ptn_plan* plan, BlockNet& net, int j, int sta
     // and forth between trajectory and network level cuts the fused runs (44
     // runs and 159 single network steps for a 100-qubit block of the paper's
     // family).  Listed class by class its small steps form one run per class.
-    // Buffers then live longer (up to twice the bytes per trajectory), so this is
-    // done only while a trajectory's take at most kByClassBytes, a network's grow
-    // by no more than a sixteenth of that, and a memory cap the caller set still
-    // holds one network.  The path's order is kept beside it for calls that the
-    // larger buffers would split into too many chunks (contract_level).
+    // Buffers then live longer (2.4 times the bytes per trajectory in a block of
+    // that circuit, mostly 1.1 to 1.7 times), so this is done only while a
+    // trajectory's take at most kByClassBytes, a network's grow by no more than a
+    // sixteenth of that, and a memory cap the caller set still holds one network.
+    // The path's order is kept beside it for calls that the larger buffers would
+    // split into too many chunks (contract_level).
     if (!expval && plan->opts.fuse_max > 1) {
         auto bytes = [](const BlockPlan& p, int k) {
             return 8.0 * (double)p.arena_peak[k] + 4.0 * (double)(p.pack_peak[0][k] + p.pack_peak[1][k]);

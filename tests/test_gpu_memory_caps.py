@@ -1,8 +1,8 @@
-"""Memory caps on blocks listed class by class, whose buffers are up to twice those
-of the path's own order (the order of plans with fuse_max = 1): a cap that holds
-a network in the path's order is accepted, a call is not split into chunks that
-cost more launches than the path's order takes, and every result has the bits of
-the uncapped call."""
+"""Memory caps on blocks listed class by class, whose buffers are larger than those
+of the path's own order (the order of plans with fuse_max = 1): a cap that holds a
+network in the path's order is accepted, a call is not split into chunks that cost
+more launches than the path's order takes, and every result has the bits of the
+uncapped call."""
 import numpy as np
 import pytest
 
