@@ -211,6 +211,7 @@ struct BlockPlan {
     int32_t ket_only = 0;                // sampling block lowered in the ket-only network form
     int32_t by_class = 0;                // steps listed class by class: constant, trajectory, network level
     std::shared_ptr<BlockPlan> path_order;   // (by_class) the same steps in the path's order: smaller buffers
+    int32_t n_launch = 0;                // launches of a chunk, counted when first asked for
     std::vector<StepDesc> steps;
     RootRef root;
     int64_t arena_peak[N_ARENAS] = {0, 0, 0, 0, 0};   // elements per instance, per arena

@@ -258,10 +258,23 @@ void free_block(BlockPlan& bp) {
     free_small_runs(bp.small);
     if (bp.path_order) free_block(*bp.path_order);
 }
+// Workspace bytes of a block: constant, per trajectory and per network of a chunk.
+struct ChunkBytes {
+    double C, T, N;
+    explicit ChunkBytes(const BlockPlan& p) {
+        auto of = [&](int c) {
+            return 8.0 * (double)p.arena_peak[c] + 4.0 * (double)(p.pack_peak[0][c] + p.pack_peak[1][c]);
+        };
+        C = of(CLS_CONST);
+        T = of(CLS_TRAJ);
+        N = of(CLS_NET) + 4.0 + 8.0;
+    }
+};
 // Launches of one chunk of a block (about: a tensor-core step packs twice, and a
-// stacked one lays out its tiles by three more).
-int64_t chunk_launches(const BlockPlan& bp, int fuse_max) {
-    int64_t n = 1;
+// stacked one lays out its tiles by three more); counted once per plan.
+int32_t chunk_launches(BlockPlan& bp, int fuse_max) {
+    if (bp.n_launch) return bp.n_launch;
+    int32_t n = 1;
     const StepDesc* closing = closing_product(bp);
     for (size_t k = 0; k < bp.steps.size(); k++) {
         const StepDesc& h = bp.steps[k];
@@ -274,7 +287,7 @@ int64_t chunk_launches(const BlockPlan& bp, int fuse_max) {
             n += h.kind == STEP_DIRECT ? 1 : (h.kind == STEP_GEMM_STACKED ? 6 : 3);
         }
     }
-    return n;
+    return bp.n_launch = n;
 }
 
 ptn_status ensure_device(const ptn_plan* cplan) {
@@ -405,29 +418,51 @@ ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const
     PTN_CUDA(cudaMemcpyAsync(ws->h_traj.p, d_net_traj, sizeof(int32_t) * n_net, cudaMemcpyDeviceToHost, s));
     PTN_CUDA(cudaStreamSynchronize(s));
     const int32_t* ht = ws->h_traj.as<int32_t>();
+    int64_t n_traj = 1;
     for (int64_t i = 0; i < n_net; i++) {
         if (ht[i] < 0 || ht[i] >= tr->n_unique)
             return set_error(PTN_ERR_INVALID_ARG, "net_traj[%lld] = %d out of range", (long long)i, ht[i]);
         if (i && ht[i] < ht[i - 1]) return set_error(PTN_ERR_INVALID_ARG, "net_traj must be non-decreasing");
+        n_traj += i && ht[i] != ht[i - 1];
     }
+    const double cap = plan->mem_cap;
+    // chunks of a listing that are as full as the cap allows (infinity: it holds no network)
+    auto chunks_of = [&](const BlockPlan& p) {
+        const ChunkBytes by(p);
+        if (by.C + by.T + by.N > cap) return INFINITY;
+        double c = std::ceil((by.T * (double)n_traj + by.N * (double)n_net) / (cap - by.C));
+        if (max_traj_chunk > 0) c = std::max(c, std::ceil((double)n_traj / max_traj_chunk));
+        return (float)std::max(c, 1.0);
+    };
+    BlockPlan* use = const_cast<BlockPlan*>(&plan->blocks[j]);
+    if (BlockPlan* path = use->path_order.get()) {
+        // Where one chunk does not hold the call class by class, the path's order takes
+        // over if it makes fewer launches of the whole call (its chunks hold more
+        // networks), or if it alone holds a network.  Measured: 256 trajectories of a
+        // 40-qubit brickwork's block in 29 chunks 5.4 ms, by class in 43 chunks 7.2;
+        // 2000 of a 60-qubit one's in 42 chunks 8.1 ms, by class in 52 chunks 6.2 (half
+        // the launches per chunk).  Counted from the bytes: a pass over 30,000
+        // trajectories to fill chunks of both listings took 0.28 ms.
+        const float n_cls = chunks_of(*use);
+        if (n_cls > 1.f && chunks_of(*path) * (float)chunk_launches(*path, plan->opts.fuse_max) <
+                               n_cls * (float)chunk_launches(*use, plan->opts.fuse_max)) {
+            use = path;
+            if ((e = upload_block(*use))) return e;
+        }
+    }
+    const BlockPlan& bp = *use;
     if ((e = ws->h_chunk_traj.grow(sizeof(int32_t) * n_net))) return e;
     if ((e = ws->h_net_tl.grow(sizeof(int32_t) * n_net))) return e;
     int32_t* hct = ws->h_chunk_traj.as<int32_t>();
     int32_t* htl = ws->h_net_tl.as<int32_t>();
+    // chunking against the memory cap (arenas + GEMM operand packing, per instance)
+    const ChunkBytes by(bp);
+    if (by.C + by.T + by.N > cap)
+        return set_error(PTN_ERR_TOO_LARGE, "block %d needs %.3g bytes for one network (cap %.3g)", j,
+                         by.C + by.T + by.N, cap);
+    std::vector<Chunk> chunks;
     int64_t n_ct = 0;
-    // chunking against the memory cap (arenas + GEMM operand packing, per instance);
-    // write: the chunks' trajectories and networks too
-    auto split = [&](const BlockPlan& p, std::vector<Chunk>& chunks, bool write) -> ptn_status {
-        auto pk = [&](int c) { return 4.0 * (double)(p.pack_peak[0][c] + p.pack_peak[1][c]); };
-        const double bT = 8.0 * (double)p.arena_peak[CLS_TRAJ] + pk(CLS_TRAJ);
-        const double bN = 8.0 * (double)p.arena_peak[CLS_NET] + 4.0 + 8.0 + pk(CLS_NET);
-        const double bC = 8.0 * (double)p.arena_peak[CLS_CONST] + pk(CLS_CONST);
-        const double cap = plan->mem_cap;
-        if (bC + bT + bN > cap)
-            return set_error(PTN_ERR_TOO_LARGE, "block %d needs %.3g bytes for one network (cap %.3g)", j, bC + bT + bN,
-                             cap);
-        chunks.clear();
-        n_ct = 0;
+    {
         Chunk c{0, 0, 0, 0};
         int64_t i = 0;
         while (i < n_net) {
@@ -437,8 +472,8 @@ ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const
             int64_t done = 0;
             while (done < run) {
                 bool traj_limit = max_traj_chunk > 0 && c.n_traj >= max_traj_chunk;
-                double room = cap - bC - bT * (double)(c.n_traj + 1) - bN * (double)c.n_net;
-                int64_t fit = room > 0 ? (int64_t)(room / bN) : 0;
+                double room = cap - by.C - by.T * (double)(c.n_traj + 1) - by.N * (double)c.n_net;
+                int64_t fit = room > 0 ? (int64_t)(room / by.N) : 0;
                 if (traj_limit || fit <= 0) {
                     if (c.n_net == 0) return set_error(PTN_ERR_TOO_LARGE, "block %d: no room for one network", j);
                     chunks.push_back(c);
@@ -446,10 +481,8 @@ ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const
                     continue;
                 }
                 int64_t take = std::min(fit, run - done);
-                if (write) {
-                    hct[n_ct] = ht[i];
-                    for (int64_t q = 0; q < take; q++) htl[c.net0 + c.n_net + q] = (int32_t)c.n_traj;
-                }
+                hct[n_ct] = ht[i];
+                for (int64_t q = 0; q < take; q++) htl[c.net0 + c.n_net + q] = (int32_t)c.n_traj;
                 n_ct++;
                 c.n_traj++;
                 c.n_net += take;
@@ -458,34 +491,7 @@ ptn_status contract_level(const ptn_plan* plan, const ptn_traj* tr, int j, const
             i = k;
         }
         if (c.n_net) chunks.push_back(c);
-        return PTN_OK;
-    };
-    BlockPlan* use = const_cast<BlockPlan*>(&plan->blocks[j]);
-    std::vector<Chunk> chunks;
-    e = split(*use, chunks, true);
-    BlockPlan* path = use->path_order.get();
-    if (path && (e || chunks.size() > 1)) {
-        // The class-by-class listing does not hold the call in one chunk: the path's
-        // order takes over where it makes fewer launches of the whole call (its chunks
-        // hold more networks), or where it alone holds a network.  Measured: 256
-        // trajectories of a 40-qubit brickwork's block in 29 chunks 5.4 ms, by class in
-        // 43 chunks 7.2; 2000 of a 60-qubit one's in 42 chunks 8.2 ms, by class in 52
-        // chunks 6.3 (a third of the launches per chunk saved).
-        const int64_t n_ct_cls = n_ct;
-        std::vector<Chunk> other;
-        if (split(*path, other, false) == PTN_OK &&
-            (e || (int64_t)other.size() * chunk_launches(*path, plan->opts.fuse_max) <
-                      (int64_t)chunks.size() * chunk_launches(*use, plan->opts.fuse_max))) {
-            clear_error();
-            use = path;
-            if (!(e = split(*use, chunks, true))) e = upload_block(*use);
-        } else {
-            if (!e) clear_error();
-            n_ct = n_ct_cls;
-        }
     }
-    if (e) return e;
-    const BlockPlan& bp = *use;
     if ((e = ws->chunk_traj.grow(sizeof(int32_t) * n_ct))) return e;
     if ((e = ws->net_tl.grow(sizeof(int32_t) * n_net))) return e;
     PTN_CUDA(cudaMemcpyAsync(ws->chunk_traj.p, hct, sizeof(int32_t) * n_ct, cudaMemcpyHostToDevice, s));
